@@ -57,7 +57,7 @@ typedef enum {
 /* Arithmetic of a state.  The truncation SVD is FP64-accurate and the energy
  * sum FP64 in every mode unless mps_config.svd_fp64 = 0.  MPS_PREC_FP64
  * stores complex128; its CUDA-core contractions (theta, B~_q, environments)
- * and the FP64-accurate Jacobi sweeps compute in double-float arithmetic
+ * and the FP64-accurate SVD compute in double-float arithmetic
  * (pairs of FP32 values, about 2^-46 relative per operation) on the FP32
  * units, since this part executes FP64 at 1/64 of the FP32 rate; results
  * are stored as complex128.  The split-product modes keep
@@ -81,13 +81,12 @@ typedef struct {
   int32_t chi_max;        /* bond-dimension cap (>= 1) */
   int32_t precision;      /* mps_precision */
   double trunc_rel;       /* keep s_i > trunc_rel * s_1 (0: keep all nonzero) */
-  int32_t svd_fp64;       /* 0: Jacobi SVD in the storage precision;
-                             1: FP64-accurate Jacobi SVD (thetas whose column capacity is 32 or
-                                more: FP32 sweeps to FP32 convergence, two FP64
-                                re-orthonormalisation passes of V, A = C~ V rebuilt in FP64,
-                                double-float sweeps on the FP32 units to a stopping rule at unit
-                                roundoff 2^-46; smaller thetas: every sweep in FP64);
-                             2: every Jacobi sweep in FP64 */
+  int32_t svd_fp64;       /* 0: Jacobi SVD in FP32;
+                             1: FP64-accurate SVD: pivoted Gram-Schmidt, then Jacobi sweeps on the
+                                triangular factor, in double-float on the FP32 units to a stopping
+                                rule at unit roundoff 2^-46, singular values from the product C V^H
+                                (thetas whose column capacity is below 32: every step in FP64);
+                             2: the same with every step in FP64 */
   int32_t svd_max_sweeps; /* Jacobi sweep cap; 0 selects 60 */
   double svd_tol;         /* rotate a pair while |b_ij| > tol sqrt(b_ii b_jj); 0: default */
   int32_t tensor_cores;   /* complex64 states: 1 = environment contractions on the tensor
@@ -128,17 +127,17 @@ typedef struct {
   int64_t two_qubit_gates;  /* two-qubit gates applied */
   double svd_flops;         /* real flops of the Jacobi sweeps run (dots + rotations) */
   int64_t svd_sweeps_fp32;  /* Jacobi sweeps run in FP32, summed over SVDs */
-  int64_t svd_sweeps_fp64;  /* Jacobi sweeps run in FP64, summed over SVDs */
-  double svd_phase_cycles[4]; /* SM clock cycles of the cluster SVDs (first CTA), summed: column
-                                 load, FP32 sweeps, FP64 re-orthonormalisation of V and A = C~ V,
-                                 FP64 sweeps with the truncation and output */
+  int64_t svd_sweeps_fp64;  /* Jacobi sweeps run in double-float or FP64, summed over SVDs */
+  double svd_phase_cycles[4]; /* SM clock cycles of the SVDs (first CTA), summed: column load,
+                                 Gram-Schmidt factorisation, sweeps, truncation (the FP32 cluster
+                                 SVD: load, 0, sweeps and output, 0) */
 } mps_report;
 
 /* Kernel classes for mps_ctx_profile_read. */
 typedef enum {
   MPS_K_THETA = 0,     /* theta contraction + gate + lam scaling */
   MPS_K_SVD = 1,       /* Jacobi SVD + truncation */
-  MPS_K_G3 = 2,        /* B~_q = C V^dagger */
+  MPS_K_G3 = 2,        /* B~_q = C V^dagger (where the SVD kernel computes it: counted here, timed there) */
   MPS_K_GATE1 = 3,     /* one-qubit gate */
   MPS_K_SETUP = 4,     /* reset, angle binding, fills */
   MPS_K_ENV_M = 5,     /* environment times site tensor */

@@ -103,6 +103,8 @@ struct KernelScope {
 }  // namespace mpsv
 
 namespace mpsv {
+// Counts a launch for a class whose work another class's kernel does.
+void count_launch(mps_ctx* ctx, int k);
 mps_status dev_alloc(mps_ctx* ctx, void** p, size_t bytes);
 void dev_free(mps_ctx* ctx, void* p);
 }  // namespace mpsv
@@ -123,7 +125,6 @@ struct mps_state {
   int n = 0;
   mps_config cfg{};
   bool fp32 = false;   // complex64 storage
-  bool svd64 = true;   // FP64 Jacobi
   bool tc = false;     // tensor-core environment contractions (complex64 states)
   std::vector<int> cap;          // bond capacities, n + 1
   std::vector<size_t> site_off;  // complex elements
@@ -136,8 +137,7 @@ struct mps_state {
   uint8_t* d_bits = nullptr;
   mpsv::DevReport* d_rep = nullptr;
   void* d_C = nullptr;  // theta C, m x n (storage precision)
-  void* d_A = nullptr;  // SVD matrix, m x n (SVD precision)
-  void* d_V = nullptr;  // n x n (SVD precision)
+  char* d_svd = nullptr;  // workspace of the truncation SVD
   mpsv::DevGate* d_gates = nullptr;
   size_t gates_cap = 0;
   size_t total_lam = 0;
@@ -203,6 +203,46 @@ struct mps_ham {
 };
 
 namespace mpsv {
+// Arithmetic of a truncation SVD (svd_arith.cuh) for mps_config.svd_fp64 and
+// the theta's column capacity: svd_fp64 = 1 runs thetas of fewer than 32
+// columns in FP64 and larger ones in double-float.
+enum SvdArith { SVD_F32, SVD_DF, SVD_F64 };
+inline SvdArith svd_arith(int svd_fp64, int ncap) {
+  return svd_fp64 == 0 ? SVD_F32 : (svd_fp64 == 2 || ncap < 32 ? SVD_F64 : SVD_DF);
+}
+// One truncation SVD: theta C (row-major, capacity mcap x ncap; the actual
+// sizes are 2 chi[q] x 2 chi[q + 2]), row weights lam_l, workspace ws.
+struct SvdJob {
+  int mcap, ncap;
+  bool storage32;  // complex64 C and Bnext
+  const void* C;
+  const double* lam_l;
+  int* chi;
+  int q;
+  SvdParams p;
+  void* Bnext;
+  double* lam_next;
+  DevReport* rep;
+  void* Bq;  // B~_q = C V^H / ||s[:k]|| (nullable: not wanted)
+  char* ws;
+  cudaStream_t stream;
+};
+#define MPSV_SVD_DECL(x)                            \
+  size_t svd_workspace_##x(int mcap, int ncap);     \
+  void svd_prime_##x();                             \
+  void svd_launch_##x(const SvdJob& j);
+MPSV_SVD_DECL(df)
+MPSV_SVD_DECL(f32)
+MPSV_SVD_DECL(f64)
+#undef MPSV_SVD_DECL
+inline size_t svd_workspace(SvdArith a, int mcap, int ncap) {
+  return a == SVD_DF ? svd_workspace_df(mcap, ncap)
+                     : (a == SVD_F64 ? svd_workspace_f64(mcap, ncap) : svd_workspace_f32(mcap, ncap));
+}
+inline void svd_launch(SvdArith a, const SvdJob& j) {
+  a == SVD_DF ? svd_launch_df(j) : (a == SVD_F64 ? svd_launch_f64(j) : svd_launch_f32(j));
+}
+
 // The two status flags of a state, read back with one 8-byte copy from
 // &DevReport::not_converged.
 struct StateFlags {

@@ -1,8 +1,8 @@
 // mps_gate2_noalloc: one two-qubit gate on caller-owned device buffers, with
 // no device allocation at all.
 //
-// The regular path keeps its gate scratch (the theta product C, the Jacobi
-// matrices A and V, the bond dimensions and the truncation report) in
+// The regular path keeps its gate scratch (the theta product C, the SVD's
+// workspace, the bond dimensions and the truncation report) in
 // per-state buffers from cudaMalloc.  Some callers cannot allocate: code
 // running inside a CUDA host callback or stream-ordered host function (where
 // CUDA API calls that allocate are not allowed), embedders that hand the
@@ -25,6 +25,7 @@
 
 #include "gate_kernels.cuh"
 #include "internal.h"
+#include "svd_launch.cuh"
 
 namespace mpsv {
 namespace {
@@ -32,7 +33,7 @@ namespace {
 constexpr int kMaxChi = 32;                 // largest chi_l, chi_r accepted
 constexpr int kMaxDim = 2 * kMaxChi;        // theta is at most 64 x 64
 constexpr size_t kMatBytes = (size_t)kMaxDim * kMaxDim * sizeof(double2);
-constexpr size_t kOffC = 0, kOffA = kMatBytes, kOffV = 2 * kMatBytes;
+constexpr size_t kOffC = 0, kOffWs = kMatBytes;  // theta; SVD workspace (2 kMatBytes)
 constexpr size_t kOffChi = 3 * kMatBytes;                 // int[4]
 constexpr size_t kOffGate = kOffChi + 256;                // DevGate
 constexpr size_t kOffRep = kOffGate + 512;                // DevReport
@@ -55,11 +56,7 @@ mps_status scratch_for(int dev, unsigned char** out) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc: cudaGetSymbolAddress");
-    int smem = 0;
-    e = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(svd_truncate_kernel<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               smem - 1024);
+    e = svd_attrs<ArF64, double>();
     if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc: set-up");
     g_scratch_addr[dev] = static_cast<unsigned char*>(p);
   }
@@ -153,25 +150,21 @@ extern "C" mps_status mps_gate2_noalloc(int device, void* cuda_stream, int32_t c
   const DevGate* dg = reinterpret_cast<const DevGate*>(scratch + kOffGate);
   DevReport* rep = reinterpret_cast<DevReport*>(scratch + kOffRep);
   double2* C = reinterpret_cast<double2*>(scratch + kOffC);
-  double2* A = reinterpret_cast<double2*>(scratch + kOffA);
-  double2* V = reinterpret_cast<double2*>(scratch + kOffV);
   double2* Bl = reinterpret_cast<double2*>(B_left);
   double2* Br = reinterpret_cast<double2*>(B_right);
   const dim3 blk(kTile, kTile);
-  theta_kernel<double, double><<<dim3((chi_r + kTile - 1) / kTile, (chi_l + kTile - 1) / kTile), blk, 0, s>>>(
-      Bl, Br, dg, lam_left, chi, 0, C, A);
+  theta_kernel<double><<<dim3((chi_r + kTile - 1) / kTile, (chi_l + kTile - 1) / kTile), blk, 0, s>>>(Bl, Br, dg, chi,
+                                                                                                    0, C);
   SvdParams p;
   p.chi_max = chi_max;
   p.max_sweeps = 60;
   p.trunc_rel = trunc_rel;
   p.tol = 0.0;
-  p.mixed = 0;
   const int n = 2 * chi_r, m = 2 * chi_l;
-  const size_t smem = ((size_t)m * n + (size_t)n * n) * sizeof(double2) + (size_t)n * (sizeof(double) + sizeof(int)) + 64;
-  svd_truncate_kernel<double, double><<<1, 32 * std::min(32, std::max(1, n / 2)), smem, s>>>(
-      A, V, 1, chi, 0, p, Br, lam_out, rep);
-  const int kmax = std::min(chi_max, std::min(m, n));
-  g3_kernel<double><<<dim3((kmax + kTile - 1) / kTile, (m + kTile - 1) / kTile), blk, 0, s>>>(C, Br, chi, 0, rep, Bl);
+  const size_t smem = SvdSmem<ArF64>::bytes(m, n, 1, true, true);
+  svd_kernel<ArF64, double><<<1, kSvdThreads<ArF64>, smem, s>>>(C, lam_left, chi, 0, p, Br, lam_out, rep, Bl,
+                                                                reinterpret_cast<char*>(scratch + kOffWs),
+                                                                (unsigned)smem);
   noalloc_finish_kernel<<<1, 32, 0, s>>>(scratch, chi_out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc launch");

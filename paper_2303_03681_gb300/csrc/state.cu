@@ -6,7 +6,6 @@
 
 #include "gate_kernels.cuh"
 #include "internal.h"
-#include "svd_cluster.cuh"
 
 namespace mpsv {
 
@@ -57,6 +56,8 @@ void dev_free(mps_ctx* ctx, void* p) {
   }
   cudaFree(p);
 }
+
+void count_launch(mps_ctx* c, int k) { (c->capturing ? c->capturing->counts : c->launches)[k] += 1; }
 
 KernelScope::KernelScope(mps_ctx* ctx, int k) : c(ctx), kind(k) {
   if (c->capturing) {
@@ -162,187 +163,48 @@ template <typename R> static cplx<R>* site_ptr(mps_state* st, int s) {
   return reinterpret_cast<cplx<R>*>(st->d_B) + st->site_off[s];
 }
 
-template <typename S> static size_t svd_smem_bytes(int mcap, int ncap, bool use_smem) {
-  size_t b = (size_t)ncap * (sizeof(double) + sizeof(int)) + 64;
-  if (use_smem) b += ((size_t)mcap * ncap + (size_t)ncap * ncap) * sizeof(cplx<S>);
-  return b;
-}
-
-static size_t max_dyn_smem() {
-  static size_t v = 0;
-  static std::once_flag f;
-  std::call_once(f, [] {
-    int dev = 0, val = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&val, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    v = (size_t)val;
-  });
-  return v;
-}
-
-template <typename S, typename R> static void svd_set_attr() {
-  static std::once_flag f;
-  std::call_once(f, [] {
-    cudaFuncSetAttribute(svd_truncate_kernel<S, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(max_dyn_smem() - 1024));
-  });
-}
-
-// Launch plan of the cluster Jacobi SVD for a theta with up to mcap rows and
-// ncap columns (A = C~, stacked columns [A; V] of length mcap + ncap), or
-// P = 0 when the single-CTA kernel is used.  The stacked columns stay in
-// shared memory when the capacities allow; otherwise they live in the
-// state's global workspace, and the kernel still keeps them in shared
-// memory whenever the actual bond dimensions fit the allocation given here.
-struct SvdPlan {
-  int P = 0;
-  int threads = 0;
-  size_t smem = 0;
-  bool global = false;
-};
-
-template <typename S, typename R> static SvdPlan cluster_svd_plan(int mcap, int ncap) {
-  SvdPlan pl;
-  // FP64 runs at 2 FMA/clk/SM on this part, so even small FP64 thetas gain
-  // from spreading their columns over several SMs; FP32 ones only from 96.
-  if (ncap < (sizeof(S) == 8 ? 32 : 96)) return pl;
-  static int max16 = -1;
-  static std::once_flag f;
-  std::call_once(f, [] {
-    cudaFuncSetAttribute(svd_cluster_kernel<S, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(max_dyn_smem() - 1024));
-    cudaFuncSetAttribute(svd_cluster_kernel<S, R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(kClusterMaxThreads<S>);
-    cfg.dynamicSmemBytes = max_dyn_smem() - 2048;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, svd_cluster_kernel<S, R>, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      n = 0;
-    }
-    max16 = n;
-  });
-  const size_t lim = max_dyn_smem() - 2048;
-  if constexpr (sizeof(S) == 4) {
-    // FP32 pair steps are latency-bound: few CTAs (fewer rounds and cluster
-    // barriers) with 16 warps each, so that concurrent evaluations find SMs
-    // free.  Columns stay in shared memory whenever the actual sizes fit.
-    const int P = 4, b = (ncap + 2 * P - 1) / (2 * P);
-    pl.P = P;
-    pl.threads = 512;
-    ClusterSvdSmem<S> L(b, mcap + ncap, 2 * P * b, pl.threads);
-    if (L.total <= lim) {
-      pl.smem = L.total;
-    } else {
-      pl.global = true;
-      pl.smem = std::min(lim, std::max(ClusterSvdSmem<S>(b, 0, 2 * P * b, pl.threads).total, (size_t)160 * 1024));
-    }
-    return pl;
-  } else {
-  // FP64 sweeps: at most 8 CTAs of up to 8 warps (one column pair each), so
-  // that a block holds enough pairs to keep its SM's FP64 units busy; with
-  // many evaluations in flight, 16 CTAs of 4 busy warps left most SMs waiting
-  // at cluster barriers (0.47 against 0.70 evaluations/s at 32 streams)
-  for (int P = ncap < 64 ? 4 : 8; P <= 8; P *= 2) {
-    if (P == 16 && max16 <= 0) break;
-    const int b = (ncap + 2 * P - 1) / (2 * P);
-    ClusterSvdSmem<S> L(b, mcap + ncap, 2 * P * b, 32 * b);
-    if (L.total <= lim && 32 * b <= 512) {
-      pl.P = P;
-      pl.threads = std::min(32 * b, kClusterMaxThreads<S>);
-      pl.smem = L.total;
-      return pl;
-    }
-  }
-  // columns too long for shared memory at the capacity: a global workspace,
-  // and the whole shared memory of the CTA so that the actual sizes use it
-  // whenever they fit
-  const int P = 8;
-  const int b = (ncap + 2 * P - 1) / (2 * P);
-  pl.P = P;
-  pl.threads = std::min(32 * b, kClusterMaxThreads<S>);
-  pl.global = true;
-  pl.smem = lim;
-  return pl;
-  }
-}
-
-// The truncation SVD of one theta (bond capacities mcap x ncap): the
-// cluster kernel when the plan has CTAs (it reads the row-major C and the
-// lam_l row weights itself; gbuf is its global workspace), else the
-// single-CTA kernel on the column-major lam-scaled copy A with the V
-// workspace.  Writes B~_{q+1} = V^H rows, lam_{q+1}, chi[q+1] and the report.
-template <typename R, typename S>
-static void launch_svd(mps_ctx* ctx, const SvdPlan& plan, int mcap, int ncap, const SvdParams& p,
-                       const cplx<R>* Cm, cplx<S>* A, cplx<S>* V, const double* lam_l, int* chi, int q,
-                       cplx<R>* Bnext, double* lam_next, DevReport* rep, cudaStream_t s) {
-  KernelScope k(ctx, MPS_K_SVD);
-  if (plan.P) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.P);
-    cfg.blockDim = dim3(plan.threads);
-    cfg.dynamicSmemBytes = plan.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = plan.P;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, svd_cluster_kernel<S, R>, Cm, lam_l, chi, q, p, Bnext, lam_next, rep,
-                       plan.global ? A : (cplx<S>*)nullptr, (unsigned)plan.smem);
-    return;
-  }
-  const size_t full = svd_smem_bytes<S>(mcap, ncap, true);
-  const bool use_smem = full + 2048 <= max_dyn_smem();
-  const size_t smem = svd_smem_bytes<S>(mcap, ncap, use_smem);
-  svd_set_attr<S, R>();
-  const int warps = std::min(32, std::max(1, ncap / 2));
-  svd_truncate_kernel<S, R><<<1, 32 * warps, smem, s>>>(A, V, use_smem ? 1 : 0, chi, q, p, Bnext, lam_next, rep);
-}
-
-template <typename R, typename S>
+template <typename R>
 static void launch_two_qubit(mps_state* st, const DevGate* g, int q, cudaStream_t s) {
-  const int cap_l = st->cap[q], cap_m = st->cap[q + 1], cap_r = st->cap[q + 2];
+  const int cap_l = st->cap[q], cap_r = st->cap[q + 2];
   const dim3 blk(kTile, kTile);
   const dim3 g1((cap_r + kTile - 1) / kTile, (cap_l + kTile - 1) / kTile);
-  const SvdPlan plan = cluster_svd_plan<S, R>(2 * cap_l, 2 * cap_r);
-  const int P = plan.P;
-  // split-product tensor-core contractions (complex64 states): the cluster
-  // SVD reads C itself, so they serve the bonds where it runs
-  const bool tcg = sizeof(R) == 4 && P && tc_gates_used(st, q);
+  // split-product tensor-core contractions (complex64 states): thetas of 16
+  // columns and fewer are all padding on 128-wide tiles
+  const bool tcg = sizeof(R) == 4 && 2 * cap_r >= (st->cfg.svd_fp64 ? 32 : 96) && tc_gates_used(st, q);
   if (tcg) {
     tc_theta(st, g, q, s);
   } else {
     KernelScope k(st->ctx, MPS_K_THETA);
-    theta_kernel<R, S><<<g1, blk, 0, s>>>(site_ptr<R>(st, q), site_ptr<R>(st, q + 1), g,
-                                          st->d_lam + st->lam_off[q], st->d_chi, q,
-                                          reinterpret_cast<cplx<R>*>(st->d_C),
-                                          P ? nullptr : reinterpret_cast<cplx<S>*>(st->d_A));
+    theta_kernel<R><<<g1, blk, 0, s>>>(site_ptr<R>(st, q), site_ptr<R>(st, q + 1), g, st->d_chi, q,
+                                       reinterpret_cast<cplx<R>*>(st->d_C));
   }
-  SvdParams p;
-  p.chi_max = st->cfg.chi_max;
-  p.max_sweeps = st->cfg.svd_max_sweeps > 0 ? st->cfg.svd_max_sweeps : 60;
-  p.trunc_rel = st->cfg.trunc_rel;
-  p.tol = st->cfg.svd_tol;
-  p.mixed = st->cfg.svd_fp64 == 2 ? 0 : 1;
-  const dim3 g3((cap_m + kTile - 1) / kTile, (2 * cap_l + kTile - 1) / kTile);
-  const cplx<R>* Cm = reinterpret_cast<const cplx<R>*>(st->d_C);
-  launch_svd<R, S>(st->ctx, plan, 2 * cap_l, 2 * cap_r, p, Cm, reinterpret_cast<cplx<S>*>(st->d_A),
-                   reinterpret_cast<cplx<S>*>(st->d_V), st->d_lam + st->lam_off[q], st->d_chi, q,
-                   site_ptr<R>(st, q + 1), st->d_lam + st->lam_off[q + 1], st->d_rep, s);
+  {
+    KernelScope k(st->ctx, MPS_K_SVD);
+    SvdJob j;
+    j.mcap = 2 * cap_l;
+    j.ncap = 2 * cap_r;
+    j.storage32 = sizeof(R) == 4;
+    j.C = st->d_C;
+    j.lam_l = st->d_lam + st->lam_off[q];
+    j.chi = st->d_chi;
+    j.q = q;
+    j.p.chi_max = st->cfg.chi_max;
+    j.p.max_sweeps = st->cfg.svd_max_sweeps > 0 ? st->cfg.svd_max_sweeps : 60;
+    j.p.trunc_rel = st->cfg.trunc_rel;
+    j.p.tol = st->cfg.svd_tol;
+    j.Bnext = site_ptr<R>(st, q + 1);
+    j.lam_next = st->d_lam + st->lam_off[q + 1];
+    j.rep = st->d_rep;
+    j.Bq = tcg || st->cfg.svd_fp64 == 0 ? nullptr : site_ptr<R>(st, q);
+    if (j.Bq) count_launch(st->ctx, MPS_K_G3);  // done inside the SVD kernel
+    j.ws = st->d_svd;
+    j.stream = s;
+    svd_launch(svd_arith(st->cfg.svd_fp64, j.ncap), j);
+  }
   if (tcg) {
     tc_g3(st, q, s);
-  } else {
+  } else if (st->cfg.svd_fp64 == 0) {
+    const dim3 g3((st->cap[q + 1] + kTile - 1) / kTile, (2 * cap_l + kTile - 1) / kTile);
     KernelScope k(st->ctx, MPS_K_G3);
     g3_kernel<R><<<g3, blk, 0, s>>>(reinterpret_cast<cplx<R>*>(st->d_C), site_ptr<R>(st, q + 1), st->d_chi, q,
                                     st->d_rep, site_ptr<R>(st, q));
@@ -367,17 +229,10 @@ mps_status state_apply_device_gates(mps_state* st, const DevGate* d_gates, const
       else
         launch_one_qubit<double>(st, g, q[i], s);
     } else {
-      if (st->fp32) {
-        if (st->svd64)
-          launch_two_qubit<float, double>(st, g, q[i], s);
-        else
-          launch_two_qubit<float, float>(st, g, q[i], s);
-      } else {
-        if (st->svd64)
-          launch_two_qubit<double, double>(st, g, q[i], s);
-        else
-          launch_two_qubit<double, float>(st, g, q[i], s);
-      }
+      if (st->fp32)
+        launch_two_qubit<float>(st, g, q[i], s);
+      else
+        launch_two_qubit<double>(st, g, q[i], s);
     }
   }
   MPSV_CUDA(cudaGetLastError());
@@ -455,18 +310,11 @@ mps_status state_bind_circuit(mps_state* st, const mps_circuit* c, const double*
   return MPS_OK;
 }
 
-// One-time launch attributes (shared-memory opt-ins, the 16-CTA cluster
-// occupancy query) set before a capture, outside it.
-template <typename R, typename S> static void prime_launch_attrs() {
-  svd_set_attr<S, R>();
-  (void)cluster_svd_plan<S, R>(256, 256);
-}
-
-static void prime_launch_attrs(const mps_state* st) {
-  if (st->fp32)
-    st->svd64 ? prime_launch_attrs<float, double>() : prime_launch_attrs<float, float>();
-  else
-    st->svd64 ? prime_launch_attrs<double, double>() : prime_launch_attrs<double, float>();
+// One-time launch attributes (shared-memory opt-ins), set before a capture.
+static void prime_launch_attrs() {
+  svd_prime_df();
+  svd_prime_f32();
+  svd_prime_f64();
 }
 
 mps_status state_run_circuit(mps_state* st, const mps_circuit* c, const double* theta, int theta_on_device) {
@@ -493,7 +341,7 @@ mps_status state_run_circuit(mps_state* st, const mps_circuit* c, const double* 
     g->theta_ptr = st->d_theta;
     g->bound_ptr = st->d_bound;
     g->mask = ctx->prof_mask;
-    prime_launch_attrs(st);
+    prime_launch_attrs();
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) {
       delete g;
@@ -534,7 +382,7 @@ static void destroy_state(mps_state* st) {
   }
   tc_gates_free(st);
   for (void* p : {st->d_B, (void*)st->d_lam, (void*)st->d_chi, (void*)st->d_site_off, (void*)st->d_lam_off,
-                  (void*)st->d_bits, (void*)st->d_rep, st->d_C, st->d_A, st->d_V, (void*)st->d_gates,
+                  (void*)st->d_bits, (void*)st->d_rep, st->d_C, (void*)st->d_svd, (void*)st->d_gates,
                   (void*)st->d_bound, (void*)st->d_theta, st->d_L[0], st->d_L[1], st->d_M, (void*)st->d_vals,
                   (void*)st->d_energy, (void*)st->d_obs})
     dev_free(c, p);
@@ -551,19 +399,19 @@ static void host_gate_to_dev(const mps_gate& g, DevGate& d) {
 
 // ---- workspace and kernels of mps_truncated_svd (one theta on its own)
 struct SvdWork {
-  int mcap = 0, ncap = 0, sbytes = 0;
+  int mcap = 0, ncap = 0;
+  size_t ws_bytes = 0;
   int* d_chi = nullptr;
   DevReport* d_rep = nullptr;
   double* d_ones = nullptr;
   double* d_lam = nullptr;
-  void* d_A = nullptr;
-  void* d_V = nullptr;
+  char* d_ws = nullptr;
 };
 
 void svd_work_free(mps_ctx* ctx) {
   SvdWork* w = ctx->svdw;
   if (!w) return;
-  for (void* p : {(void*)w->d_chi, (void*)w->d_rep, (void*)w->d_ones, (void*)w->d_lam, w->d_A, w->d_V})
+  for (void* p : {(void*)w->d_chi, (void*)w->d_rep, (void*)w->d_ones, (void*)w->d_lam, (void*)w->d_ws})
     dev_free(ctx, p);
   delete w;
   ctx->svdw = nullptr;
@@ -588,15 +436,6 @@ static __global__ void svd_setup_kernel(int* chi, int chi_l, int chi_r, DevRepor
   for (int i = 0; i < 4; ++i) rep->phase_cycles[i] = 0.0;
 }
 
-// column-major copy of the row-major theta (the single-CTA kernel's input; lam = 1)
-template <typename R, typename S>
-static __global__ void svd_c_to_a_kernel(const cplx<R>* __restrict__ C, int m, int n, cplx<S>* __restrict__ A) {
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= (size_t)m * n) return;
-  const int col = (int)(t / m), row = (int)(t % m);
-  A[t] = ccast<cplx<S>>(C[(size_t)row * n + col]);
-}
-
 // the kept singular values without the renormalisation of the gate update
 static __global__ void svd_finish_kernel(const int* chi, const DevReport* rep, const double* lam, double* s_out) {
   const int k = chi[1];
@@ -604,12 +443,13 @@ static __global__ void svd_finish_kernel(const int* chi, const DevReport* rep, c
   for (int a = threadIdx.x; a < k; a += blockDim.x) s_out[a] = lam[a] * nrm;
 }
 
-template <typename R, typename S>
-static mps_status truncated_svd(mps_ctx* ctx, int m, int n, const void* C, const SvdParams& p, double* s_out,
-                                void* Vh_out) {
+static mps_status truncated_svd(mps_ctx* ctx, bool storage32, int svd_fp64, int m, int n, const void* C,
+                                const SvdParams& p, double* s_out, void* Vh_out) {
   cudaStream_t s = ctx->stream;
+  const SvdArith ar = svd_arith(svd_fp64, n);
+  const size_t need = svd_workspace(ar, m, n);
   SvdWork* w = ctx->svdw;
-  if (w && (m > w->mcap || n > w->ncap || (int)sizeof(S) > w->sbytes)) {
+  if (w && (m > w->mcap || n > w->ncap || need > w->ws_bytes)) {
     MPSV_CUDA(cudaStreamSynchronize(s));
     svd_work_free(ctx);
     w = nullptr;
@@ -619,15 +459,12 @@ static mps_status truncated_svd(mps_ctx* ctx, int m, int n, const void* C, const
     ctx->svdw = w;
     w->mcap = m;
     w->ncap = n;
-    w->sbytes = (int)sizeof(S);
-    const size_t celem = sizeof(cplx<S>);
+    w->ws_bytes = need;
     mps_status rc = dev_alloc(ctx, (void**)&w->d_chi, 4 * sizeof(int));
     if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&w->d_rep, sizeof(DevReport));
     if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&w->d_ones, (size_t)m * sizeof(double));
     if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&w->d_lam, (size_t)n * sizeof(double));
-    if (rc == MPS_OK)
-      rc = dev_alloc(ctx, &w->d_A, std::max((size_t)m * n, cluster_svd_workspace(m, n, sizeof(S))) * celem);
-    if (rc == MPS_OK) rc = dev_alloc(ctx, &w->d_V, (size_t)n * n * celem);
+    if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&w->d_ws, need);
     if (rc == MPS_OK) {
       std::vector<double> ones(m, 1.0);
       cudaError_t e = cudaMemcpyAsync(w->d_ones, ones.data(), m * sizeof(double), cudaMemcpyHostToDevice, s);
@@ -639,15 +476,11 @@ static mps_status truncated_svd(mps_ctx* ctx, int m, int n, const void* C, const
       return rc;
     }
   }
-  const SvdPlan plan = cluster_svd_plan<S, R>(m, n);
-  const cplx<R>* Cm = static_cast<const cplx<R>*>(C);
   svd_setup_kernel<<<1, 32, 0, s>>>(w->d_chi, m / 2, n / 2, w->d_rep);
-  if (!plan.P) {
-    const size_t tot = (size_t)m * n;
-    svd_c_to_a_kernel<R, S><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(Cm, m, n, static_cast<cplx<S>*>(w->d_A));
+  {
+    KernelScope k(ctx, MPS_K_SVD);
+    svd_launch(ar, SvdJob{m, n, storage32, C, w->d_ones, w->d_chi, 0, p, Vh_out, w->d_lam, w->d_rep, nullptr, w->d_ws, s});
   }
-  launch_svd<R, S>(ctx, plan, m, n, p, Cm, static_cast<cplx<S>*>(w->d_A), static_cast<cplx<S>*>(w->d_V), w->d_ones,
-                   w->d_chi, 0, static_cast<cplx<R>*>(Vh_out), w->d_lam, w->d_rep, s);
   svd_finish_kernel<<<1, 256, 0, s>>>(w->d_chi, w->d_rep, w->d_lam, s_out);
   MPSV_CUDA(cudaGetLastError());
   return MPS_OK;
@@ -811,7 +644,6 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
                   cfg->precision == MPS_PREC_AUTO)
                      ? cfg->precision
                      : 0;
-  st->svd64 = cfg->svd_fp64 != 0;
   st->tc = st->fp32 && (cfg->tensor_cores != 0 || st->tc_gates != 0);
   const int n = n_qubits;
   st->cap.resize(n + 1);
@@ -819,7 +651,7 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
   st->site_off.resize(n);
   st->lam_off.resize(n + 1);
   size_t off = 0, loff = 0;
-  size_t max_mn = 1, max_nn = 1, max_stack = 1;
+  size_t max_mn = 1, max_svd = 1;
   for (int s = 0; s < n; ++s) {
     st->site_off[s] = off;
     off += (size_t)st->cap[s] * 2 * st->cap[s + 1];
@@ -831,13 +663,11 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
   for (int q = 0; q + 1 < n; ++q) {
     const size_t m = 2 * (size_t)st->cap[q], nn = 2 * (size_t)st->cap[q + 2];
     max_mn = std::max(max_mn, m * nn);
-    max_stack = std::max(max_stack, cluster_svd_workspace(m, nn, st->svd64 ? 8 : 4));
-    max_nn = std::max(max_nn, nn * nn);
+    max_svd = std::max(max_svd, svd_workspace(svd_arith(cfg->svd_fp64, (int)nn), (int)m, (int)nn));
   }
   st->total_elems = off;
   st->total_lam = loff;
   const size_t celem = st->fp32 ? sizeof(float2) : sizeof(double2);
-  const size_t selem = st->svd64 ? sizeof(double2) : sizeof(float2);
   mps_status rc = MPS_OK;
   auto A = [&](void** p, size_t bytes) {
     if (rc == MPS_OK) rc = dev_alloc(ctx, p, bytes);
@@ -850,8 +680,7 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
   A((void**)&st->d_bits, n);
   A((void**)&st->d_rep, sizeof(DevReport));
   A(&st->d_C, max_mn * celem);
-  A(&st->d_A, std::max(max_mn, max_stack) * selem);  // theta copy, or the cluster SVD's stacked columns
-  A(&st->d_V, max_nn * selem);
+  A((void**)&st->d_svd, max_svd);
   if (rc == MPS_OK && st->tc_gates) rc = tc_gates_setup(st);
   if (rc != MPS_OK) {
     destroy_state(st);
@@ -1126,14 +955,7 @@ mps_status mps_truncated_svd(mps_ctx* ctx, int32_t precision, int32_t m, int32_t
   p.max_sweeps = 60;
   p.trunc_rel = trunc_rel;
   p.tol = 0.0;
-  p.mixed = svd_fp64 == 2 ? 0 : 1;
-  mps_status rc;
-  if (precision == MPS_PREC_FP64)
-    rc = svd_fp64 ? truncated_svd<double, double>(ctx, m, n, C, p, s_out, Vh_out)
-                  : truncated_svd<double, float>(ctx, m, n, C, p, s_out, Vh_out);
-  else
-    rc = svd_fp64 ? truncated_svd<float, double>(ctx, m, n, C, p, s_out, Vh_out)
-                  : truncated_svd<float, float>(ctx, m, n, C, p, s_out, Vh_out);
+  mps_status rc = truncated_svd(ctx, precision == MPS_PREC_FP32, svd_fp64, m, n, C, p, s_out, Vh_out);
   if (rc != MPS_OK) return rc;
   DevReport r;
   int k = 0;

@@ -1,4 +1,4 @@
-// One-sided Jacobi SVD on a thread-block cluster (Algorithm 1 of the paper's
+// FP32 one-sided Jacobi SVD on a thread-block cluster (Algorithm 1 of the paper's
 // "SVD and one-side jacobi" subsection, parallelised over up to 16 SMs).
 //
 // The kernel orthogonalises the n = 2 chi_r columns of A = C~ (m = 2 chi_l
@@ -22,29 +22,186 @@
 // stacked columns do not fit the shared memory they stay in a global
 // workspace, and a round only renames the positions.
 //
-// FP64 accuracy at FP32 speed.  This part runs FP64 at 2 FMA/clk/SM, so an
-// all-FP64 Jacobi of a 100-column theta takes tens of milliseconds.  The
-// mixed form runs the sweeps in FP32 to FP32 convergence (V32 accumulated as
-// usual), re-orthonormalises V32 in FP64 with two pairwise first-order
-// passes v_i <- v_i - 1/2 sum_j (v_j^H v_i) v_j (the symmetric update
-// V (I - E / 2), E = V^H V - I, which leaves ||E||^2), rebuilds A = C~ V in
-// FP64 from the theta, converts the stacked columns to double-float
-// (dfloat.cuh) and finishes with double-float sweeps on the FP32 units,
-// which start near convergence and converge quadratically.  The singular
-// values, the truncation and B~_{q+1} then come from columns accurate to
-// about 2^-46 (the all-FP64 form, svd_fp64 = 2, sweeps in FP64 throughout).
+// This form serves the FP32 SVD (mps_config.svd_fp64 = 0); the FP64-accurate
+// SVDs run svd_jacobi.cuh.
 #pragma once
 
 #include <cooperative_groups.h>
 
-#include <type_traits>
-
 #include "common.cuh"
-#include "dfloat.cuh"
 
 namespace mpsv {
 
 namespace cg = cooperative_groups;
+
+// Rotation of a column pair of the one-sided Jacobi SVD from its Gram entries
+// alpha = a_i^H a_i, beta = a_j^H a_j, g = gr + i gi = a_i^H a_j (Algorithm 1
+// of the paper, with the phase of g moved onto column j): the new columns are
+// a_i' = c a_i - conj(s e^{i phi}) a_j and a_j' = c a_j + s e^{i phi} a_i.
+// Returns false when the pair is left alone: already orthogonal to tol, or a
+// column at the rounding floor.
+template <typename S>
+__device__ __forceinline__ bool jacobi_rotation(S alpha, S beta, S gr, S gi, S tol, S floor, S tiny, S& c,
+                                                cplx<S>& sph) {
+  const S mag = sqrt(gr * gr + gi * gi);
+  if (!(mag > tiny) || !(mag > tol * sqrt(alpha * beta)) || !(min(alpha, beta) > floor)) return false;
+  const S zeta = (beta - alpha) / (S(2) * mag);
+  const S t = (zeta >= S(0) ? S(1) : S(-1)) / (fabs(zeta) + sqrt(S(1) + zeta * zeta));
+  c = S(1) / sqrt(S(1) + t * t);
+  const S s = t * c;
+  sph = cmk<S>(s * gr / mag, s * gi / mag);  // s e^{i phi}
+  return true;
+}
+
+// The pair rules of the truncation SVD (tail columns).  Jacobi only has to
+// make the columns that the truncation keeps orthogonal to each other and to
+// all others; the columns it discards may stay mixed among themselves as long
+// as none of their singular values could reach the cut.  At the start of a
+// sweep, from the squared column norms nrm2[0..n): the kept set K is what the
+// truncation would keep now (nrm2 > trunc_rel^2 max nrm2, the chi_max largest
+// by rank when more pass), D the rest, and the cut is trunc_rel^2 max nrm2 (or
+// the smallest kept nrm2 under a chi_max cut).  The class of column c goes to
+// cls[c]:
+//  * kTailSkip when sum_D nrm2 <= cut / 4: every singular value of the D
+//    block is then at most half of every kept column's norm, so once K is
+//    orthogonal to itself and to D, K holds the leading singular vectors
+//    whatever D looks like (and the discarded weight is sum_D nrm2); pairs of
+//    two such columns are not rotated.  The factor 1/4 also bounds how much
+//    rotating a kept column against one D column disturbs its orthogonality
+//    to the others, so the kept columns converge quickly (a bare per-column
+//    threshold did not: a column just above it never converged against mixed
+//    columns just below it).
+//  * kTailLoose otherwise, for the deep tail T: the D columns with nrm2 <=
+//    t_d, where t_d <= cut / 4 is the largest such norm below a gap, i.e.
+//    the next larger nrm2 of any column is at least 4 t_d.  Pairs of two of
+//    them are rotated only while |g| > loose_tol sqrt(b_ii b_jj), loose_tol =
+//    min(2 / n, cut / (16 sum_T nrm2)), returned in *loose.  By Gershgorin on
+//    their Gram matrix the singular values of T then stay below
+//    (cut / 4)(1 + n loose_tol) < cut.  Every other column has nrm2 >= 4
+//    t_d, so its rotations against T have small angles (|s| <= 4|g| / (3
+//    nrm2)) and disturb its orthogonality to the rest of T by at most
+//    loose_tol sum_T nrm2 / nrm2 <= 1/4 of what it was: it still converges.
+//    (Without the gap a degenerate pair of columns straddling the threshold
+//    rotated by large angles and carried the loose couplings of its deep
+//    member into its tight one, and with 2 / n alone columns just above the
+//    threshold crawled against many mixed columns just below it.)
+//  * 0 for every other column (the normal stopping rule).
+// Every thread of the block calls it; blocks with the same nrm2 and size
+// compute the same classes.
+constexpr int kTailLoose = 1, kTailSkip = 2;
+
+__device__ __forceinline__ void truncation_tail(const double* nrm2, int n, double trunc_rel, int chi_max, int* cls,
+                                                double* loose) {
+  __shared__ double s_red[33];
+  __shared__ int s_cnt;
+  __shared__ double s_cut;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  // largest squared norm
+  double mx = 0.0;
+  for (int c = threadIdx.x; c < n; c += blockDim.x) mx = fmax(mx, nrm2[c]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) s_red[warp] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < nw; ++w) v = fmax(v, s_red[w]);
+    s_red[32] = v;
+    s_cnt = 0;
+  }
+  __syncthreads();
+  const double thr = trunc_rel * trunc_rel * s_red[32];
+  int cnt = 0;
+  for (int c = threadIdx.x; c < n; c += blockDim.x) cnt += nrm2[c] > thr;
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) atomicAdd(&s_cnt, cnt);
+  __syncthreads();
+  const bool by_rank = s_cnt > chi_max;
+  if (threadIdx.x == 0) s_cut = thr;
+  __syncthreads();
+  // kept flags (1 = kept) into cls[] first
+  for (int c = threadIdx.x; c < n; c += blockDim.x) {
+    if (by_rank) {
+      const double v = nrm2[c];
+      int rk = 0;
+      for (int h = 0; h < n; ++h) rk += (nrm2[h] > v) || (nrm2[h] == v && h < c);
+      cls[c] = rk < chi_max;
+      if (rk == chi_max - 1) s_cut = v;
+    } else {
+      cls[c] = nrm2[c] > thr;
+    }
+  }
+  __syncthreads();
+  // weight of D, summed in a fixed order
+  double part = 0.0;
+  for (int c = threadIdx.x; c < n; c += blockDim.x)
+    if (!cls[c]) part += nrm2[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  __syncthreads();
+  if (lane == 0) s_red[warp] = part;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < nw; ++w) v += s_red[w];
+    s_red[32] = v;
+  }
+  __syncthreads();
+  const double cut = s_cut;
+  const bool skip = s_red[32] <= 0.25 * cut;
+  // deep-tail threshold t_d: the largest candidate norm (a discarded column
+  // with nrm2 <= cut / 4) whose next larger norm among all columns is at
+  // least 4 times it
+  double td = -1.0;
+  if (!skip)
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      const double v = nrm2[c];
+      if (cls[c] || !(v <= 0.25 * cut)) continue;
+      double nxt = INFINITY;
+      for (int h = 0; h < n; ++h)
+        if (nrm2[h] > v) nxt = fmin(nxt, nrm2[h]);
+      if (nxt >= 4.0 * v) td = fmax(td, v);
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) td = fmax(td, __shfl_xor_sync(0xffffffffu, td, o));
+  __syncthreads();
+  if (lane == 0) s_red[warp] = td;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = -1.0;
+    for (int w = 0; w < nw; ++w) v = fmax(v, s_red[w]);
+    s_red[32] = v;
+  }
+  __syncthreads();
+  td = s_red[32];
+  for (int c = threadIdx.x; c < n; c += blockDim.x)
+    cls[c] = cls[c] ? 0 : (skip ? kTailSkip : (nrm2[c] <= td ? kTailLoose : 0));
+  __syncthreads();
+  // weight of the deep tail T, summed in a fixed order, for the loose tolerance
+  part = 0.0;
+  for (int c = threadIdx.x; c < n; c += blockDim.x)
+    if (cls[c] == kTailLoose) part += nrm2[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  __syncthreads();
+  if (lane == 0) s_red[warp] = part;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < nw; ++w) v += s_red[w];
+    const double l = 2.0 / n;
+    *loose = v > 0.0 ? fmin(l, cut / (16.0 * v)) : l;
+  }
+  __syncthreads();
+}
+
+// The stopping tolerance of a pair from the classes of its columns (see
+// truncation_tail): a negative value means the pair is not rotated.
+template <typename S>
+__device__ __forceinline__ S pair_tol(int ci, int cj, S tol, S loose) {
+  const int c = min(ci, cj);
+  return c == kTailSkip ? S(-1) : (c == kTailLoose ? max(tol, loose) : tol);
+}
 
 // Position (0 .. 2P-1) -> (CTA rank, slot 0 = top / 1 = bottom).
 __device__ __forceinline__ void pos_owner(int pos, int P, int& rank, int& slot) {
@@ -133,172 +290,10 @@ __device__ __forceinline__ int jacobi_pair_reg(cplx<S> (&x)[kClusterRegs], cplx<
 
 
 
-// Double-float forms of the two pair steps (FP64-accurate sweeps; the columns
-// hold float4 = (re_h, re_l, im_h, im_l)).  The Gram entries accumulate per
-// lane as exact heads plus FP32 error terms (GramAcc) and in double-float
-// across the warp; the rotation (an FP32 angle
-// brought to unit norm in double-float, ff_angle) is applied in
-// double-float.
-__device__ __forceinline__ void ff_warp_sum4(ff& a, ff& b, ff& c, ff& d) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a = ff_add(a, ff_shfl_xor(a, o));
-    b = ff_add(b, ff_shfl_xor(b, o));
-    c = ff_add(c, ff_shfl_xor(c, o));
-    d = ff_add(d, ff_shfl_xor(d, o));
-  }
-}
-
-__device__ __forceinline__ void ff_gram_row(const float4& x, const float4& y, GramAcc& alpha, GramAcc& beta,
-                                            GramAcc& gr, GramAcc& gi) {
-  const ff xr = re_of(x), xi = im_of(x), yr = re_of(y), yi = im_of(y);
-  alpha.add(xr, xr);
-  alpha.add(xi, xi);
-  beta.add(yr, yr);
-  beta.add(yi, yi);
-  gr.add(xr, yr);
-  gr.add(xi, yi);
-  gi.add(xr, yi);
-  gi.add(ff_neg(xi), yr);
-}
-
-// x' = c x - conj(s) y, y' = c y + s x with s = sr + i si
-__device__ __forceinline__ void ff_rotate(float4& x, float4& y, ff c, ff sr, ff si) {
-  const ff xr = re_of(x), xi = im_of(x), yr = re_of(y), yi = im_of(y);
-  const ff nxr = ff_sub(ff_mul(c, xr), ff_add(ff_mul(sr, yr), ff_mul(si, yi)));
-  const ff nxi = ff_sub(ff_mul(c, xi), ff_sub(ff_mul(sr, yi), ff_mul(si, yr)));
-  const ff nyr = ff_add(ff_mul(c, yr), ff_sub(ff_mul(sr, xr), ff_mul(si, xi)));
-  const ff nyi = ff_add(ff_mul(c, yi), ff_add(ff_mul(sr, xi), ff_mul(si, xr)));
-  x = cff(nxr, nxi);
-  y = cff(nyr, nyi);
-}
-
-// 2^-e for the exponent e of a positive normal float x (x 2^-e in [1, 2)).
-__device__ __forceinline__ float pow2_inv_exponent(float x) {
-  const int e = ((__float_as_int(x) >> 23) & 0xff) - 127;
-  return __int_as_float((127 - e) << 23);
-}
-
-// The rotation of a pair from its double-float Gram entries, on the FP32
-// pipes only (this part runs FP64 at 2 FMA/clk/SM, and an FP64 angle for
-// every pair of 16 warps cost more than the rest of the pair step).  The
-// stopping test and the angle use FP32 values of the heads, scaled by a
-// power of two so that max(b_ii, b_jj) lies in [1, 2) (|g| is taken as a
-// scaled hypot, so no square underflows); b_jj - b_ii is formed in
-// double-float first, so the angle of a nearly degenerate pair is not
-// rounding noise.  The FP32 angle gives (c, s e^{i phi}) with c^2 + |s|^2 =
-// 1 + d, |d| ~ 2^-24; d is evaluated to ~2^-47 with exact products and sums
-// (two_prod, two_sum) and the rotation is scaled by f = 1 - d/2 + 3d^2/8
-// (the binomial series of (1 + d)^(-1/2)), which makes it unitary to
-// double-float rounding.  The angle itself is FP32-accurate: a pair left
-// with |g| ~ 1e-7 of its old value is rotated again in the next sweep.
-__device__ __forceinline__ bool ff_angle(ff alpha, ff beta, ff gr, ff gi, float tol, float floor, ff& c, ff& sr,
-                                         ff& si) {
-  const float a = alpha.h, b = beta.h;
-  if (!(fminf(a, b) > floor)) return false;
-  const float scl = pow2_inv_exponent(fmaxf(a, b));
-  const float xr = gr.h * scl, xi = gi.h * scl;  // |x| <= sqrt(a b) scl < 2
-  const float ax = fabsf(xr), ay = fabsf(xi);
-  const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-  if (!(mx > 0.f)) return false;
-  const float rr = mn / mx;
-  const float mag = mx * sqrtf(fmaf(rr, rr, 1.f));
-  if (!(mag > tol * sqrtf(a * scl) * sqrtf(b * scl))) return false;
-  const ff dba = ff_sub(beta, alpha);
-  const float zeta = (dba.h * scl) / (2.f * mag);
-  if (!(fabsf(zeta) < 3e38f)) return false;
-  const float t = fabsf(zeta) > 1e15f ? 0.5f / zeta
-                                       : copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
-  const float cf = rsqrtf(fmaf(t, t, 1.f));
-  const float sf = t * cf / mag;
-  // s e^{i phi} = sf (xr + i xi), exact as double-float
-  const ff s_r = two_prod(sf, xr), s_i = two_prod(sf, xi);
-  // d = c^2 + |s|^2 - 1 with exact products and sums of the heads (cf^2
-  // can round just below 1/2, so even cf^2 - 1 goes through two_sum)
-  const ff c2 = two_prod(cf, cf), r2 = two_prod(s_r.h, s_r.h), i2 = two_prod(s_i.h, s_i.h);
-  const ff u0 = two_sum(c2.h, -1.f);
-  const ff u1 = two_sum(u0.h, r2.h);
-  const ff u2 = two_sum(u1.h, i2.h);
-  const float tail = __fadd_rn(__fadd_rn(__fadd_rn(u0.l, u1.l), u2.l), __fadd_rn(c2.l, __fadd_rn(r2.l, i2.l)));
-  const float cross = 2.f * __fmaf_rn(s_r.h, s_r.l, __fmul_rn(s_i.h, s_i.l));
-  const float d = __fadd_rn(u2.h, __fadd_rn(tail, cross));
-  const float fl = __fmaf_rn(0.375f * d, d, -0.5f * d);  // f = 1 + fl
-  c = quick_two_sum(cf, __fmul_rn(cf, fl));
-  sr = quick_two_sum(s_r.h, __fmaf_rn(s_r.h, fl, s_r.l));
-  si = quick_two_sum(s_i.h, __fmaf_rn(s_i.h, fl, s_i.l));
-  return true;
-}
-
-__device__ __forceinline__ int ff_pair_smem(float4* ai, float4* aj, int m, int len, int lane, double tol, double floor,
-                                            double tiny) {
-  GramAcc ga, gb, gc, gd;
-  for (int r = lane; r < m; r += 32) ff_gram_row(ai[r], aj[r], ga, gb, gc, gd);
-  ff alpha = ga.value(), beta = gb.value(), gr = gc.value(), gi = gd.value();
-  ff_warp_sum4(alpha, beta, gr, gi);
-  ff c, sr, si;
-  if (!ff_angle(alpha, beta, gr, gi, float(tol), float(floor), c, sr, si)) return 0;
-  for (int r = lane; r < len; r += 32) {
-    float4 x = ai[r], y = aj[r];
-    ff_rotate(x, y, c, sr, si);
-    ai[r] = x;
-    aj[r] = y;
-  }
-  return 1;
-}
-
-__device__ __forceinline__ int ff_pair_reg(float4 (&x)[kClusterRegs], float4* aj, int m, int len, int lane,
-                                           double tol, double floor, double tiny) {
-  GramAcc ga, gb, gc, gd;
-#pragma unroll
-  for (int i = 0; i < kClusterRegs; ++i) {
-    const int r = lane + 32 * i;
-    if (r < m) ff_gram_row(x[i], aj[r], ga, gb, gc, gd);
-  }
-  ff alpha = ga.value(), beta = gb.value(), gr = gc.value(), gi = gd.value();
-  ff_warp_sum4(alpha, beta, gr, gi);
-  ff c, sr, si;
-  if (!ff_angle(alpha, beta, gr, gi, float(tol), float(floor), c, sr, si)) return 0;
-#pragma unroll
-  for (int i = 0; i < kClusterRegs; ++i) {
-    const int r = lane + 32 * i;
-    if (r < len) {
-      float4 y = aj[r];
-      ff_rotate(x[i], y, c, sr, si);
-      aj[r] = y;
-    }
-  }
-  return 1;
-}
-
-// |z|^2 of a stored column entry in double (complex S or double-float)
-template <bool kDF, typename C>
+// |z|^2 of a stored column entry in double
+template <typename C>
 __device__ __forceinline__ double entry_nrm2(const C* col, int r) {
-  if constexpr (kDF) {
-    const double2 z = cff_to_double2(reinterpret_cast<const float4*>(col)[r]);
-    return z.x * z.x + z.y * z.y;
-  } else {
-    return double(col[r].x) * col[r].x + double(col[r].y) * col[r].y;
-  }
-}
-
-// Symmetric first-order orthonormalisation of the V parts (rows m .. len) of
-// two stacked columns: with e = v_i^H v_j, v_i -= conj(e)/2 v_j and
-// v_j -= e/2 v_i (from the old values).
-template <typename S>
-__device__ __forceinline__ void orth_pair(cplx<S>* vi, cplx<S>* vj, int m, int len, int lane) {
-  S gr = 0, gi = 0;
-  for (int r = m + lane; r < len; r += 32) {
-    const cplx<S> x = vi[r], y = vj[r];
-    gr = fma(x.x, y.x, fma(x.y, y.y, gr));
-    gi = fma(x.x, y.y, fma(-x.y, y.x, gi));
-  }
-  gr = S(0.5) * warp_sum(gr);
-  gi = S(0.5) * warp_sum(gi);
-  for (int r = m + lane; r < len; r += 32) {
-    const cplx<S> x = vi[r], y = vj[r];
-    vi[r] = cmk<S>(x.x - fma(gr, y.x, gi * y.y), x.y - fma(gr, y.y, -gi * y.x));
-    vj[r] = cmk<S>(y.x - fma(gr, x.x, -gi * x.y), y.y - fma(gr, x.y, gi * x.x));
-  }
+  return double(col[r].x) * col[r].x + double(col[r].y) * col[r].y;
 }
 
 // Cluster-uniform sizes of one SVD.
@@ -343,55 +338,48 @@ struct ColStore {
   }
 };
 
-// Sweeps of the circle-method round robin.  kOp 0: Jacobi rotations until a
-// sweep rotates no pair (or max_sweeps); kOp 1: max_sweeps orthonormalisation
-// sweeps.  Every CTA of the cluster calls it (non-members only keep the
-// cluster barriers in step).  Returns the sweeps run.
+// Sweeps of the circle-method round robin: Jacobi rotations until a sweep
+// rotates no pair (or max_sweeps).  Every CTA of the cluster calls it
+// (non-members only keep the cluster barriers in step).  Returns the sweeps
+// run.
 //
-// Tail rule (kOp 0): at the start of each sweep every CTA learns the squared
-// norms of all columns (nrm2, through distributed shared memory) and marks
-// the columns the truncation discards (truncation_tail, into tail[]); a pair
-// of two marked columns is not rotated.
+// Tail rule: at the start of each sweep every CTA learns the squared norms of
+// all columns (nrm2, through distributed shared memory) and marks the columns
+// the truncation discards (truncation_tail, into tail[]); a pair of two
+// marked columns is not rotated.
 //
-// Clean pairs (kOp 0): a pair whose two columns have not changed since the
-// pair was last tested at the tight tolerance, and found orthogonal, is
-// orthogonal still; it is not tested again.  Byte flags per column id, kept
-// identical in every member CTA: dirty[] (rotated in this sweep; a rotation
-// sets both columns' flags in every member CTA through distributed shared
-// memory, visible by the next round's cluster barrier), dirty_prev[] (rotated
-// in the previous sweep) and tight_prev[] (tail class 0 in the previous
-// sweep).  A pair is clean when both columns are tight now and were in the
-// previous sweep, and neither was rotated in the previous sweep or so far in
-// this one.  The first sweep tests every pair.
-//
-// kDF: the columns hold double-float values (float4, see dfloat.cuh) and the
-// rotations run in double-float; T is double then.
-template <typename T, int kOp, bool kGlobal, bool kDF = false>
+// Clean pairs: a pair whose two columns have not changed since the pair was
+// last tested at the tight tolerance, and found orthogonal, is orthogonal
+// still; it is not tested again.  Byte flags per column id, kept identical in
+// every member CTA: dirty[] (rotated in this sweep; a rotation sets both
+// columns' flags in every member CTA through distributed shared memory,
+// visible by the next round's cluster barrier), dirty_prev[] (rotated in the
+// previous sweep) and tight_prev[] (tail class 0 in the previous sweep).  A
+// pair is clean when both columns are tight now and were in the previous
+// sweep, and neither was rotated in the previous sweep or so far in this one.
+// The first sweep tests every pair.
+template <typename T, bool kGlobal>
 __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColStore<T, kGlobal>& cs, int& cur, int max_sweeps, T tol, T floor,
                               T tiny, double trunc_rel, int chi_max, double* nrm2, int* tail, unsigned char* flags,
                               bool& converged, const cg::cluster_group& cluster, int* s_flag_in, int* s_any) {
   using C = cplx<T>;
-  using E = std::conditional_t<kDF, float4, C>;  // a stored entry
-  static_assert(!kDF || (sizeof(float4) == sizeof(C) && kOp == 0), "double-float columns replace complex128 ones");
   // In the cross rounds, when every warp has one top-slot column, warp w
   // keeps it in registers for the b rotations it takes part in; only the
   // bottom-slot columns are re-read, so one barrier per sub-round orders
   // their hand-off.
-  const bool cache_x = kOp == 0 && g.len <= 32 * kClusterRegs && g.b <= g.nw;
+  const bool cache_x = g.len <= 32 * kClusterRegs && g.b <= g.nw;
   __shared__ double s_loose;
   T loose = T(0);  // the tail rule's loose tolerance of the sweep (pair_tol)
   const bool active = g.member && g.wp < g.b;
   unsigned char* dirty = flags;
   unsigned char* dirty_prev = flags + g.ncols_pad;
   unsigned char* tight_prev = flags + 2 * g.ncols_pad;
-  if (kOp == 0) {
-    for (int id = threadIdx.x; id < g.ncols_pad; id += g.nt) {
-      dirty[id] = 0;
-      dirty_prev[id] = 1;
-      tight_prev[id] = 0;
-    }
-    __syncthreads();
+  for (int id = threadIdx.x; id < g.ncols_pad; id += g.nt) {
+    dirty[id] = 0;
+    dirty_prev[id] = 1;
+    tight_prev[id] = 0;
   }
+  __syncthreads();
   // a pair (column ids i, j) that needs no test (see above)
   auto clean = [&](int i, int j) -> bool {
     return tail[i] == 0 && tail[j] == 0 && tight_prev[i] && tight_prev[j] && !(dirty_prev[i] | dirty_prev[j] |
@@ -410,24 +398,22 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
   converged = false;
   for (; sweep < max_sweeps; ++sweep) {
     int rotated = 0;
-    if (kOp == 0) {
-      // squared norms of this CTA's columns (positions hold their own blocks
-      // at the start of a sweep) to every member CTA
-      for (int c = g.wp; g.member && c < 2 * g.b; c += g.nw) {
-        const C* a = cs.col(cur, c / g.b, c % g.b, 0);
-        double acc = 0.0;
-        for (int r = g.wl; r < g.m; r += 32) acc += entry_nrm2<kDF>(a, r);
-        acc = warp_sum(acc);
-        if (g.wl == 0) {
-          const int id = col_id(g, c / g.b, c % g.b, 0);
-          for (int r2 = 0; r2 < g.P; ++r2) *cluster.map_shared_rank(nrm2 + id, r2) = acc;
-        }
+    // squared norms of this CTA's columns (positions hold their own blocks
+    // at the start of a sweep) to every member CTA
+    for (int c = g.wp; g.member && c < 2 * g.b; c += g.nw) {
+      const C* a = cs.col(cur, c / g.b, c % g.b, 0);
+      double acc = 0.0;
+      for (int r = g.wl; r < g.m; r += 32) acc += entry_nrm2(a, r);
+      acc = warp_sum(acc);
+      if (g.wl == 0) {
+        const int id = col_id(g, c / g.b, c % g.b, 0);
+        for (int r2 = 0; r2 < g.P; ++r2) *cluster.map_shared_rank(nrm2 + id, r2) = acc;
       }
-      cluster.sync();
-      if (g.member) {
-        truncation_tail(nrm2, g.ncols_pad, trunc_rel, chi_max, tail, &s_loose);
-        loose = T(s_loose);
-      }
+    }
+    cluster.sync();
+    if (g.member) {
+      truncation_tail(nrm2, g.ncols_pad, trunc_rel, chi_max, tail, &s_loose);
+      loose = T(s_loose);
     }
     for (int rnd = 0; rnd < 2 * g.P - 1; ++rnd) {
       if (!g.member) {
@@ -447,35 +433,24 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
             }
             C* x = cs.col(cur, a0 / g.b, a0 % g.b, rnd);
             C* y = cs.col(cur, a1 / g.b, a1 % g.b, rnd);
-            if (kOp == 0) {
-              const int i0 = col_id(g, a0 / g.b, a0 % g.b, rnd), i1 = col_id(g, a1 / g.b, a1 % g.b, rnd);
-              const T tl = pair_tol(tail[i0], tail[i1], tol, loose);
-              if (tl >= T(0) && !clean(i0, i1)) {
-                int r;
-                if constexpr (kDF)
-                  r = ff_pair_smem(reinterpret_cast<float4*>(x), reinterpret_cast<float4*>(y), g.m, g.len, g.wl, tl,
-                                   floor, tiny);
-                else
-                  r = jacobi_pair_smem<T>(x, y, g.m, g.len, g.wl, tl, floor, tiny);
-                if (r) mark(i0, i1);
-                rotated |= r;
-              }
-            } else
-              orth_pair<T>(x, y, g.m, g.len, g.wl);
+            const int i0 = col_id(g, a0 / g.b, a0 % g.b, rnd), i1 = col_id(g, a1 / g.b, a1 % g.b, rnd);
+            const T tl = pair_tol(tail[i0], tail[i1], tol, loose);
+            if (tl >= T(0) && !clean(i0, i1)) {
+              const int r = jacobi_pair_smem<T>(x, y, g.m, g.len, g.wl, tl, floor, tiny);
+              if (r) mark(i0, i1);
+              rotated |= r;
+            }
           }
           __syncthreads();
         }
       } else {
-        E xr[kClusterRegs];
-        E* xcol = reinterpret_cast<E*>(cs.col(cur, 0, active ? g.wp : 0, rnd));
+        C xr[kClusterRegs];
+        C* xcol = cs.col(cur, 0, active ? g.wp : 0, rnd);
         if (active && cache_x) {
 #pragma unroll
           for (int i = 0; i < kClusterRegs; ++i) {
             const int r = g.wl + 32 * i;
-            if constexpr (kDF)
-              xr[i] = r < g.len ? xcol[r] : make_float4(0.f, 0.f, 0.f, 0.f);
-            else
-              xr[i] = r < g.len ? xcol[r] : cmk<T>(0, 0);
+            xr[i] = r < g.len ? xcol[r] : cmk<T>(0, 0);
           }
         }
         for (int sr = 0; sr < g.b; ++sr) {
@@ -484,13 +459,8 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
               const int i0 = col_id(g, 0, g.wp, rnd), i1 = col_id(g, 1, (g.wp + sr) % g.b, rnd);
               const T tl = pair_tol(tail[i0], tail[i1], tol, loose);
               if (tl >= T(0) && !clean(i0, i1)) {
-                int r;
-                if constexpr (kDF)
-                  r = ff_pair_reg(xr, reinterpret_cast<float4*>(cs.col(cur, 1, (g.wp + sr) % g.b, rnd)), g.m, g.len,
-                                  g.wl, tl, floor, tiny);
-                else
-                  r = jacobi_pair_reg<T>(xr, cs.col(cur, 1, (g.wp + sr) % g.b, rnd), g.m, g.len, g.wl, tl, floor,
-                                         tiny);
+                const int r = jacobi_pair_reg<T>(xr, cs.col(cur, 1, (g.wp + sr) % g.b, rnd), g.m, g.len, g.wl, tl,
+                                                 floor, tiny);
                 if (r) mark(i0, i1);
                 rotated |= r;
               }
@@ -499,21 +469,13 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
             for (int pw = g.wp; pw < g.b; pw += g.nw) {
               C* x = cs.col(cur, 0, pw, rnd);
               C* y = cs.col(cur, 1, (pw + sr) % g.b, rnd);
-              if (kOp == 0) {
-                const int i0 = col_id(g, 0, pw, rnd), i1 = col_id(g, 1, (pw + sr) % g.b, rnd);
-                const T tl = pair_tol(tail[i0], tail[i1], tol, loose);
-                if (tl >= T(0) && !clean(i0, i1)) {
-                  int r;
-                  if constexpr (kDF)
-                    r = ff_pair_smem(reinterpret_cast<float4*>(x), reinterpret_cast<float4*>(y), g.m, g.len, g.wl,
-                                     tl, floor, tiny);
-                  else
-                    r = jacobi_pair_smem<T>(x, y, g.m, g.len, g.wl, tl, floor, tiny);
-                  if (r) mark(i0, i1);
-                  rotated |= r;
-                }
-              } else
-                orth_pair<T>(x, y, g.m, g.len, g.wl);
+              const int i0 = col_id(g, 0, pw, rnd), i1 = col_id(g, 1, (pw + sr) % g.b, rnd);
+              const T tl = pair_tol(tail[i0], tail[i1], tol, loose);
+              if (tl >= T(0) && !clean(i0, i1)) {
+                const int r = jacobi_pair_smem<T>(x, y, g.m, g.len, g.wl, tl, floor, tiny);
+                if (r) mark(i0, i1);
+                rotated |= r;
+              }
             }
           }
           __syncthreads();
@@ -547,7 +509,6 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
         cluster.sync();  // global columns: this round's writes before the next round's reads
       }
     }
-    if (kOp == 1) continue;
     // ---- convergence: every CTA tells every CTA whether it rotated
     if (threadIdx.x == 0) *s_any = 0;
     __syncthreads();
@@ -578,10 +539,8 @@ __device__ __forceinline__ int cluster_sweeps(const ClusterGeom& g, const ColSto
   return sweep;
 }
 
-// Threads per CTA of the cluster SVD: FP64 columns need more registers per
-// thread (the cached column alone is 64), so FP64 CTAs stop at 8 warps and a
-// warp takes several pairs in turn when a block has more than 8 columns.
-template <typename S> constexpr int kClusterMaxThreads = sizeof(S) == 8 ? 256 : 512;
+// Threads per CTA of the cluster SVD.
+constexpr int kClusterMaxThreads = 512;
 
 template <typename S>
 struct ClusterSvdSmem {
@@ -600,19 +559,15 @@ struct ClusterSvdSmem {
   }
 };
 
-// Elements of cplx<S> the global workspace needs for a theta of capacity
-// mcap x ncap: the stacked columns (at most 2 P - 1 padding columns, P <= 16)
-// in S, plus an FP32 copy for the mixed form.
-__host__ __device__ inline size_t cluster_svd_workspace(size_t mcap, size_t ncap, size_t s_bytes) {
-  const size_t e = (ncap + 32) * (mcap + ncap);
-  return s_bytes == 8 ? e + (e + 1) / 2 : e;
+// Complex entries of the global workspace for a theta of capacity mcap x ncap:
+// the stacked columns (at most 2 P - 1 padding columns, P <= 16).
+__host__ __device__ inline size_t cluster_svd_workspace(size_t mcap, size_t ncap) {
+  return (ncap + 32) * (mcap + ncap);
 }
 
 // Everything after the geometry: the column layout (shared or global) is a
 // compile-time choice so that shared-memory accesses compile as such.
-// kDF: the FP64-accurate sweeps of the mixed form run in double-float (the
-// rebuilt FP64 columns are converted in place; see dfloat.cuh).
-template <typename S, typename R, bool kGlobal, bool kDF>
+template <typename S, typename R, bool kGlobal>
 __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg::cluster_group& cluster,
                                                  const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l,
                                                  int* __restrict__ chi, int q, const SvdParams& p,
@@ -621,19 +576,11 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
                                                  unsigned char* smem, int* s_flag_in, double* s_fro, int& s_k,
                                                  double& s_nrm, int* s_any, long long t_start) {
   using C = cplx<S>;
-  long long t_load = 0, t_lo = 0, t_fix = 0;
-  const bool mixed = sizeof(S) == 8 && p.mixed;
   const int m = g.m, ncols = g.ncols, len = g.len, b = g.b, P = g.P, me = g.me, nt = g.nt;
   const ClusterSvdSmem<S> L(b, kGlobal ? 0 : len, g.ncols_pad, nt);
   double* sig = reinterpret_cast<double*>(smem + L.sig);
   int* rnk = reinterpret_cast<int*>(smem + L.rank);
   const ColStore<S, kGlobal> cs{kGlobal ? gbuf : reinterpret_cast<C*>(smem + L.buf), b, len, P, me};
-  // FP32 columns of the mixed form: in shared memory both FP32 ping-pong
-  // buffers fit in the first S ping-pong buffer; in global memory they follow
-  // the S blocks.
-  const ColStore<float, kGlobal> cs32{kGlobal ? reinterpret_cast<cplx<float>*>(gbuf + (size_t)g.ncols_pad * len)
-                                               : reinterpret_cast<cplx<float>*>(smem + L.buf),
-                                      b, len, P, me};
 
   // ---- load: position pos holds the initial block pos (columns pos*b ..)
   for (int slot = 0; slot < 2 && g.member; ++slot) {
@@ -652,10 +599,7 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
           vr = 1.0;
         }
       }
-      if (mixed)
-        cs32.col(0, slot, c, 0)[r] = cmk<float>(float(vr), float(vi));
-      else
-        cs.col(0, slot, c, 0)[r] = cmk<S>(S(vr), S(vi));
+      cs.col(0, slot, c, 0)[r] = cmk<S>(S(vr), S(vi));
     }
   }
   // ||A||_F^2 from the theta: each CTA's share goes to every CTA, summed in rank order
@@ -689,85 +633,15 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
   double* nrm2 = sig;
   int* tail = rnk;
   unsigned char* flags = smem + L.flags;
-  int cur = 0, used = 0, used32 = 0;
+  int cur = 0;
   bool converged = false;
-  t_load = clock64();
-  t_lo = t_fix = t_load;
-  if (mixed) {
-    const float u32 = 5.9604645e-08f;
-    int cur32 = 0;
-    bool conv32 = false;
-    used32 = cluster_sweeps<float, 0, kGlobal>(g, cs32, cur32, p.max_sweeps, float(tol_scale) * u32,
-                                               float(16.0 * double(u32) * double(u32) * fro2), 1e-35f, p.trunc_rel,
-                                               p.chi_max, nrm2, tail, flags, conv32, cluster, s_flag_in, s_any);
-    used = used32;
-    t_lo = clock64();
-    // FP64 columns: V promoted (A follows from the theta below)
-    cur = kGlobal ? 0 : 1;
-    for (int slot = 0; slot < 2 && g.member; ++slot)
-      for (size_t t = threadIdx.x; t < (size_t)b * ncols; t += nt) {
-        const int c = (int)(t / ncols), r = m + (int)(t % ncols);
-        const cplx<float> v = cs32.col(cur32, slot, c, 0)[r];
-        cs.col(cur, slot, c, 0)[r] = cmk<S>(S(v.x), S(v.y));
-      }
-    // every CTA has read its FP32 columns before the first hand-over may
-    // overwrite them (in shared memory they share a buffer with FP64 ones)
-    cluster.sync();
-    // two first-order passes: E ~ 1e-6 -> E^2 -> E^4 (one pass left V
-    // unitary only to ~1e-10 after long FP32 phases)
-    for (int pass = 0; pass < 2; ++pass) {
-      bool dummy;
-      cluster_sweeps<S, 1, kGlobal>(g, cs, cur, 1, S(0), S(0), S(0), 0.0, 0, nrm2, tail, flags, dummy, cluster,
-                                    s_flag_in, s_any);
-      // the diagonal of the first-order step: |v|^2 -> 1
-      for (int c = g.wp; g.member && c < 2 * b; c += g.nw) {
-        C* v = cs.col(cur, c / b, c % b, 0);
-        S n2 = 0;
-        for (int r = m + g.wl; r < len; r += 32) n2 = fma(v[r].x, v[r].x, fma(v[r].y, v[r].y, n2));
-        n2 = warp_sum(n2);
-        const S f = S(1.5) - S(0.5) * n2;
-        if (n2 > S(0))
-          for (int r = m + g.wl; r < len; r += 32) v[r] = cmk<S>(f * v[r].x, f * v[r].y);
-      }
-      __syncthreads();
-    }
-    // A = C~ V in FP64 for this CTA's columns
-    for (size_t t = threadIdx.x; g.member && t < (size_t)2 * b * m; t += nt) {
-      const int c = (int)(t / m), r = (int)(t % m);
-      C* x = cs.col(cur, c / b, c % b, 0);
-      const cplx<R>* crow = Cm + (size_t)r * ncols;
-      S ar = 0, ai = 0;
-      for (int k = 0; k < ncols; ++k) {
-        const cplx<R> cv = crow[k];
-        const C v = x[m + k];
-        ar = fma(S(cv.x), v.x, fma(-S(cv.y), v.y, ar));
-        ai = fma(S(cv.x), v.y, fma(S(cv.y), v.x, ai));
-      }
-      const S w = S(lam_l[r >> 1]);
-      x[r] = cmk<S>(w * ar, w * ai);
-    }
-    __syncthreads();
-    if constexpr (kDF) {
-      // the stacked FP64 columns of this CTA to double-float, in place
-      for (size_t t = threadIdx.x; g.member && t < (size_t)2 * b * len; t += nt) {
-        C* col = cs.col(cur, (int)(t / ((size_t)b * len)), (int)((t / len) % b), 0);
-        const int r = (int)(t % len);
-        const double2 z = make_double2(double(col[r].x), double(col[r].y));
-        reinterpret_cast<float4*>(col)[r] = cff_from_double2(z);
-      }
-      __syncthreads();
-    }
-    t_fix = clock64();
-  }
-  // unit roundoff of the last sweeps: FP64, double-float (about 48 bits with
-  // the sloppy additions of dfloat.cuh: 2^-46 to be safe) or FP32
-  const S eps_u = kDF ? S(1.4210854715202004e-14) : (sizeof(S) == 8 ? S(1.1102230246251565e-16) : S(5.9604645e-08f));
+  const long long t_load = clock64();
+  const S eps_u = S(5.9604645e-08f);
   const S tol = p.tol > 0 ? S(p.tol) : S(tol_scale) * eps_u;
   const S floor = S(16.0 * double(eps_u) * double(eps_u) * fro2);
-  const S tiny = sizeof(S) == 8 ? S(1e-290) : S(1e-35f);
-  used += cluster_sweeps<S, 0, kGlobal, kDF>(g, cs, cur, p.max_sweeps, tol, floor, tiny, p.trunc_rel, p.chi_max, nrm2, tail,
-                                        flags, converged, cluster, s_flag_in, s_any);
-  const int sweep = used;
+  const S tiny = S(1e-35f);
+  const int sweep = cluster_sweeps<S, kGlobal>(g, cs, cur, p.max_sweeps, tol, floor, tiny, p.trunc_rel, p.chi_max, nrm2,
+                                               tail, flags, converged, cluster, s_flag_in, s_any);
 
   // ---- singular values: norms of the A parts, shared with every CTA
   const int lane = g.wl, warp = g.wp;
@@ -775,7 +649,7 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
   for (int c = warp; g.member && c < 2 * b; c += g.nw) {
     const C* a = cs.col(cur, c / b, c % b, 0);
     double acc = 0.0;
-    for (int r = lane; r < m; r += 32) acc += entry_nrm2<kDF>(a, r);
+    for (int r = lane; r < m; r += 32) acc += entry_nrm2(a, r);
     acc = warp_sum(acc);
     if (lane == 0) {
       const double sv = sqrt(acc);
@@ -834,13 +708,9 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
       // and one rotation of the stacked columns (12 (m + n) flops)
       rep->svd_flops += (double)sweep * 0.5 * ncols * (ncols - 1) * (16.0 * m + 12.0 * len);
       rep->inv_norm = 1.0 / nrm;
-      rep->sweeps_fp32 += used32;
-      (sizeof(S) == 8 ? rep->sweeps_fp64 : rep->sweeps_fp32) += sweep - used32;
-      const long long t_end = clock64();
+      rep->sweeps_fp32 += sweep;
       rep->phase_cycles[0] += double(t_load - t_start);
-      rep->phase_cycles[1] += double(t_lo - t_load);
-      rep->phase_cycles[2] += double(t_fix - t_lo);
-      rep->phase_cycles[3] += double(t_end - t_fix);
+      rep->phase_cycles[2] += double(clock64() - t_load);
       chi[q + 1] = k;
     }
   }
@@ -857,11 +727,7 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
     if (a >= k) continue;
     const C* v = cs.col(cur, c / b, c % b, 0) + m;
     for (int r = lane; r < ncols; r += 32) {
-      if constexpr (kDF)
-        Bnext[(size_t)a * ncols + r] =
-            ccast<cplx<R>>(cconj(cff_to_double2(reinterpret_cast<const float4*>(v)[r])));
-      else
-        Bnext[(size_t)a * ncols + r] = ccast<cplx<R>>(cconj(v[r]));
+      Bnext[(size_t)a * ncols + r] = ccast<cplx<R>>(cconj(v[r]));
     }
   }
   cluster.sync();  // no CTA leaves while its shared memory may still be read
@@ -869,11 +735,10 @@ __device__ __forceinline__ void svd_cluster_body(const ClusterGeom& g, const cg:
 
 
 template <typename S, typename R>
-__global__ void __launch_bounds__(kClusterMaxThreads<S>, 1)
+__global__ void __launch_bounds__(kClusterMaxThreads, 1)
     svd_cluster_kernel(const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l, int* __restrict__ chi, int q,
                        SvdParams p, cplx<R>* __restrict__ Bnext, double* __restrict__ lam_next,
                        DevReport* __restrict__ rep, cplx<S>* __restrict__ gbuf, unsigned smem_bytes) {
-  using C = cplx<S>;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_flag_in[16];
@@ -894,12 +759,10 @@ __global__ void __launch_bounds__(kClusterMaxThreads<S>, 1)
   g.nt = blockDim.x;
   g.wl = threadIdx.x & 31;
   g.wp = threadIdx.x >> 5;
-  // CTAs that take part, from the actual bond dimensions: complex64 pair
-  // steps are latency-bound, so as few CTAs as the warps allow (fewer rounds
-  // and cluster barriers); FP64 ones are bound by the FP64 units, so one pair
-  // per warp on as many CTAs as there are.  The others (rank >= P) only keep
-  // the cluster barriers in step.
-  const int per = sizeof(S) == 8 ? 1 : g.nw;
+  // CTAs that take part, from the actual bond dimensions: the pair steps are
+  // latency-bound, so as few CTAs as the warps allow (fewer rounds and cluster
+  // barriers).  The others (rank >= P) only keep the cluster barriers in step.
+  const int per = g.nw;
   g.P = min(g.Pl, max(1, (g.ncols + 2 * per - 1) / (2 * per)));
   // Without a global workspace the columns must fit the launch's shared
   // memory: fewer CTAs mean wider blocks (an FP32 theta of 96 columns takes 3
@@ -925,24 +788,254 @@ __global__ void __launch_bounds__(kClusterMaxThreads<S>, 1)
     return;
   }
   const bool in_smem = fits;
-  // the mixed form's FP64-accurate sweeps run in double-float
-  if constexpr (sizeof(S) == 8) {
-    if (p.mixed) {
-      if (in_smem)
-        svd_cluster_body<S, R, false, true>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem,
-                                            s_flag_in, s_fro, s_k, s_nrm, &s_any, t_start);
-      else
-        svd_cluster_body<S, R, true, true>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem,
-                                           s_flag_in, s_fro, s_k, s_nrm, &s_any, t_start);
-      return;
-    }
-  }
   if (in_smem)
-    svd_cluster_body<S, R, false, false>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem, s_flag_in,
+    svd_cluster_body<S, R, false>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem, s_flag_in,
                                          s_fro, s_k, s_nrm, &s_any, t_start);
   else
-    svd_cluster_body<S, R, true, false>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem, s_flag_in,
+    svd_cluster_body<S, R, true>(g, cluster, Cm, lam_l, chi, q, p, Bnext, lam_next, rep, gbuf, smem, s_flag_in,
                                         s_fro, s_k, s_nrm, &s_any, t_start);
+}
+
+// ---------------------------------------------------------------------------
+// one CTA: thetas of fewer than 96 columns
+// ---------------------------------------------------------------------------
+
+// Round-robin (circle method) schedule: in round r of nn-1 rounds, pair k.
+__device__ __forceinline__ void rr_pair(int r, int k, int nn, int& i, int& j) {
+  const int mod = nn - 1;
+  int a, b;
+  if (k == 0) {
+    a = mod;
+    b = r;
+  } else {
+    a = (r + k) % mod;
+    b = (r - k + mod) % mod;
+  }
+  i = min(a, b);
+  j = max(a, b);
+}
+
+template <typename S> struct SvdEps;
+template <> struct SvdEps<float> {
+  static __device__ float unit() { return 5.9604645e-08f; }
+  static __device__ float tiny() { return 1e-35f; }
+};
+
+// Jacobi sweeps on A (m x n, column-major) accumulating V (n x n, column-major).
+// Returns the number of sweeps used (max_sweeps + 1 if not converged).
+// Columns whose squared norm is at most `floor` (the rounding level of A)
+// are left alone: rotating two of them only reshuffles rounding noise, and a
+// rotation against a larger column would move it by less than that noise.
+// Pairs of two columns the truncation discards follow the tail rules
+// (truncation_tail, pair_tol); nrm2 and tail are n-entry shared-memory scratch.
+template <typename S>
+__device__ int jacobi_sweeps(cplx<S>* A, cplx<S>* V, int m, int n, int max_sweeps, S tol, S floor, double trunc_rel,
+                             int chi_max, double* nrm2, int* tail, int* s_flag) {
+  using C = cplx<S>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int nn = n + (n & 1);
+  const int pairs = nn / 2;
+  const S tiny = SvdEps<S>::tiny();
+  int sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    for (int j = warp; j < n; j += nwarps) {
+      double acc = 0.0;
+      for (int row = lane; row < m; row += 32) {
+        const C x = A[(size_t)j * m + row];
+        acc += double(x.x) * x.x + double(x.y) * x.y;
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) nrm2[j] = acc;
+    }
+    __syncthreads();
+    __shared__ double s_loose;
+    truncation_tail(nrm2, n, trunc_rel, chi_max, tail, &s_loose);
+    const S loose = S(s_loose);
+    if (threadIdx.x == 0) *s_flag = 0;
+    __syncthreads();
+    bool rotated = false;
+    for (int r = 0; r < nn - 1; ++r) {
+      for (int k = warp; k < pairs; k += nwarps) {
+        int i, j;
+        rr_pair(r, k, nn, i, j);
+        if (j >= n) continue;
+        const S tl = pair_tol(tail[i], tail[j], tol, loose);
+        if (tl < S(0)) continue;
+        C* ai = A + (size_t)i * m;
+        C* aj = A + (size_t)j * m;
+        S alpha = 0, beta = 0;
+        C gam = cmk<S>(0, 0);
+        for (int row = lane; row < m; row += 32) {
+          const C x = ai[row], y = aj[row];
+          alpha = fma(x.x, x.x, fma(x.y, x.y, alpha));
+          beta = fma(y.x, y.x, fma(y.y, y.y, beta));
+          cfmac(gam, x, y);
+        }
+        alpha = warp_sum(alpha);
+        beta = warp_sum(beta);
+        gam.x = warp_sum(gam.x);
+        gam.y = warp_sum(gam.y);
+        S c;
+        C sph;  // s e^{i phi}
+        if (!jacobi_rotation<S>(alpha, beta, gam.x, gam.y, tl, floor, tiny, c, sph)) continue;
+        rotated = true;
+        for (int row = lane; row < m; row += 32) {
+          const C x = ai[row], y = aj[row];
+          C ni = cmk<S>(c * x.x, c * x.y);
+          ni = csub(ni, cmulc(sph, y));  // - s e^{-i phi} y
+          C nj = cmk<S>(c * y.x, c * y.y);
+          nj = cadd(nj, cmul(sph, x));
+          ai[row] = ni;
+          aj[row] = nj;
+        }
+        C* vi = V + (size_t)i * n;
+        C* vj = V + (size_t)j * n;
+        for (int row = lane; row < n; row += 32) {
+          const C x = vi[row], y = vj[row];
+          C ni = cmk<S>(c * x.x, c * x.y);
+          ni = csub(ni, cmulc(sph, y));
+          C nj = cmk<S>(c * y.x, c * y.y);
+          nj = cadd(nj, cmul(sph, x));
+          vi[row] = ni;
+          vj[row] = nj;
+        }
+      }
+      __syncthreads();
+    }
+    if (lane == 0 && rotated) *s_flag = 1;
+    __syncthreads();
+    const int any = *s_flag;
+    __syncthreads();
+    if (!any) return sweep + 1;
+  }
+  return max_sweeps + 1;
+}
+
+// Dynamic shared memory: [A m*n | V n*n] (when use_smem) then sig[n] (double), perm[n] (int).
+template <typename S, typename R>
+__global__ void __launch_bounds__(1024, 1)
+    svd_truncate_kernel(const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l, cplx<S>* __restrict__ Ag,
+                        cplx<S>* __restrict__ Vg, int use_smem, int* __restrict__ chi, int q, SvdParams p,
+                        cplx<R>* __restrict__ Bnext, double* __restrict__ lam_next, DevReport* __restrict__ rep) {
+  using C = cplx<S>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_flag;
+  __shared__ int s_k;
+  __shared__ double s_nrm;
+  const int chi_l = chi[q], chi_r = chi[q + 2];
+  const int m = 2 * chi_l, n = 2 * chi_r;
+  C* A = Ag;
+  C* V = Vg;
+  unsigned char* tail = smem_raw;
+  if (use_smem) {
+    A = reinterpret_cast<C*>(smem_raw);
+    V = A + (size_t)m * n;
+    tail = reinterpret_cast<unsigned char*>(V + (size_t)n * n);
+  }
+  // column-major A = lam C from the row-major theta
+  for (size_t t = threadIdx.x; t < (size_t)m * n; t += blockDim.x) {
+    const int col = (int)(t % n), row = (int)(t / n);
+    const C o = ccast<C>(Cm[t]);
+    const S lam = S(lam_l[row >> 1]);
+    A[(size_t)col * m + row] = cmk<S>(lam * o.x, lam * o.y);
+  }
+  double* sig = reinterpret_cast<double*>(tail);
+  int* perm = reinterpret_cast<int*>(sig + n);
+  for (size_t t = threadIdx.x; t < (size_t)n * n; t += blockDim.x) {
+    const size_t col = t / n, row = t % n;
+    V[t] = cmk<S>(col == row ? S(1) : S(0), S(0));
+  }
+  __syncthreads();
+
+  // rotate while |b_ij| > tol sqrt(b_ii b_jj), tol = 4 sqrt(max(m, n)) u
+  const S tol = p.tol > 0 ? S(p.tol) : S(4.0 * sqrt(double(max(m, n)))) * SvdEps<S>::unit();
+  // ||A||_F^2 sets the noise floor of a column
+  {
+    double part = 0.0;
+    for (size_t t = threadIdx.x; t < (size_t)m * n; t += blockDim.x) {
+      const double x = A[t].x, y = A[t].y;
+      part += x * x + y * y;
+    }
+    part = warp_sum(part);
+    if (threadIdx.x == 0) s_nrm = 0.0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_nrm, part);
+    __syncthreads();
+  }
+  const double fro2 = s_nrm;
+  const S floor = S(16.0 * double(SvdEps<S>::unit()) * double(SvdEps<S>::unit()) * fro2);
+  __syncthreads();
+  const int sweeps = jacobi_sweeps<S>(A, V, m, n, p.max_sweeps, tol, floor, p.trunc_rel, p.chi_max, sig, perm, &s_flag);
+
+  // sigma_j = ||A_j|| (Algorithm 1: column norms)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int j = warp; j < n; j += nwarps) {
+    double acc = 0.0;
+    const C* aj = A + (size_t)j * m;
+    for (int row = lane; row < m; row += 32) {
+      const double x = aj[row].x, y = aj[row].y;
+      acc += x * x + y * y;
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) sig[j] = sqrt(acc);
+  }
+  __syncthreads();
+  // descending order, ties by index (deterministic)
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const double sj = sig[j];
+    int rank = 0;
+    for (int i = 0; i < n; ++i) {
+      const double si = sig[i];
+      rank += (si > sj) || (si == sj && i < j);
+    }
+    perm[rank] = j;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double total = 0.0;
+    for (int a = 0; a < n; ++a) total += sig[perm[a]] * sig[perm[a]];
+    const double smax = sig[perm[0]];
+    int cnt = 0;
+    for (int a = 0; a < n; ++a) {
+      const double s = sig[perm[a]];
+      if (p.trunc_rel > 0.0 ? (s > p.trunc_rel * smax) : (s > 0.0)) ++cnt;
+    }
+    int k = min(cnt, min(p.chi_max, min(m, n)));
+    if (k < 1) k = 1;
+    double kept = 0.0;
+    for (int a = 0; a < k; ++a) kept += sig[perm[a]] * sig[perm[a]];
+    double nrm = sqrt(kept);
+    if (!(nrm > 0.0)) nrm = 1.0;
+    s_k = k;
+    s_nrm = nrm;
+    rep->discarded_weight += total > 0.0 ? 1.0 - kept / total : 0.0;
+    const double smin = sig[perm[k - 1]] / nrm;
+    if (smin < rep->min_kept_sv) rep->min_kept_sv = smin;
+    if (k > rep->max_chi) rep->max_chi = k;
+    if (k < n && k == p.chi_max) {
+      const double a0 = sig[perm[k - 1]], a1 = sig[perm[k]];
+      if (a1 > 0.0 && fabs(a0 - a1) <= 1e-10 * a0) rep->degenerate_cuts += 1;
+    }
+    if (sweeps > p.max_sweeps) rep->not_converged += 1;
+    if (sweeps > rep->max_sweeps) rep->max_sweeps = sweeps;
+    rep->two_qubit_gates += 1;
+    // per sweep and column pair: three dot products over m rows (16 m flops)
+    // and one rotation of the A and V columns (12 (m + n) flops)
+    rep->svd_flops += (double)min(sweeps, p.max_sweeps) * 0.5 * n * (n - 1) * (16.0 * m + 12.0 * (m + n));
+    rep->sweeps_fp32 += min(sweeps, p.max_sweeps);
+    rep->inv_norm = 1.0 / nrm;
+    chi[q + 1] = k;
+  }
+  __syncthreads();
+  const int k = s_k;
+  const double inv = 1.0 / s_nrm;
+  for (int a = threadIdx.x; a < k; a += blockDim.x) lam_next[a] = sig[perm[a]] * inv;
+  // B~_{q+1}[a, c] = conj(V[c, perm[a]])   (V = W, right singular vectors)
+  for (size_t t = threadIdx.x; t < (size_t)k * n; t += blockDim.x) {
+    const int a = (int)(t / n), c = (int)(t % n);
+    const C v = V[(size_t)perm[a] * n + c];
+    Bnext[t] = ccast<cplx<R>>(cconj(v));
+  }
 }
 
 }  // namespace mpsv

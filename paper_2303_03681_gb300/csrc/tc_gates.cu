@@ -343,7 +343,6 @@ struct ContractWork {
   TcWork tcw;
   int* d_chi = nullptr;
   DevGate* d_gate = nullptr;
-  double* d_ones = nullptr;
   DevReport* d_rep = nullptr;
 };
 
@@ -351,7 +350,7 @@ void contract_work_free(mps_ctx* ctx) {
   if (!ctx->contract) return;
   ContractWork* c = ctx->contract;
   tc_work_free(ctx, &c->tcw);
-  for (void* p : {(void*)c->d_chi, (void*)c->d_gate, (void*)c->d_ones, (void*)c->d_rep}) dev_free(ctx, p);
+  for (void* p : {(void*)c->d_chi, (void*)c->d_gate, (void*)c->d_rep}) dev_free(ctx, p);
   delete c;
   ctx->contract = nullptr;
 }
@@ -394,12 +393,9 @@ extern "C" mps_status mps_contract_theta(mps_ctx* ctx, int32_t precision, int32_
     mps_status rc = dev_alloc(ctx, (void**)&c->d_chi, 4 * sizeof(int));
     if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&c->d_gate, sizeof(DevGate));
     if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&c->d_rep, sizeof(DevReport));
-    if (rc == MPS_OK) rc = dev_alloc(ctx, (void**)&c->d_ones, (size_t)cap * sizeof(double));
     if (rc == MPS_OK && need_tc) rc = tc_work_alloc(ctx, cap, mode, &c->tcw);
     if (rc == MPS_OK) {
-      std::vector<double> ones(cap, 1.0);
-      cudaError_t e = cudaMemcpyAsync(c->d_ones, ones.data(), cap * sizeof(double), cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(c->d_rep, 0, sizeof(DevReport), s);
+      cudaError_t e = cudaMemsetAsync(c->d_rep, 0, sizeof(DevReport), s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) rc = cuda_fail(e, "mps_contract_theta set-up");
     }
@@ -424,8 +420,7 @@ extern "C" mps_status mps_contract_theta(mps_ctx* ctx, int32_t precision, int32_
     KernelScope k(ctx, MPS_K_THETA);
     if (!need_tc) {
       const dim3 blk(kTile, kTile), grid((chi_r + kTile - 1) / kTile, (chi_l + kTile - 1) / kTile);
-      theta_kernel<float, float><<<grid, blk, 0, s>>>(Bq, Bq1, c->d_gate, c->d_ones, c->d_chi, 0, Cm,
-                                                      (float2*)nullptr);
+      theta_kernel<float><<<grid, blk, 0, s>>>(Bq, Bq1, c->d_gate, c->d_chi, 0, Cm);
     } else if (mode == kTF32) {
       launch_theta_raw<kTF32>(c->tcw, Bq, Bq1, c->d_chi, 0, chi_l, chi_m, chi_r, c->d_gate, Cm, &c->d_rep->tc_error,
                               s);

@@ -1,4 +1,5 @@
-// Double-float arithmetic for the FP64-accurate Jacobi sweeps.
+// Double-float arithmetic for the FP64-accurate SVD and the contractions of
+// complex128 states.
 //
 // This part executes FP64 at two fused multiply-adds per clock per SM and
 // FP32 at 128: a value held as the unevaluated sum of two floats (h + l,
@@ -10,8 +11,8 @@
 // about 2^-46.  The exponent range is FP32's: the kernels that use it keep
 // squared norms above the rounding floor, far from 1e-38.
 //
-// Complex double-float values are float4 (re_h, re_l, im_h, im_l): 16 bytes,
-// the size of a complex128, so the stacked-column layouts are unchanged.
+// Complex values keep (re, im) pairs of heads and of error terms, so that both
+// parts go through the packed FP32 instructions (add / mul / fma .f32x2).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -71,29 +72,8 @@ __device__ __forceinline__ ff two_prod(float a, float b) {
   return ff_make(p, __fmaf_rn(a, b, -p));
 }
 
-__device__ __forceinline__ ff ff_from_double(double x) {
-  const float h = __double2float_rn(x);
-  return ff_make(h, __double2float_rn(x - (double)h));
-}
-
-__device__ __forceinline__ double ff_to_double(ff a) { return (double)a.h + (double)a.l; }
-
 __device__ __forceinline__ ff ff_shfl_xor(ff a, int o) {
   return ff_make(__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o));
-}
-
-// complex parts of a float4 (re_h, re_l, im_h, im_l)
-__device__ __forceinline__ ff re_of(const float4& z) { return ff_make(z.x, z.y); }
-__device__ __forceinline__ ff im_of(const float4& z) { return ff_make(z.z, z.w); }
-__device__ __forceinline__ float4 cff(ff re, ff im) { return make_float4(re.h, re.l, im.h, im.l); }
-
-__device__ __forceinline__ float4 cff_from_double2(double2 z) {
-  const ff r = ff_from_double(z.x), i = ff_from_double(z.y);
-  return cff(r, i);
-}
-
-__device__ __forceinline__ double2 cff_to_double2(const float4& z) {
-  return make_double2(ff_to_double(re_of(z)), ff_to_double(im_of(z)));
 }
 
 // Sums of double-float products (the per-lane Gram sums of the Jacobi SVD,
@@ -117,27 +97,119 @@ struct GramAcc {
   __device__ __forceinline__ ff value() const { return quick_two_sum(h, e); }
 };
 
-// Complex multiply-adds on double-float operands into a pair of GramAcc.
+// ---- packed FP32 pairs --------------------------------------------------
+__device__ __forceinline__ float2 mk2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a - b, exactly rounded (the product with -1 is exact)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, mk2(-1.f, -1.f), a); }
+// s + e = a + b exactly (Knuth's two-sum)
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = add2(a, b);
+  const float2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+// (h, l) <- h + l renormalised, |h| >= |l|
+__device__ __forceinline__ void renorm2(float2& h, float2& l) {
+  const float2 s = add2(h, l);
+  l = sub2(l, sub2(s, h));
+  h = s;
+}
+// A pair of running sums of double-float products: exact heads h, error
+// terms e (the GramAcc of dfloat.cuh, two at a time).
+struct Acc2 {
+  float2 h = {0.f, 0.f}, e = {0.f, 0.f};
+  // += a b for a = (ah, al) given with its negatives
+  __device__ __forceinline__ void add(float2 ah, float2 nah, float2 nal, float2 bh, float2 bl) {
+    const float2 p = mul2(ah, bh);
+    float2 ne = fma2(nah, bh, p);  // minus the product's rounding error
+    ne = fma2(nah, bl, ne);
+    ne = fma2(nal, bh, ne);
+    float2 t;
+    two_sum2(h, p, h, t);
+    e = add2(e, sub2(t, ne));
+  }
+  __device__ __forceinline__ ff x() const { return quick_two_sum(h.x, e.x); }
+  __device__ __forceinline__ ff y() const { return quick_two_sum(h.y, e.y); }
+};
+
+// A double as a float pair by integer operations: FP64 conversions and
+// subtractions run at 1/64 of the FP32 rate here (three of them per value took
+// longer than reading the theta).  h is the value rounded to 24 bits (half up
+// in magnitude), l the signed rest rounded to 24 bits: 2^-49 relative, as
+// rounding by conversions.  Values below 2^-126 give 0; infinities and NaN
+// stay.
+__device__ __forceinline__ ff ff_split(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  const int e = (int)(b >> 52) - 1023;
+  const float sign = (__double2hiint(x) < 0) ? -1.f : 1.f;
+  if (e < -126) return ff_make(0.f, 0.f);
+  if (e > 126) return ff_make((float)x, 0.f);  // inf, NaN, and values that may overflow
+  const unsigned long long hb = (b + (1ull << 28)) >> 29;  // exponent and 23 mantissa bits, rounded
+  const int rest = (int)(long long)(b - (hb << 29));       // |rest| <= 2^28, units of 2^(e - 52)
+  const float h = __int_as_float((int)((unsigned)hb - (896u << 23)));
+  const float l = e > -75 ? (float)rest * __int_as_float((e - 52 + 127) << 23) : 0.f;
+  return ff_make(sign * h, sign * l);
+}
+
+// The double nearest to h + l, by integer operations for the same reason.
+__device__ __forceinline__ double ff_join(ff a) {
+  const unsigned hb = (unsigned)__float_as_int(a.h) & 0x7fffffffu;
+  const int e = (int)(hb >> 23);  // biased
+  if (e == 0 || e == 255) return (double)a.h;
+  // l in units of 2^(e - 127 - 52), |l| <= 2^28 of them; two exact factors
+  // keep 2^(179 - e) inside the FP32 range
+  const int up = 179 - e;
+  const float u = a.l * __int_as_float((min(up, 100) + 127) << 23) * __int_as_float((max(up - 100, 0) + 127) << 23);
+  // below a power of two the spacing halves
+  const float l = a.h < 0.f ? -u : u;
+  const int li = __float2int_rn((hb & 0x7fffffu) == 0 && l < 0.f ? 2.f * l : l);
+  const long long m = (((long long)hb + (896ll << 23)) << 29) + li;
+  return __longlong_as_double(m | (a.h < 0.f ? (long long)0x8000000000000000ull : 0ll));
+}
+
+// A complex double-float value as the contraction tiles hold it: (re, im) of
+// the heads and of the error terms.
+struct Cff {
+  float2 h, l;
+};
+__device__ __forceinline__ Cff cff_split(double2 z) {
+  const ff a = ff_split(z.x), b = ff_split(z.y);
+  Cff c;
+  c.h = mk2(a.h, b.h);
+  c.l = mk2(a.l, b.l);
+  return c;
+}
+
+// Sums of complex double-float products, re and im packed: a += (xr, xi) o
+// (yr, yi) and b += (xr, xi) o (yi, yr), from which x y and conj(x) y both
+// follow.  26 packed instructions a product, two of them the negatives of x,
+// which products with the same x share; the scalar form took 48 (the pipe
+// rate is the same, the issue slots halve).
 struct CAcc {
-  GramAcc re, im;
-  // += a b
-  __device__ __forceinline__ void fma(const float4& a, const float4& b) {
-    const ff ar = re_of(a), ai = im_of(a), br = re_of(b), bi = im_of(b);
-    re.add(ar, br);
-    re.add(ff_neg(ai), bi);
-    im.add(ar, bi);
-    im.add(ai, br);
+  Acc2 a, b;
+  __device__ __forceinline__ void add(const Cff& x, const Cff& y) {
+    const float2 m1 = mk2(-1.f, -1.f);
+    const float2 nh = mul2(x.h, m1), nl = mul2(x.l, m1);
+    a.add(x.h, nh, nl, y.h, y.l);
+    b.add(x.h, nh, nl, swap2(y.h), swap2(y.l));
   }
-  // += conj(a) b
-  __device__ __forceinline__ void fmac(const float4& a, const float4& b) {
-    const ff ar = re_of(a), ai = im_of(a), br = re_of(b), bi = im_of(b);
-    re.add(ar, br);
-    re.add(ai, bi);
-    im.add(ar, bi);
-    im.add(ff_neg(ai), br);
+  static __device__ __forceinline__ ff sum(const Acc2& p, float s) {  // p.x + s p.y, s = +-1
+    ff t = two_sum(p.h.x, s * p.h.y);
+    t.l = __fadd_rn(t.l, __fadd_rn(p.e.x, s * p.e.y));
+    return quick_two_sum(t.h, t.l);
   }
-  __device__ __forceinline__ double2 value() const {
-    return make_double2(ff_to_double(re.value()), ff_to_double(im.value()));
+  __device__ __forceinline__ double2 value() const {  // sum of x y
+    return make_double2(ff_join(sum(a, -1.f)), ff_join(sum(b, 1.f)));
+  }
+  __device__ __forceinline__ Cff value_ff() const {
+    const ff r = sum(a, -1.f), i = sum(b, 1.f);
+    return Cff{mk2(r.h, i.h), mk2(r.l, i.l)};
+  }
+  __device__ __forceinline__ double2 value_conj() const {  // sum of conj(x) y
+    return make_double2(ff_join(sum(a, 1.f)), ff_join(sum(b, -1.f)));
   }
 };
 

@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(kTile* kTile)
     __syncthreads();
   }
   if (b < chi_r && d < chi_r) {
-    C out = cmul(ccast<C>(pr.ph0), MT::value(acc0));
-    out = cadd(out, cmul(ccast<C>(pr.ph1), MT::value(acc1)));
+    C out = cmul(ccast<C>(pr.ph0), MT::value_conj(acc0));
+    out = cadd(out, cmul(ccast<C>(pr.ph1), MT::value_conj(acc1)));
     Lcur[(size_t)cidx * lv.cap_r * lv.cap_r + (size_t)b * chi_r + d] = out;
   }
 }

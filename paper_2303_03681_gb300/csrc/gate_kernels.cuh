@@ -25,9 +25,9 @@ constexpr int kTile = 16;
 // (theta, G3, the environments).  Complex64 states multiply-add in FP32.
 // Complex128 states hold their shared-memory tiles as double-float values
 // (converted once per tile load) and accumulate with exact heads plus FP32
-// error terms (CAcc) on the FP32 pipes: this part executes FP64 at 2 FMA
+// error terms (CAcc, packed) on the FP32 pipes: this part executes FP64 at 2 FMA
 // per clock per SM against 128 FP32, and a double-float multiply-add costs
-// 12 FP32 operations per real product (relative error about K 2^-47 of the
+// 13 FP32 operations per real product (relative error about K 2^-47 of the
 // sum of |terms| for K products, 1e-12 at K = 128).
 template <typename R> struct Mac;
 template <> struct Mac<float> {
@@ -39,16 +39,20 @@ template <> struct Mac<float> {
   static __device__ __forceinline__ Elem zero() { return make_float2(0.f, 0.f); }
   static __device__ __forceinline__ void fma(Acc& a, Elem x, Elem y) { cfma(a.v, x, y); }    // += x y
   static __device__ __forceinline__ void fmac(Acc& a, Elem x, Elem y) { cfmac(a.v, x, y); }  // += conj(x) y
-  static __device__ __forceinline__ float2 value(const Acc& a) { return a.v; }
+  static __device__ __forceinline__ float2 value(const Acc& a) { return a.v; }       // of fma sums
+  static __device__ __forceinline__ float2 value_conj(const Acc& a) { return a.v; }  // of fmac sums
+  static __device__ __forceinline__ Elem as_elem(const Acc& a) { return a.v; }
 };
 template <> struct Mac<double> {
-  using Elem = float4;
+  using Elem = Cff;
   using Acc = CAcc;
-  static __device__ __forceinline__ Elem load(double2 x) { return cff_from_double2(x); }
-  static __device__ __forceinline__ Elem zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-  static __device__ __forceinline__ void fma(Acc& a, Elem x, Elem y) { a.fma(x, y); }
-  static __device__ __forceinline__ void fmac(Acc& a, Elem x, Elem y) { a.fmac(x, y); }
+  static __device__ __forceinline__ Elem load(double2 x) { return cff_split(x); }
+  static __device__ __forceinline__ Elem zero() { return Cff{mk2(0.f, 0.f), mk2(0.f, 0.f)}; }
+  static __device__ __forceinline__ void fma(Acc& a, Elem x, Elem y) { a.add(x, y); }
+  static __device__ __forceinline__ void fmac(Acc& a, Elem x, Elem y) { a.add(x, y); }
   static __device__ __forceinline__ double2 value(const Acc& a) { return a.value(); }
+  static __device__ __forceinline__ double2 value_conj(const Acc& a) { return a.value_conj(); }
+  static __device__ __forceinline__ Elem as_elem(const Acc& a) { return a.value_ff(); }
 };
 
 // ---------------------------------------------------------------------------
@@ -89,67 +93,82 @@ __global__ void reset_kernel(cplx<R>* __restrict__ B, const size_t* __restrict__
 // ---------------------------------------------------------------------------
 // theta = B_q B_{q+1}; gate (G1 + G2; the SVD applies the lam scaling as it loads)
 // ---------------------------------------------------------------------------
+// One 16 x 16 tile (a_l, a_r) with both physical indices, by 256 threads (tx,
+// ty).  sL, sR: the group's tiles, 2 x 16 x 17 entries each.  Every thread of
+// the block calls it (act false: no tile, only the barriers).  The site tensors
+// are read past L1: a run of gates changes them between calls.
 template <typename R>
-__global__ void __launch_bounds__(kTile* kTile)
-    theta_kernel(const cplx<R>* __restrict__ Bl, const cplx<R>* __restrict__ Br,
-                 const DevGate* __restrict__ gate, const int* __restrict__ chi, int q, cplx<R>* __restrict__ Cm) {
+__device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const cplx<R>* __restrict__ Br,
+                                           const double2* __restrict__ u, int chi_l, int chi_m, int chi_r, int al0,
+                                           int ar0, int tx, int ty, bool act, typename Mac<R>::Elem (*sL)[kTile][kTile + 1],
+                                           typename Mac<R>::Elem (*sR)[kTile][kTile + 1], cplx<R>* __restrict__ Cm) {
   using C = cplx<R>;
   using MT = Mac<R>;
   using E = typename MT::Elem;
-  const int chi_l = chi[q], chi_m = chi[q + 1], chi_r = chi[q + 2];
-  const int al0 = blockIdx.y * kTile, ar0 = blockIdx.x * kTile;
-  if (al0 >= chi_l || ar0 >= chi_r) return;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  __shared__ E sL[2][kTile][kTile + 1];
-  __shared__ E sR[2][kTile][kTile + 1];
   typename MT::Acc acc[2][2];
-  const C zero = cmk<R>(0, 0);
+  const int al = al0 + ty, ar = ar0 + tx;
+  act = act && al0 < chi_l && ar0 < chi_r;
+  const bool mine = act && al < chi_l && ar < chi_r;
   for (int m0 = 0; m0 < chi_m; m0 += kTile) {
-    {
-      const int al = al0 + ty, mm = m0 + tx;
+    if (act) {
+      const int mm = m0 + tx;
       const bool ok = al < chi_l && mm < chi_m;
-      sL[0][ty][tx] = ok ? MT::load(Bl[(size_t)(al * 2 + 0) * chi_m + mm]) : MT::zero();
-      sL[1][ty][tx] = ok ? MT::load(Bl[(size_t)(al * 2 + 1) * chi_m + mm]) : MT::zero();
-    }
-    {
-      const int mm = m0 + ty, ar = ar0 + tx;
-      const bool ok = mm < chi_m && ar < chi_r;
-      sR[0][ty][tx] = ok ? MT::load(Br[(size_t)(mm * 2 + 0) * chi_r + ar]) : MT::zero();
-      sR[1][ty][tx] = ok ? MT::load(Br[(size_t)(mm * 2 + 1) * chi_r + ar]) : MT::zero();
+      sL[0][ty][tx] = ok ? MT::load(__ldcg(Bl + (size_t)(al * 2 + 0) * chi_m + mm)) : MT::zero();
+      sL[1][ty][tx] = ok ? MT::load(__ldcg(Bl + (size_t)(al * 2 + 1) * chi_m + mm)) : MT::zero();
+      const int mr = m0 + ty;
+      const bool okr = mr < chi_m && ar < chi_r;
+      sR[0][ty][tx] = okr ? MT::load(__ldcg(Br + (size_t)(mr * 2 + 0) * chi_r + ar)) : MT::zero();
+      sR[1][ty][tx] = okr ? MT::load(__ldcg(Br + (size_t)(mr * 2 + 1) * chi_r + ar)) : MT::zero();
     }
     __syncthreads();
+    if (mine) {
+      const int kend = min(kTile, chi_m - m0);
 #pragma unroll 4
-    for (int kk = 0; kk < kTile; ++kk) {
-      const E l0 = sL[0][ty][kk], l1 = sL[1][ty][kk];
-      const E r0 = sR[0][kk][tx], r1 = sR[1][kk][tx];
-      MT::fma(acc[0][0], l0, r0);
-      MT::fma(acc[0][1], l0, r1);
-      MT::fma(acc[1][0], l1, r0);
-      MT::fma(acc[1][1], l1, r1);
+      for (int kk = 0; kk < kend; ++kk) {
+        const E l0 = sL[0][ty][kk], l1 = sL[1][ty][kk];
+        const E r0 = sR[0][kk][tx], r1 = sR[1][kk][tx];
+        MT::fma(acc[0][0], l0, r0);
+        MT::fma(acc[0][1], l0, r1);
+        MT::fma(acc[1][0], l1, r0);
+        MT::fma(acc[1][1], l1, r1);
+      }
     }
     __syncthreads();
   }
-  const int al = al0 + ty, ar = ar0 + tx;
-  if (al >= chi_l || ar >= chi_r) return;
+  if (!mine) return;
+  // the gate on (i', j'), in the tile's arithmetic (64 FP64 multiply-adds a
+  // thread took as long as a 16-column theta's sums)
   const int n = 2 * chi_r;
-  C th[2][2];
+  E th[2][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) th[i][j] = MT::value(acc[i][j]);
+    for (int j = 0; j < 2; ++j) th[i][j] = MT::as_elem(acc[i][j]);
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      C out = zero;
+      typename MT::Acc out;
 #pragma unroll
       for (int ip = 0; ip < 2; ++ip)
 #pragma unroll
-        for (int jp = 0; jp < 2; ++jp) cfma(out, ccast<C>(gate->u[(2 * i + j) * 4 + 2 * ip + jp]), th[ip][jp]);
-      const int row = 2 * al + i, col = j * chi_r + ar;
-      Cm[(size_t)row * n + col] = out;
+        for (int jp = 0; jp < 2; ++jp)
+          MT::fma(out, MT::load(ccast<C>(u[(2 * i + j) * 4 + 2 * ip + jp])), th[ip][jp]);
+      Cm[(size_t)(2 * al + i) * n + j * chi_r + ar] = MT::value(out);
     }
   }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kTile* kTile)
+    theta_kernel(const cplx<R>* __restrict__ Bl, const cplx<R>* __restrict__ Br,
+                 const DevGate* __restrict__ gate, const int* __restrict__ chi, int q, cplx<R>* __restrict__ Cm) {
+  __shared__ typename Mac<R>::Elem sL[2][kTile][kTile + 1];
+  __shared__ typename Mac<R>::Elem sR[2][kTile][kTile + 1];
+  const int chi_l = chi[q], chi_r = chi[q + 2];
+  const int al0 = blockIdx.y * kTile, ar0 = blockIdx.x * kTile;
+  if (al0 >= chi_l || ar0 >= chi_r) return;
+  theta_tile<R>(Bl, Br, gate->u, chi_l, chi[q + 1], chi_r, al0, ar0, threadIdx.x, threadIdx.y, true, sL, sR, Cm);
 }
 
 // ---------------------------------------------------------------------------
@@ -191,16 +210,13 @@ __global__ void __launch_bounds__(kTile* kTile)
 // one-qubit gate (exact, keeps the canonical form)
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void gate1_kernel(cplx<R>* __restrict__ B, const DevGate* __restrict__ gate, const int* __restrict__ chi,
-                             int q) {
+__device__ __forceinline__ void gate1_entry(cplx<R>* __restrict__ B, const DevGate* __restrict__ gate, int chi_r,
+                                            int t) {
   using C = cplx<R>;
-  const int chi_l = chi[q], chi_r = chi[q + 1];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= chi_l * chi_r) return;
   const int al = t / chi_r, ar = t % chi_r;
   C* p0 = B + (size_t)(al * 2 + 0) * chi_r + ar;
   C* p1 = B + (size_t)(al * 2 + 1) * chi_r + ar;
-  const C b0 = *p0, b1 = *p1;
+  const C b0 = __ldcg(p0), b1 = __ldcg(p1);
   C n0 = cmk<R>(0, 0), n1 = cmk<R>(0, 0);
   cfma(n0, ccast<C>(gate->u[0]), b0);
   cfma(n0, ccast<C>(gate->u[1]), b1);
@@ -208,6 +224,13 @@ __global__ void gate1_kernel(cplx<R>* __restrict__ B, const DevGate* __restrict_
   cfma(n1, ccast<C>(gate->u[3]), b1);
   *p0 = n0;
   *p1 = n1;
+}
+
+template <typename R>
+__global__ void gate1_kernel(cplx<R>* __restrict__ B, const DevGate* __restrict__ gate, const int* __restrict__ chi,
+                             int q) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < chi[q] * chi[q + 1]) gate1_entry<R>(B, gate, chi[q + 1], t);
 }
 
 // ---------------------------------------------------------------------------

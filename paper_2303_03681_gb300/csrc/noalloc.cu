@@ -25,7 +25,6 @@
 
 #include "gate_kernels.cuh"
 #include "internal.h"
-#include "svd_launch.cuh"
 
 namespace mpsv {
 namespace {
@@ -56,7 +55,8 @@ mps_status scratch_for(int dev, unsigned char** out) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc: cudaGetSymbolAddress");
-    e = svd_attrs<ArF64, double>();
+    svd_prime_f64();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc: set-up");
     g_scratch_addr[dev] = static_cast<unsigned char*>(p);
   }
@@ -160,11 +160,9 @@ extern "C" mps_status mps_gate2_noalloc(int device, void* cuda_stream, int32_t c
   p.max_sweeps = 60;
   p.trunc_rel = trunc_rel;
   p.tol = 0.0;
-  const int n = 2 * chi_r, m = 2 * chi_l;
-  const size_t smem = SvdSmem<ArF64>::bytes(m, n, 1, true, true);
-  svd_kernel<ArF64, double><<<1, kSvdThreads<ArF64>, smem, s>>>(C, lam_left, chi, 0, p, Br, lam_out, rep, Bl,
-                                                                reinterpret_cast<char*>(scratch + kOffWs),
-                                                                (unsigned)smem);
+  // the workspace of a 64 x 64 theta is 83 KB of the 128 KB behind C
+  svd_launch_f64(SvdJob{2 * chi_l, 2 * chi_r, false, C, lam_left, chi, 0, p, Br, lam_out, rep, Bl,
+                        reinterpret_cast<char*>(scratch + kOffWs), s});
   noalloc_finish_kernel<<<1, 32, 0, s>>>(scratch, chi_out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "mps_gate2_noalloc launch");

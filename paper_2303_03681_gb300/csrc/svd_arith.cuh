@@ -18,44 +18,6 @@
 
 namespace mpsv {
 
-// ---- packed FP32 pairs --------------------------------------------------
-__device__ __forceinline__ float2 mk2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b, exactly rounded (the product with -1 is exact)
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, mk2(-1.f, -1.f), a); }
-// s + e = a + b exactly (Knuth's two-sum)
-__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
-  s = add2(a, b);
-  const float2 bb = sub2(s, a);
-  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-}
-// (h, l) <- h + l renormalised, |h| >= |l|
-__device__ __forceinline__ void renorm2(float2& h, float2& l) {
-  const float2 s = add2(h, l);
-  l = sub2(l, sub2(s, h));
-  h = s;
-}
-// A pair of running sums of double-float products: exact heads h, error
-// terms e (the GramAcc of dfloat.cuh, two at a time).
-struct Acc2 {
-  float2 h = {0.f, 0.f}, e = {0.f, 0.f};
-  // += a b for a = (ah, al) given with its negatives
-  __device__ __forceinline__ void add(float2 ah, float2 nah, float2 nal, float2 bh, float2 bl) {
-    const float2 p = mul2(ah, bh);
-    float2 ne = fma2(nah, bh, p);  // minus the product's rounding error
-    ne = fma2(nah, bl, ne);
-    ne = fma2(nal, bh, ne);
-    float2 t;
-    two_sum2(h, p, h, t);
-    e = add2(e, sub2(t, ne));
-  }
-  __device__ __forceinline__ ff x() const { return quick_two_sum(h.x, e.x); }
-  __device__ __forceinline__ ff y() const { return quick_two_sum(h.y, e.y); }
-};
-
 // 1 / sqrt(a) in double-float: FP32 seed and one Newton step whose residual
 // 1 - a y^2 is formed with the exact square of the seed
 __device__ __forceinline__ ff ff_rsqrt(ff a) {
@@ -63,25 +25,6 @@ __device__ __forceinline__ ff ff_rsqrt(ff a) {
   const ff p = ff_mul(a, two_prod(y, y));
   const float d = __fadd_rn(__fsub_rn(1.f, p.h), -p.l);
   return quick_two_sum(y, y * fmaf(0.375f * d, d, 0.5f * d));
-}
-
-// A double as a float pair by integer operations: FP64 conversions and
-// subtractions run at 1/64 of the FP32 rate here (three of them per value took
-// longer than reading the theta).  h is the value rounded to 24 bits (half up
-// in magnitude), l the signed rest rounded to 24 bits: 2^-49 relative, as
-// rounding by conversions.  Values below 2^-126 give 0; infinities and NaN
-// stay.
-__device__ __forceinline__ ff ff_split(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-  const int e = (int)(b >> 52) - 1023;
-  const float sign = (__double2hiint(x) < 0) ? -1.f : 1.f;
-  if (e < -126) return ff_make(0.f, 0.f);
-  if (e > 126) return ff_make((float)x, 0.f);  // inf, NaN, and values that may overflow
-  const unsigned long long hb = (b + (1ull << 28)) >> 29;  // exponent and 23 mantissa bits, rounded
-  const int rest = (int)(long long)(b - (hb << 29));       // |rest| <= 2^28, units of 2^(e - 52)
-  const float h = __int_as_float((int)((unsigned)hb - (896u << 23)));
-  const float l = e > -75 ? (float)rest * __int_as_float((e - 52 + 127) << 23) : 0.f;
-  return ff_make(sign * h, sign * l);
 }
 
 // ---- rotations -----------------------------------------------------------
@@ -229,8 +172,8 @@ struct ArDF {
     v.l = mk2(a.l, b.l);
     return v;
   }
-  __device__ static __forceinline__ S from_double(double x) { return ff_from_double(x); }
-  __device__ static __forceinline__ double to_double(S x) { return ff_to_double(x); }
+  __device__ static __forceinline__ S from_double(double x) { return ff_split(x); }
+  __device__ static __forceinline__ double to_double(S x) { return ff_join(x); }
   __device__ static __forceinline__ float to_float(S x) { return x.h; }
   __device__ static __forceinline__ S zero() { return ff_make(0.f, 0.f); }
   __device__ static __forceinline__ S shfl_add(S x, int o) { return ff_add(x, ff_shfl_xor(x, o)); }
@@ -256,6 +199,40 @@ struct ArDF {
     }
     re = quick_two_sum(h.x, e.x);
     im = quick_two_sum(h.y, e.y);
+  }
+  // dot_sum and the sum of a squared norm in one run of stages
+  __device__ static __forceinline__ void dot_norm_sum(const Acc& a, const Acc2& q, int G, S& re, S& im, S& nn) {
+    float2 h, t;
+    two_sum2(mk2(a.a.h.x, a.b.h.x), mk2(a.a.h.y, -a.b.h.y), h, t);
+    float2 e = add2(add2(mk2(a.a.e.x, a.b.e.x), mk2(a.a.e.y, -a.b.e.y)), t);
+    ff u = two_sum(q.h.x, q.h.y);
+    u.l = __fadd_rn(__fadd_rn(q.e.x, q.e.y), u.l);
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      const float2 h2 = mk2(__shfl_xor_sync(0xffffffffu, h.x, o), __shfl_xor_sync(0xffffffffu, h.y, o));
+      const float2 e2 = mk2(__shfl_xor_sync(0xffffffffu, e.x, o), __shfl_xor_sync(0xffffffffu, e.y, o));
+      const ff u2 = ff_shfl_xor(u, o);
+      two_sum2(h, h2, h, t);
+      e = add2(add2(e, e2), t);
+      const ff s = two_sum(u.h, u2.h);
+      u = ff_make(s.h, __fadd_rn(__fadd_rn(u.l, u2.l), s.l));
+    }
+    re = quick_two_sum(h.x, e.x);
+    im = quick_two_sum(h.y, e.y);
+    nn = quick_two_sum(u.h, u.l);
+  }
+  // the sums of two squared norms
+  __device__ static __forceinline__ void norm2_sum(const Acc2& p, const Acc2& q, int G, S& a, S& b) {
+    float2 h, t;
+    two_sum2(mk2(p.h.x, q.h.x), mk2(p.h.y, q.h.y), h, t);
+    float2 e = add2(add2(mk2(p.e.x, q.e.x), mk2(p.e.y, q.e.y)), t);
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      const float2 h2 = mk2(__shfl_xor_sync(0xffffffffu, h.x, o), __shfl_xor_sync(0xffffffffu, h.y, o));
+      const float2 e2 = mk2(__shfl_xor_sync(0xffffffffu, e.x, o), __shfl_xor_sync(0xffffffffu, e.y, o));
+      two_sum2(h, h2, h, t);
+      e = add2(add2(e, e2), t);
+    }
+    a = quick_two_sum(h.x, e.x);
+    b = quick_two_sum(h.y, e.y);
   }
   using NAcc = Acc2;
   __device__ static __forceinline__ void nrm(NAcc& acc, V x) {
@@ -345,8 +322,13 @@ struct ArDF {
   __device__ static __forceinline__ V scale(V x, S f) {
     return cval(ff_mul(ff_make(x.h.x, x.l.x), f), ff_mul(ff_make(x.h.y, x.l.y), f));
   }
+  __device__ static __forceinline__ V times(V x, float pow2) {  // exact
+    x.h = mul2(x.h, mk2(pow2, pow2));
+    x.l = mul2(x.l, mk2(pow2, pow2));
+    return x;
+  }
   __device__ static __forceinline__ double2 value(V x) {
-    return make_double2((double)x.h.x + (double)x.l.x, (double)x.h.y + (double)x.l.y);
+    return make_double2(ff_join(ff_make(x.h.x, x.l.x)), ff_join(ff_make(x.h.y, x.l.y)));
   }
   __device__ static __forceinline__ float2 value32(V x) { return x.h; }
 };
@@ -394,6 +376,24 @@ struct ArF64 {
   struct NAcc {
     double v = 0.0;
   };
+  __device__ static __forceinline__ void dot_norm_sum(const Acc& a, const NAcc& q, int G, S& re, S& im, S& nn) {
+    re = a.re;
+    im = a.im;
+    nn = q.v;
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+      nn += __shfl_xor_sync(0xffffffffu, nn, o);
+    }
+  }
+  __device__ static __forceinline__ void norm2_sum(const NAcc& p, const NAcc& q, int G, S& a, S& b) {
+    a = p.v;
+    b = q.v;
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+  }
   __device__ static __forceinline__ void nrm(NAcc& a, V x) { a.v = fma(x.x, x.x, fma(x.y, x.y, a.v)); }
   __device__ static __forceinline__ S nrm_value(const NAcc& a) { return a.v; }
   // FP32 seed and two Newton steps (1e-7 -> 1e-14 -> rounding); a within the FP32 range
@@ -443,6 +443,7 @@ struct ArF64 {
     return true;
   }
   __device__ static __forceinline__ V scale(V x, S f) { return make_double2(x.x * f, x.y * f); }
+  __device__ static __forceinline__ V times(V x, float pow2) { return make_double2(x.x * pow2, x.y * pow2); }
   __device__ static __forceinline__ double2 value(V x) { return x; }
   __device__ static __forceinline__ float2 value32(V x) { return mk2((float)x.x, (float)x.y); }
 };

@@ -74,7 +74,11 @@ struct ClusterTeam {
   static constexpr bool kGlobalA = false;
   int me, P;
   float2* mail;  // shared memory: [2][16] candidates
-  __device__ void barrier() { cg::this_cluster().sync(); }
+  int barriers = 0;
+  __device__ void barrier() {
+    cg::this_cluster().sync();
+    ++barriers;
+  }
   __device__ void publish(int par, float v, int idx) {  // threads 0 .. P-1 of one warp
     const int t = threadIdx.x;
     if (t < P) *cg::this_cluster().map_shared_rank(mail + par * 16 + me, t) = make_float2(v, __int_as_float(idx));
@@ -138,6 +142,10 @@ struct GridTeam {
 // threads, 4) outputs per thread over K steps of 16.
 constexpr int kPK = 16, kPN = 16, kPM = 64;
 constexpr size_t kProductTileBytes = (size_t)(kPM + kPK) * 20 * 16 + 16 * 16 * sizeof(double);
+// Dynamic shared memory a CTA can have (the device's 227 KB less the kernels'
+// static part); the number of CTAs a theta gets depends on its sizes and this
+// alone, so a gate's arithmetic does not depend on the launch it runs in.
+constexpr size_t kSvdSmemLimit = 232448 - 1024;
 
 // ---- layout -----------------------------------------------------------------
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -145,7 +153,7 @@ __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size
 // Dynamic shared memory of one CTA: the columns, then the per-column arrays.
 template <class A>
 struct SvdSmem {
-  size_t cols, nrm, sg, srt, rnk, na, fl, cls, total;
+  size_t nrm, sg, srt, rnk, na, fl, cls, total;
   // bytes of the column area when P CTAs share an m x n theta; a_smem: A's
   // columns in shared memory (with a copy of the pivot column when P > 1),
   // x_smem: X's blocks too
@@ -156,11 +164,24 @@ struct SvdSmem {
     const size_t b = (r + 2 * P - 1) / (2 * P);
     size_t x = x_smem ? (P == 1 ? r : 2 * b) * cx : 0;
     size_t a = a_smem ? (nloc + (P > 1 ? 1 : 0)) * ca : 0;
-    a = a > x ? a : x;
+    if (P == 1) {
+      a += x;  // one CTA writes X beside A, and keeps a copy of C where it fits
+      if (SvdSmem(align16(a + n * ca), n).total <= kSvdSmemLimit) a += n * ca;
+    } else {
+      a = a > x ? a : x;
+    }
     return align16(a > kProductTileBytes ? a : kProductTileBytes);
   }
+  // one CTA: the copy of C fits
+  __host__ __device__ static bool has_copy(int m, int n) {
+    const size_t ca = (size_t)A::ld(m) * A::kBytes, cx = (size_t)A::ld(n) * A::kBytes;
+    return SvdSmem(align16(2 * n * ca + (m < n ? m : n) * cx), n).total <= kSvdSmemLimit;
+  }
+  // allocation for one CTA and every theta within the capacities
+  __host__ __device__ static size_t bytes_one(int mcap, int ncap) {
+    return has_copy(mcap, ncap) ? bytes(mcap, ncap, 1, true, true) : kSvdSmemLimit;
+  }
   __host__ __device__ SvdSmem(size_t col, int n) {
-    cols = 0;
     nrm = align16(col);
     sg = align16(nrm + 2 * sizeof(float) * n);
     srt = align16(sg + sizeof(double) * n);
@@ -196,12 +217,21 @@ struct SvdWs {
 // rotation eight independent chains.
 constexpr int kHold = 4;
 
-// Lanes per column: a power of two in 8..32, as few as hold a column of length
-// len in registers, or give every one of the `items` columns a group.
-__device__ __forceinline__ int lanes_for(int items, int len, int T) {
-  int G = 32;
-  while (G > 8 && (items * G > T || kHold * (G >> 1) >= len)) G >>= 1;
-  return G;
+// Columns up to which the sweeps take full Gram terms from the start.
+constexpr int kHeadsCols = 24;
+
+// log2 of the lanes per column, 3 to 5.  A step's critical path is its column
+// length over the lanes, and one warp alone reaches about 60 % of a
+// scheduler's FP32 rate: as many lanes as keep 12 warps at work, but no more
+// than the column has entries (angle and reductions cost every group the
+// same, so further warps only repeat them; 34 columns: 8, 12, 16 warps 852,
+// 730, 735 us).  FP64 work fills the SM's two FP64 units from any warp: the
+// fewest lanes.  The same for every block size, and so are the sums.
+template <class A> __device__ __forceinline__ int lanes_log2(int items, int len) {
+  constexpr int cap = 32 * (std::is_same<A, ArF64>::value ? 1 : 12);
+  int lg = 5;
+  while (lg > 3 && ((items << lg) > cap || (1 << (lg - 1)) >= len)) --lg;
+  return lg;
 }
 
 // Largest value and its lowest index over nrm[0 .. n) (non-negative floats
@@ -262,7 +292,6 @@ __device__ __forceinline__ bool jacobi_pair(typename Mem<kG>::H cx, typename Mem
                                             float sig2, PairStat& st, bool& significant) {
   using S = typename A::S;
   using V = typename A::V;
-  auto add = [](S x, int o) { return A::shfl_add(x, o); };
   V x[kHold], y[kHold];
   load_hold<A, kG>(x, cx, ld, len, gl, G);
   load_hold<A, kG>(y, cy, ld, len, gl, G);
@@ -324,7 +353,8 @@ __device__ __forceinline__ bool jacobi_pair(typename Mem<kG>::H cx, typename Mem
         A::nrm(xa, A::template load<kG>(cx, ld, r));
         A::nrm(ya, A::template load<kG>(cy, ld, r));
       }
-      const S sa = group_sum(A::nrm_value(xa), G, add), sb = group_sum(A::nrm_value(ya), G, add);
+      S sa, sb;
+      A::norm2_sum(xa, ya, G, sa, sb);
       if (close) {
         na = sa;
         nb = sb;
@@ -357,7 +387,8 @@ __device__ __forceinline__ bool jacobi_pair(typename Mem<kG>::H cx, typename Mem
 
 // ---- the SVD ------------------------------------------------------------------
 // Every thread of every CTA of the team calls it.  gws: the global workspace
-// (SvdWs).  The dynamic shared memory holds an SvdSmem of the team's size.  kGX: X's blocks stay in the
+// (SvdWs).  C and lam_l are read past L1: a run of gates changes them between
+// calls.  The dynamic shared memory holds an SvdSmem of the team's size.  kGX: X's blocks stay in the
 // global workspace.  Writes B~_{q+1} (k x n), lam_{q+1}, *chi_out and the
 // report; returns k.  Bq (nullable): B~_q = C V^H / ||s[:k]|| as well.
 template <class A, class R, class Team, bool kGX>
@@ -375,6 +406,11 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   const SvdWs<A> W(m, n, kGA);
   const SvdSmem<A> L(SvdSmem<A>::col_bytes(m, n, P, !kGA, !kGX), n);
   char* gx = gws + W.x;
+  // one CTA: X follows A's n columns in shared memory
+  const unsigned x0 = std::is_same<Team, OneTeam>::value ? (unsigned)(n * ca) : 0u;
+  // and conj(C) 2^-ec follows X where it fits
+  const bool direct = std::is_same<Team, OneTeam>::value && SvdSmem<A>::has_copy(m, n);
+  const unsigned c0 = x0 + (unsigned)(rmax * cx);
   double* gnrm = reinterpret_cast<double*>(gws + W.nrm);
   double* gna = reinterpret_cast<double*>(gws + W.na);
   unsigned char* gfl = reinterpret_cast<unsigned char*>(gws + W.fl);
@@ -404,12 +440,15 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   const int nloc = (n - me + P - 1) / P;  // columns me, me + P, ... of A
   if (tid == 0) s_i[0] = s_i[1] = -100000;
   __syncthreads();
+  // small thetas are read once and held in registers
+  constexpr int kKeep = 2;
+  const bool keep = m * nloc <= kKeep * T;
+  cplx<R> zk[kKeep];
+  double lk[kKeep];
   {
     int emax = -100000, cmax = -100000;
-    for (int t = tid; t < m * nloc; t += T) {
-      const int r = t / nloc, c = me + (t - r * nloc) * P;
-      const cplx<R> z = Cm[(size_t)r * n + c];
-      const int el = ((__double2hiint(lam_l[r >> 1]) >> 20) & 0x7ff) - 1023;
+    auto look = [&](const cplx<R> z, double lam) {
+      const int el = ((__double2hiint(lam) >> 20) & 0x7ff) - 1023;
       int ez;
       if constexpr (sizeof(R) == 8) {
         ez = max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff) - 1023;
@@ -418,6 +457,23 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       }
       emax = max(emax, el + ez);
       cmax = max(cmax, ez);
+    };
+    if (keep) {
+#pragma unroll
+      for (int i = 0; i < kKeep; ++i) {
+        const int t = tid + i * T;
+        if (t < m * nloc) {
+          const int r = t / nloc;
+          zk[i] = __ldcg(Cm + (size_t)r * n + me + (t - r * nloc) * P);
+          lk[i] = __ldcg(lam_l + (r >> 1));
+          look(zk[i], lk[i]);
+        }
+      }
+    } else {
+      for (int t = tid; t < m * nloc; t += T) {
+        const int r = t / nloc;
+        look(__ldcg(Cm + (size_t)r * n + me + (t - r * nloc) * P), __ldcg(lam_l + (r >> 1)));
+      }
     }
     emax = __reduce_max_sync(0xffffffffu, emax);
     cmax = __reduce_max_sync(0xffffffffu, cmax);
@@ -450,15 +506,26 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   const double cscl = __longlong_as_double((long long)(1023 - ec) << 52);  // 2^-ec
 
   // ---- load this CTA's columns of A and their squared norms
-  for (int t = tid; t < m * nloc; t += T) {
-    const int r = t / nloc, i = t - r * nloc, c = me + i * P;
-    const cplx<R> z = Cm[(size_t)r * n + c];
-    const double w = lam_l[r >> 1] * scl;
-    A::template store<kGA>(acol(i, c), lda, r, A::make(w * double(z.x), w * double(z.y)));
+  auto place = [&](int t, const cplx<R> z, double lam) {
+    const int r = t / nloc, i = t - r * nloc;
+    const double w = lam * scl;
+    A::template store<kGA>(acol(i, me + i * P), lda, r, A::make(w * double(z.x), w * double(z.y)));
+    if (direct)
+      A::template store<false>(c0 + (unsigned)(i * ca), lda, r, A::make(cscl * double(z.x), -cscl * double(z.y)));
+  };
+  if (keep) {
+#pragma unroll
+    for (int i = 0; i < kKeep; ++i)
+      if (tid + i * T < m * nloc) place(tid + i * T, zk[i], lk[i]);
+  } else {
+    for (int t = tid; t < m * nloc; t += T) {
+      const int r = t / nloc;
+      place(t, __ldcg(Cm + (size_t)r * n + me + (t - r * nloc) * P), __ldcg(lam_l + (r >> 1)));
+    }
   }
   __syncthreads();
   {
-    const int G = lanes_for(nloc, m, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+    const int lg = lanes_log2<A>(nloc, m), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
     for (int i0 = 0; i0 < nloc; i0 += NG) {
       const int i = i0 + grp;
       const int ii = i < nloc ? i : 0;
@@ -482,7 +549,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   float fro2 = 0.f;
   int r = 0;
   {
-    const int G = lanes_for(nloc, m, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+    const int lg = lanes_log2<A>(nloc, m), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
     if constexpr (!std::is_same<Team, OneTeam>::value) {
       // Frobenius norm over the team
       if (tid < 32) {
@@ -499,7 +566,14 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       fro2 = warp_sum(f);
     }
     const float stop2 = fmaxf(kZeroNorm2, cut_rel * cut_rel * fro2);
-    for (int j = 0; j < rmax; ++j) {
+    // Without a truncation threshold every nonzero direction is kept (the rows
+    // of B~_{q+1} then span those of the unscaled C, which keeps B~_q
+    // right-canonical on the rows that lam_q weighs with rounding noise): a
+    // residual below the noise floor is scaled up to u ||A||_F, a perturbation
+    // of A within its own rounding, and the factorisation goes on.
+    const bool keep_noise = p.trunc_rel < 8.0 * A::unit();
+    const float floor2 = (float)(A::unit() * A::unit()) * fro2;
+    for (int j = 0; j < rmax;) {
       float* nc = nrm + (j & 1) * n;
       float* nn = nrm + ((j & 1) ^ 1) * n;
       float best;
@@ -527,7 +601,21 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           }
         }
       }
-      if (!(best > stop2)) break;
+      if (!(best > stop2)) {
+        if (!keep_noise || !(best > 0.f) || !(floor2 > stop2)) break;
+        const float up = pow2f(max(1, min(60, (exp_of(floor2) - exp_of(best)) / 2)));
+        for (int t = tid; t < m * nloc; t += T) {
+          const int i = t / m, rr = t - i * m;
+          if (nc[i] < 0.f) continue;
+          const HA col = acol(i, me + i * P);
+          A::template store<kGA>(col, lda, rr, A::times(A::template load<kGA>(col, lda, rr), up));
+        }
+        __syncthreads();
+        for (int i = tid; i < nloc; i += T)
+          if (nc[i] >= 0.f) nc[i] *= up * up;
+        tm.barrier();
+        continue;
+      }
       const int pc = owner + li * P;  // pivot column of A
       HA pcol = acol(li, pc);
       if constexpr (std::is_same<Team, ClusterTeam>::value) {
@@ -542,25 +630,31 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       // the pivot's norm, then per column: dot product with the pivot, its
       // share subtracted, the new residual norm
       V px[kHold];
-      load_hold<A, kGA>(px, pcol, lda, m, gl, G);
       const int step = kHold * G, nh = held_count(m, G);
-      typename A::NAcc pn;
-#pragma unroll
-      for (int i = 0; i < kHold; ++i)
-        if (i < nh) A::nrm(pn, px[i]);
-      for (int rr = gl + step; rr < m; rr += G) A::nrm(pn, A::template load<kGA>(pcol, lda, rr));
-      const S p2 = group_sum(A::nrm_value(pn), G, addS);
-      const S pinv = A::rsqrt(p2);
-      const S pinv2 = A::mul(pinv, pinv);
-      char* xj = gx + (size_t)j * cx;
+      S p2 = A::zero(), pinv = p2, pinv2 = p2;  // |p|^2, 1 / |p|, 1 / |p|^2
+      bool have_p = false;
+      auto put = [&](int c, V v) {  // X[c, j]
+        if constexpr (std::is_same<Team, OneTeam>::value)
+          A::template store<false>((unsigned)(x0 + j * cx), ldx, c, v);
+        else
+          A::template store<true>(gx + (size_t)j * cx, ldx, c, v);
+      };
       for (int i0 = 0; i0 < nloc; i0 += NG) {
         const int i = i0 + grp;
         const int c = me + i * P;
         const bool in = i < nloc;
         const bool alive = in && nc[in ? i : 0] >= 0.f && c != pc;
-        if (__any_sync(0xffffffffu, alive)) {
+        if (__any_sync(0xffffffffu, alive || (in && c == pc))) {
           const HA col = alive ? acol(i, c) : pcol;
           V y[kHold];
+          typename A::NAcc pn;
+          if (!have_p) {
+            load_hold<A, kGA>(px, pcol, lda, m, gl, G);
+#pragma unroll
+            for (int t = 0; t < kHold; ++t)
+              if (t < nh) A::nrm(pn, px[t]);
+            for (int rr = gl + step; rr < m; rr += G) A::nrm(pn, A::template load<kGA>(pcol, lda, rr));
+          }
           load_hold<A, kGA>(y, col, lda, m, gl, G);
           typename A::Acc acc;
 #pragma unroll
@@ -569,7 +663,14 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           for (int rr = gl + step; rr < m; rr += G)
             A::dot(acc, A::template load<kGA>(pcol, lda, rr), A::template load<kGA>(col, lda, rr));
           S dr, di;
-          A::dot_sum(acc, G, dr, di);
+          if (!have_p) {
+            have_p = true;
+            A::dot_norm_sum(acc, pn, G, dr, di, p2);
+            pinv = A::rsqrt(p2);
+            pinv2 = A::mul(pinv, pinv);
+          } else {
+            A::dot_sum(acc, G, dr, di);
+          }
           float v = 0.f;
           if (alive) {
             const auto k = A::axpy_const(A::mul(dr, pinv2), A::mul(di, pinv2));
@@ -589,15 +690,15 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           if (alive && gl == 0) {
             nn[i] = v;
-            A::template store<true>(xj, ldx, c, A::cval(A::mul(dr, pinv), A::sub(A::zero(), A::mul(di, pinv))));
+            put(c, A::cval(A::mul(dr, pinv), A::sub(A::zero(), A::mul(di, pinv))));
           }
         }
         if (in && !alive && gl == 0) {
           nn[i] = -1.f;
-          A::template store<true>(xj, ldx, c, A::cval(c == pc ? A::mul(p2, pinv) : A::zero(), A::zero()));
+          put(c, A::cval(c == pc ? A::mul(p2, pinv) : A::zero(), A::zero()));
         }
       }
-      ++r;
+      r = ++j;
       __syncthreads();
     }
   }
@@ -608,7 +709,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       const double z = fro2 - fro2;
       for (int c = tid; c < n; c += T) Bnext[c] = cmk<R>(R(c == 0 ? 1.0 + z : z), R(0));
       if (Bq)
-        for (int row = tid; row < m; row += T) Bq[row] = Cm[(size_t)row * n];
+        for (int row = tid; row < m; row += T) Bq[row] = __ldcg(Cm + (size_t)row * n);
       if (tid == 0) {
         lam_next[0] = z;
         *chi_out = 1;
@@ -635,7 +736,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     if constexpr (kGX)
       return gx + (size_t)id * cx;
     else
-      return (unsigned)(i * cx);
+      return (unsigned)(x0 + i * cx);
   };
   auto fetch = [&](int slot, int blk) {  // home -> slot
     if constexpr (!kGX) {
@@ -674,8 +775,9 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       fl[id] = __ldcg(gfl + id);
     }
   };
-  tm.barrier();  // X complete (and A's shared memory free)
-  for (int slot = 0; slot < nslots; ++slot) fetch(slot, block_at(slot, 0));
+  tm.barrier();  // X complete (and, with several CTAs, A's shared memory free)
+  if (P > 1)
+    for (int slot = 0; slot < nslots; ++slot) fetch(slot, block_at(slot, 0));
   for (int id = tid; id < r; id += T) fl[id] = 2;  // bit 0: rotated in this sweep, bit 1: in the previous one
   __syncthreads();
 
@@ -689,18 +791,22 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   // the pair step compares squares
   const float sig2 = tol_sig * tol_sig, rot2 = tol_rot * tol_rot, heads2 = tol_heads * tol_heads;
   const int kcap = min(p.chi_max, rmax);
-  const float thr_rel2 = (float)(p.trunc_rel * p.trunc_rel);
+  const double trunc2 = p.trunc_rel * p.trunc_rel;
+  const float thr_rel2 = (float)trunc2;
   int sweep = 0;
-  bool converged = false, heads = A::kRough, prev_full = false;
+  // (few columns: the full Gram terms cost little more than the heads, and a
+  // sweep less is run)
+  bool converged = false, heads = A::kRough && r > kHeadsCols, prev_full = false;
   for (;; ++sweep) {
     // squared norms of this CTA's columns, to everyone
     {
       const int items = nslots * b;
-      const int G = lanes_for(items, n, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+      const int lg = lanes_log2<A>(items, n), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
       for (int i0 = 0; i0 < items; i0 += NG) {
         const int i = i0 + grp, slot = i >= b ? 1 : 0, c = i - slot * b;
         const int blk = block_at(slot, 0), id = blk * b + c;
         const bool ok = i < items && id < r;
+        if (!__any_sync(0xffffffffu, ok)) continue;
         const HX col = held(ok ? i : 0, ok ? id : 0);
         typename A::NAcc acc;
         if (ok)
@@ -709,9 +815,10 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         if (ok && gl == 0) {
           nA[id] = v;
           const double d = A::to_double(v);
-          if (P == 1)
+          if (P == 1) {
             sg[id] = d;
-          else
+            nrm[id] = A::to_float(v);
+          } else
             __stcg(gnrm + id, d);
         }
       }
@@ -751,17 +858,44 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     // orthogonal to each other and to T they hold the leading singular vectors
     // whatever T looks like: pairs inside T are left alone (the discarded
     // weight is the sum).
-    for (int id = tid; id < r; id += T) nrm[id] = (float)sg[id];
+    if (P > 1) {
+      for (int id = tid; id < r; id += T) nrm[id] = (float)sg[id];
+      __syncthreads();
+    }
     if (tid == 0) {
       s_i[0] = 0;
       s_i[1] = r;
       s_f[0] = 0.f;
       s_f[1] = 0.f;
     }
+    // every warp for itself: the largest norm, the columns above the threshold
+    // and the weight of the rest.  When the threshold decides the cut that
+    // weight alone settles T (all of the rest, or nothing for few columns)
+    int vm = 0, above = 0;
+    float rest = 0.f;
+    for (int id = lane; id < r; id += 32) vm = max(vm, __float_as_int(nrm[id]));
+    const float thr = thr_rel2 * __int_as_float(__reduce_max_sync(0xffffffffu, vm));
+    for (int id = lane; id < r; id += 32) {
+      const float v = nrm[id];
+      above += v > thr;
+      rest += v > thr ? 0.f : v;
+    }
+    above = __reduce_add_sync(0xffffffffu, above);
+    rest = warp_sum(rest);
+    const bool all_rest = above <= kcap && rest <= 0.25f * thr;
+    if (all_rest || r <= 32) {
+      __syncthreads();
+      for (int id = tid; id < r; id += T) {
+        const unsigned char c = all_rest && !(nrm[id] > thr) ? 1 : 0;
+        if (sweep > 0 && c != cls[id]) fl[id] |= 2;  // tested again when it joins or leaves T
+        cls[id] = c;
+      }
+    } else {
     __syncthreads();
     {
-      const int G = lanes_for(r, r, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+      const int lg = lanes_log2<A>(r, r), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
       for (int i0 = 0; i0 < r; i0 += NG) {
+        if (!__any_sync(0xffffffffu, i0 + grp < r)) continue;
         const int id = min(i0 + grp, r - 1);
         const float v = nrm[id];
         int rk = 0;
@@ -779,14 +913,8 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     }
     __syncthreads();
     {
-      const float thr = thr_rel2 * srt[0];
-      int cnt = 0;
-      for (int t = tid; t < r; t += T) cnt += srt[t] > thr;
-      cnt = __reduce_add_sync(0xffffffffu, cnt);
-      if (lane == 0 && cnt) atomicAdd(&s_i[0], cnt);
-      __syncthreads();
-      const int kept = max(1, min(s_i[0], kcap));
-      const float lim = s_i[0] >= kcap ? INFINITY : thr;
+      const int kept = max(1, min(above, kcap));
+      const float lim = above >= kcap ? INFINITY : thr;
       for (int t = tid; t < r; t += T) {
         if (t < kept) continue;
         float w = 0.f;
@@ -801,6 +929,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       // a column that joins or leaves T is tested again
       if (sweep > 0 && c != cls[id]) fl[id] |= 2;
       cls[id] = c;
+    }
     }
     __syncthreads();
 
@@ -829,7 +958,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     // the others pair the columns of its two blocks.
     const int nl = P == 1 ? r : 2 * b;  // columns held
     const int np = nl + (nl & 1), mod = np - 1, pairs = np >> 1;
-    const int G = lanes_for(pairs, n, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+    const int lg = lanes_log2<A>(pairs, n), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
     for (int rnd = 0; rnd < (P == 1 ? 1 : M); ++rnd) {
       const int b0 = block_at(0, rnd), b1 = block_at(1, rnd);
       const int ns = rnd == 0 ? mod : b;
@@ -887,22 +1016,27 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       }
     }
     __syncthreads();
+    if (P == 1 && !heads && s_f[1] == 0.f) {
+      // nothing above the tolerance was rotated: the norms stand
+      converged = true;
+      ++sweep;
+      break;
+    }
     if (P > 1 && tid == 0) __stcg(gstat + ((sweep + 1) & 1) * 256 + me, make_float2(s_f[0], s_f[1]));
     for (int id = tid; id < r; id += T) fl[id] = (fl[id] & 1) ? 2 : 0;
     __syncthreads();
   }
   const long long t_sw = clock64();
 
-  // ---- singular values (in units of 2^ex until they are written), ranks
-  // (descending, ties by index), truncation
-  for (int id = tid; id < r; id += T) {
-    const double v = sg[id];
-    sg[id] = v > (double)kZeroNorm2 * 1e-2 ? sqrt(v) : (v != v ? v : 0.0);
-  }
+  // ---- squared singular values (in units of 4^ex), ranks (descending, ties by
+  // index), truncation
+  for (int id = tid; id < r; id += T)
+    if (sg[id] <= (double)kZeroNorm2 * 1e-2) sg[id] = 0.0;
   __syncthreads();
   {
-    const int G = lanes_for(r, r, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+    const int lg = lanes_log2<A>(r, r), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
     for (int i0 = 0; i0 < r; i0 += NG) {
+      if (!__any_sync(0xffffffffu, i0 + grp < r)) continue;
       const int id = min(i0 + grp, r - 1);
       const long long v = __double_as_longlong(sg[id]);  // non-negative doubles order as integers
       int rk = 0;
@@ -915,49 +1049,68 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     }
   }
   __syncthreads();
-  if (tid < 32) {
-    double total = 0.0, smax = 0.0;
-    for (int id = lane; id < r; id += 32) {
-      const double s = sg[id];
-      total += s * s;
-      smax = fmax(smax, s);
-    }
-    total = warp_sum(total);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+  // kept count: every warp for itself
+  int k;
+  {
+    long long vmax = 0;
+    for (int id = lane; id < r; id += 32) vmax = max(vmax, rnk[id] == 0 ? __double_as_longlong(sg[id]) : 0ll);
+    const unsigned who = __ballot_sync(0xffffffffu, vmax != 0);
+    vmax = __shfl_sync(0xffffffffu, vmax, who ? __ffs(who) - 1 : 0);
+    const long long thr = __double_as_longlong(trunc2 * __longlong_as_double(vmax));
     int cnt = 0;
-    const double thr = p.trunc_rel > 0.0 ? p.trunc_rel * smax : 0.0;
-    for (int id = lane; id < r; id += 32) cnt += sg[id] > thr;
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    const int k = max(1, min(cnt, kcap));
-    double kept = 0.0, smin = 0.0, s_next = 0.0;
+    for (int id = lane; id < r; id += 32) cnt += __double_as_longlong(sg[id]) > thr;
+    k = max(1, min(__reduce_add_sync(0xffffffffu, cnt), kcap));
+  }
+  // (FP64 sweeps of few columns leave less than the product's own rounding)
+  const bool refine = sizeof(R) == 8 && (std::is_same<A, ArDF>::value || n >= 32);
+  if (tid >= T - 32 && (me == 0 || !refine)) {
+    // 1 / ||s[:k]|| and the report, by the last warp while the others go on;
+    // sums and quotients in the sweeps' arithmetic (a chain of FP64 roots and
+    // divisions took 5 us of every gate, whatever its size)
+    S kept = A::zero(), drop = kept, vmin = kept, vnext = kept;
     for (int id = lane; id < r; id += 32) {
-      const double s = sg[id];
-      if (rnk[id] < k) kept += s * s;
-      if (rnk[id] == k - 1) smin = s;
-      if (rnk[id] == k) s_next = s;
+      const S v = A::from_double(sg[id]);
+      if (rnk[id] < k)
+        kept = A::add(kept, v);
+      else
+        drop = A::add(drop, v);
+      if (rnk[id] == k - 1) vmin = v;
+      if (rnk[id] == k) vnext = v;
     }
-    kept = warp_sum(kept);
-    smin = warp_sum(smin);
-    s_next = warp_sum(s_next);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      kept = A::shfl_add(kept, o);
+      drop = A::shfl_add(drop, o);
+      vmin = A::shfl_add(vmin, o);
+      vnext = A::shfl_add(vnext, o);
+    }
+    // lanes 0, 1, 2: reciprocal roots of the kept weight, s_k^2, the total
+    const S total = A::add(kept, drop);
+    const S y = lane == 0 ? kept : (lane == 1 ? vmin : total);
+    const bool pos = A::to_float(y) > 0.f;
+    const S ry = A::rsqrt(pos ? y : A::from_double(1.0));
+    const double inv = __shfl_sync(0xffffffffu, A::to_double(ry), 0);
+    double out = inv;                                                                  // lane 0
+    if (lane == 1) out = pos ? A::to_double(A::mul(y, ry)) * inv : 0.0;                // s_k / ||s[:k]||
+    if (lane == 2) out = pos ? A::to_double(A::mul(A::mul(drop, ry), ry)) : 0.0;       // discarded share
+    const double ratio = __shfl_sync(0xffffffffu, out, 1), share = __shfl_sync(0xffffffffu, out, 2);
     if (lane == 0) {
-      double nr = sqrt(kept);
-      if (!(nr > 0.0)) nr = 1.0;
-      s_i[0] = k;
-      s_d[0] = nr;
-      s_d[1] = 1.0 / nr;
+      if (!refine) s_d[1] = inv;
       if (me == 0) {
-        rep->discarded_weight += total > 0.0 ? 1.0 - kept / total : 0.0;
-        if (smin / nr < rep->min_kept_sv) rep->min_kept_sv = smin / nr;
+        rep->discarded_weight += share;
+        if (ratio < rep->min_kept_sv) rep->min_kept_sv = ratio;
         if (k > rep->max_chi) rep->max_chi = k;
-        if (k < r && k == p.chi_max && s_next > 0.0 && fabs(smin - s_next) <= 1e-10 * smin) rep->degenerate_cuts += 1;
+        // s_k and s_{k+1} equal to 1e-10 (their squares to 2e-10)
+        if (k < r && k == p.chi_max && A::to_float(vnext) > 0.f &&
+            fabsf(A::to_float(A::sub(vmin, vnext))) <= 2e-10f * A::to_float(vmin))
+          rep->degenerate_cuts += 1;
         if (!converged) rep->not_converged += 1;
         const int used = converged ? sweep : p.max_sweeps + 1;
         if (used > rep->max_sweeps) rep->max_sweeps = used;
         rep->two_qubit_gates += 1;
         // per sweep and column pair: a dot product (8 n flops; 16 n with the
         // two norms of Algorithm 1, counted as before) and a rotation (12 n)
-        rep->svd_flops += (double)sweep * 0.5 * r * (r - 1) * 28.0 * n;
+        rep->svd_flops += (double)(sweep * (r * (r - 1) / 2)) * (double)(28 * n);
         rep->sweeps_fp64 += sweep;
         rep->phase_cycles[0] += double(t_load - t_start);
         rep->phase_cycles[1] += double(t_gs - t_load);
@@ -967,14 +1120,10 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       }
     }
   }
-  __syncthreads();
-  const int k = s_i[0];
-  // (FP64 sweeps of few columns leave less than the product's own rounding)
-  const bool refine = sizeof(R) == 8 && (std::is_same<A, ArDF>::value || n >= 32);
   // ---- B~_{q+1}[a, :] = conj(X[:, id]) / |X[:, id]|
   {
     const int items = nslots * b;
-    const int G = lanes_for(items, n, T), gl = tid & (G - 1), grp = tid / G, NG = T / G;
+    const int lg = lanes_log2<A>(items, n), G = 1 << lg, gl = tid & (G - 1), grp = tid >> lg, NG = T >> lg;
     for (int i = grp; i < items; i += NG) {
       const int slot = i >= b ? 1 : 0, c = i - slot * b;
       const int blk = block_at(slot, 0), id = blk * b + c;
@@ -994,26 +1143,135 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       }
     }
   }
-  if (!refine && me == 0)
+  if (!refine) {
+    __syncthreads();  // s_d[1]
+    if (me == 0) {
+      for (int id = tid; id < r; id += T)
+        if (rnk[id] < k) lam_next[rnk[id]] = sqrt(sg[id]) * s_d[1];
+      if (tid == 0) rep->inv_norm = s_d[1] * scl;
+    }
+    if (!Bq) return k;
+  }
+  const double w_unit = __longlong_as_double((long long)(1023 + max(-1000, min(1000, ec - ex))) << 52);
+  S* kn = reinterpret_cast<S*>(nrm);  // squared kept values, in units of 4^ec
+  // ||s||, and lam = s / ||s|| in descending order (a running minimum: the
+  // refined values of a degenerate pair can differ in their last bits either
+  // way), by warp 0.  Roots: double-float seeds, one FP64 Newton step each.
+  auto finish_lam = [&](auto value) {
+    if (tid < 32) {
+      ff kept = ff_make(0.f, 0.f);
+      for (int a = lane; a < k; a += 32) kept = ff_add(kept, value(a));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) kept = ff_add(kept, ff_shfl_xor(kept, o));
+      const ff one = ff_make(1.f, 0.f);
+      const bool any = kept.h > 1e-36f;
+      const double kd = any ? ff_join(kept) : 1.0;
+      double inv = ff_join(ff_rsqrt(any ? kept : one));
+      inv = inv * fma(-0.5 * kd * inv, inv, 1.5);
+      if (lane == 0) s_d[1] = inv;  // 1 / ||s|| in units of 2^-ec
+      if (me == 0) {
+        double run = 1e300;
+        for (int a0 = 0; a0 < k; a0 += 32) {
+          double l = run;
+          if (a0 + lane < k) {
+            const ff v = value(a0 + lane);
+            // below the FP32 range of the roots (1e-18 of ||C||): a token value,
+            // which keeps the direction alive for the next gate on its bond
+            const bool pos = v.h > 1e-36f;
+            const double vd = pos ? ff_join(v) : 0.0, y = ff_join(ff_rsqrt(pos ? v : one));
+            const double s0 = vd * y;
+            l = pos ? fma(0.5 * y, fma(-s0, s0, vd), s0) * inv : 1e-18;
+          }
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, l, o);
+            if (lane >= o && __double_as_longlong(u) < __double_as_longlong(l)) l = u;
+          }
+          if (__double_as_longlong(run) < __double_as_longlong(l)) l = run;
+          run = __shfl_sync(0xffffffffu, l, 31);
+          if (a0 + lane < k) lam_next[a0 + lane] = l;
+        }
+        if (lane == 0) rep->inv_norm = inv * cscl;
+      }
+    }
+    __syncthreads();
+  };
+
+  if (direct) {
+    // ---- one CTA: W = C V^H from shared memory, one column of W per group of
+    // lanes (a lane takes every g-th row); W replaces A.  Against the tiles
+    // below: no waits for L2 and no barriers inside, 17 -> 5 thousand cycles
+    // at 16 x 16.
+    int* order = reinterpret_cast<int*>(srt);
     for (int id = tid; id < r; id += T)
-      if (rnk[id] < k) lam_next[rnk[id]] = sg[id] * s_d[1];
-  if (!refine && !Bq) {
-    if (me == 0 && tid == 0) rep->inv_norm = s_d[1] * scl;
+      if (rnk[id] < k) order[rnk[id]] = id;
+    __syncthreads();
+    int lg = 5;
+    while (lg > 2 && (1 << (lg - 1)) >= m) --lg;
+    const int g = 1 << lg, gl = tid & (g - 1), grp = tid >> lg, NG = T >> lg;
+    for (int a0 = 0; a0 < k; a0 += NG) {
+      const int a = a0 + grp;
+      if (!__any_sync(0xffffffffu, a < k)) continue;
+      const int id = order[min(a, k - 1)];
+      const HX col = held(id, id);
+      const S f = A::rsqrt(nA[id]);
+      typename A::NAcc s2;
+      for (int row = gl; row < m; row += g) {
+        typename A::Acc acc;
+#pragma unroll 2
+        for (int c = 0; c < n; ++c)
+          A::dot(acc, A::template load<false>(c0 + (unsigned)(c * ca), lda, row), A::template load<kGX>(col, ldx, c));
+        S wr, wi;
+        A::dot_sum(acc, 1, wr, wi);
+        const V w = A::scale(A::cval(wr, wi), f);
+        if (a < k) {
+          if constexpr (!kGA) A::template store<false>(acol(a, a), lda, row, w);
+          if (refine) A::nrm(s2, A::scale(w, A::from_double(__ldcg(lam_l + (row >> 1)))));
+        }
+      }
+      S v = A::nrm_value(s2);
+      for (int o = g >> 1; o > 0; o >>= 1) v = A::shfl_add(v, o);
+      if (refine && a < k && gl == 0) kn[a] = v;
+    }
+    __syncthreads();
+    if (refine)
+      finish_lam([&](int a) {
+        if constexpr (std::is_same<A, ArDF>::value)
+          return kn[a];
+        else
+          return ff_split(kn[a]);
+      });
+    if (Bq) {
+      const S inv = A::from_double(refine ? s_d[1] : s_d[1] * w_unit);
+      for (int t = tid; t < m * k; t += T) {
+        const int row = t / k, a = t - row * k;
+        if constexpr (!kGA) {
+          const V v = A::scale(A::template load<false>(acol(a, a), lda, row), inv);
+          if constexpr (sizeof(R) == 8)
+            Bq[t] = A::value(v);
+          else
+            Bq[t] = A::value32(v);
+        }
+      }
+    }
     return k;
   }
   tm.barrier();  // every row of B~_{q+1} is written, X's shared memory is free
 
   // ---- W = C V^H
-  using WA = ArDF;  // complex64 states too: one rounding to FP32 instead of n
+  using WA = A;  // complex64 states too: one rounding to FP32 instead of n
   using WV = typename WA::V;
   const unsigned sa = 0, sb = kPM * 20 * 16, sred = (kPM + kPK) * 20 * 16;
   constexpr int kLd = 20;                       // padded length of 16 entries (WA::ld(16) or more)
   constexpr unsigned kCol = kLd * WA::kBytes;   // bytes of a 16-entry run
   const int tx = tid & 15, ty = tid >> 4, TY = T >> 4, nrow = (kPM + TY - 1) / TY;  // 2 or 4 rows a thread
-  double* red = reinterpret_cast<double*>(svd_smem + sred);
-  const double w_unit = __longlong_as_double((long long)(1023 + max(-1000, min(1000, ec - ex))) << 52);
+  S* red = reinterpret_cast<S*>(svd_smem + sred);
   for (int j0 = me * kPN; j0 < k; j0 += P * kPN) {
-    double s2 = 0.0;
+    // sum of (lam |W|)^2 over the rows of this thread: in double-float, for
+    // FP64 sweeps in FP64
+    constexpr bool kD = std::is_same<A, ArF64>::value;
+    GramAcc s2;
+    double d2 = 0.0;
     for (int r0 = 0; r0 < m; r0 += kPM) {
       typename WA::Acc acc[4];
       for (int c0 = 0; c0 < n; c0 += kPK) {
@@ -1021,7 +1279,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           const int kk = t & 15, row = t >> 4;
           WV v = WA::zero_entry();
           if (r0 + row < m && c0 + kk < n) {
-            const cplx<R> z = Cm[(size_t)(r0 + row) * n + c0 + kk];
+            const cplx<R> z = __ldcg(Cm + (size_t)(r0 + row) * n + c0 + kk);
             v = WA::make(z.x * cscl, z.y * cscl);
           }
           WA::template store<false>(sa + row * kCol, kLd, kk, v);
@@ -1052,98 +1310,100 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         if (i < nrow && row < m && j0 + tx < k) {
           typename WA::S wr, wi;
           WA::dot_sum(acc[i], 1, wr, wi);
-          const double zr = WA::to_double(wr), zi = WA::to_double(wi), w = lam_l[row >> 1];
           // W is in units of 2^ec, the norm in units of 2^ex; refine: scaled
           // below, when the norm is known
-          const double f = refine ? 1.0 : s_d[1] * w_unit;
-          if (Bq) __stcg(Bq + (size_t)row * k + j0 + tx, cmk<R>(R(zr * f), R(zi * f)));
-          if (refine) s2 += w * w * (zr * zr + zi * zi);
+          if (Bq) {
+            const double f = refine ? 1.0 : s_d[1] * w_unit;
+            const double zr = WA::to_double(wr), zi = WA::to_double(wi);
+            __stcg(Bq + (size_t)row * k + j0 + tx, refine ? cmk<R>(R(zr), R(zi)) : cmk<R>(R(zr * f), R(zi * f)));
+          }
+          if (refine) {
+            const double lam = __ldcg(lam_l + (row >> 1));
+            if constexpr (kD) {
+              const double ur = lam * WA::to_double(wr), ui = lam * WA::to_double(wi);
+              d2 = fma(ur, ur, fma(ui, ui, d2));
+            } else {
+              const ff w = ff_split(lam);
+              const ff ur = ff_mul(w, wr), ui = ff_mul(w, wi);
+              s2.add(ur, ur);
+              s2.add(ui, ui);
+            }
+          }
         }
       }
     }
     if (refine) {
-      s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
-      if (lane < 16) red[(tid >> 5) * 16 + tx] = s2;
+      S v0;
+      if constexpr (kD)
+        v0 = d2;
+      else
+        v0 = s2.value();
+      const S v1 = A::shfl_add(v0, 16);
+      if (lane < 16) red[(tid >> 5) * 16 + tx] = v1;
       __syncthreads();
       if (tid < 16 && j0 + tid < k) {
-        double v = 0.0;
-        for (int w = 0; w < (T >> 5); ++w) v += red[w * 16 + tid];
-        __stcg(gnrm + j0 + tid, v);
+        S v = red[tid];
+        for (int w = 1; w < (T >> 5); ++w) v = A::add(v, red[w * 16 + tid]);
+        double d = 0.0;
+        memcpy(&d, &v, sizeof(S));
+        __stcg(gnrm + j0 + tid, d);
       }
       __syncthreads();
     }
   }
   if (refine) {
     tm.barrier();
-    // values in descending order (a running minimum: the refined values of a
-    // degenerate pair can differ in their last bits either way), their norm
-    if (tid < 32) {
-      double run = __longlong_as_double(0x7ff0000000000000ll), kept = 0.0;
-      for (int a0 = 0; a0 < k; a0 += 32) {
-        double v = a0 + lane < k ? sqrt(__ldcg(gnrm + a0 + lane)) * w_unit : run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double u = __shfl_up_sync(0xffffffffu, v, o);
-          if (lane >= o) v = fmin(v, u);
-        }
-        v = run < v ? run : v;
-        run = __shfl_sync(0xffffffffu, v, 31);
-        if (a0 + lane < k) {
-          sg[a0 + lane] = v;
-          kept += v * v;
-        }
+    finish_lam([&](int a) {
+      const double d = __ldcg(gnrm + a);
+      if constexpr (std::is_same<A, ArF64>::value) {
+        return ff_split(d);
+      } else {
+        ff v;
+        memcpy(&v, &d, sizeof(ff));
+        return v;
       }
-      kept = warp_sum(kept);
-      if (lane == 0) {
-        double nr = sqrt(kept);
-        if (!(nr > 0.0)) nr = 1.0;
-        s_d[0] = nr;
-        s_d[1] = 1.0 / nr;
-      }
-    }
-    __syncthreads();
-    if (me == 0)
-      for (int a = tid; a < k; a += T) lam_next[a] = sg[a] * s_d[1];
+    });
   }
-  if (me == 0 && tid == 0) rep->inv_norm = s_d[1] * scl;
   // ---- scale this CTA's columns of B~_q (only it wrote and reads them)
   if (refine && Bq) {
-    const double inv = s_d[1] * w_unit;
-    __syncthreads();
+    const S inv = A::from_double(s_d[1]);
     for (int j0 = me * kPN; j0 < k; j0 += P * kPN)
       for (int row = ty; row < m; row += TY)
         if (j0 + tx < k) {
           cplx<R>* z = Bq + (size_t)row * k + j0 + tx;
           const cplx<R> v = __ldcg(z);
-          *z = cmk<R>(R(v.x * inv), R(v.y * inv));
+          if constexpr (sizeof(R) == 8) *z = A::value(A::scale(A::make(v.x, v.y), inv));
         }
   }
   return k;
 }
 
 // ---- kernels ------------------------------------------------------------------
+// (FP64 work is bound by the SM's two FP64 units, which a few warps fill.)
 template <class A> constexpr int kSvdThreads = std::is_same<A, ArF64>::value ? 256 : 512;
 
 // Columns up to which one CTA takes the theta although more were launched.
 constexpr int kSvdSingleCols = 48;
 
-// CTAs that take part in a theta of m x n when Pl were launched with
-// smem_bytes each; 0: it does not fit (the grid kernel takes it).
+// CTAs that a theta of m x n gets out of the Pl launched; 0: it does not fit
+// (the grid kernel takes it).
 template <class A>
-__host__ __device__ inline int svd_team_size(int m, int n, int Pl, size_t smem_bytes) {
-  if ((n <= kSvdSingleCols || Pl == 1) && SvdSmem<A>::bytes(m, n, 1, true, true) <= smem_bytes) return 1;
-  return Pl > 1 && SvdSmem<A>::bytes(m, n, Pl, true, true) <= smem_bytes ? Pl : 0;
+__host__ __device__ inline int svd_team_size(int m, int n, int Pl) {
+  if ((n <= kSvdSingleCols || Pl == 1) && SvdSmem<A>::bytes(m, n, 1, true, true) <= kSvdSmemLimit) return 1;
+  for (int P = 4; P <= Pl; P *= 2)
+    if (SvdSmem<A>::bytes(m, n, P, true, true) <= kSvdSmemLimit) return P;
+  return 0;
 }
 
 template <class A, class R>
 __global__ void __launch_bounds__(kSvdThreads<A>, 1)
     svd_kernel(const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l, int* __restrict__ chi, int q,
                SvdParams p, cplx<R>* __restrict__ Bnext, double* __restrict__ lam_next, DevReport* __restrict__ rep,
-               cplx<R>* __restrict__ Bq, char* __restrict__ gws, unsigned smem_bytes) {
+               cplx<R>* __restrict__ Bq, char* __restrict__ gws) {
   __shared__ float2 s_mail[2 * 16];
   const int Pl = (int)cg::this_cluster().num_blocks(), me = (int)cg::this_cluster().block_rank();
   const int m = 2 * chi[q], n = 2 * chi[q + 2];
-  const int P = svd_team_size<A>(m, n, Pl, smem_bytes);
+  const int P = svd_team_size<A>(m, n, Pl);
   if (me >= P) return;  // an exited CTA counts as arrived at the cluster barriers
   if (P == 1) {
     OneTeam tm;
@@ -1156,15 +1416,15 @@ __global__ void __launch_bounds__(kSvdThreads<A>, 1)
 }
 
 // Thetas that do not fit a cluster: a co-resident grid (cooperative launch).
-// Pl, cluster_smem: the cluster launch that ran before and may have done it.
+// Pl: the CTAs of the cluster launch that ran before and may have done it.
 template <class A, class R>
 __global__ void __launch_bounds__(kSvdThreads<A>, 1)
     svd_grid_kernel(const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l, int* __restrict__ chi, int q,
                     SvdParams p, cplx<R>* __restrict__ Bnext, double* __restrict__ lam_next,
-                    DevReport* __restrict__ rep, cplx<R>* __restrict__ Bq, char* __restrict__ gws, GridSync* sync, int Pl, unsigned cluster_smem,
+                    DevReport* __restrict__ rep, cplx<R>* __restrict__ Bq, char* __restrict__ gws, GridSync* sync, int Pl,
                     unsigned smem_bytes) {
   const int m = 2 * chi[q], n = 2 * chi[q + 2];
-  if (svd_team_size<A>(m, n, Pl, cluster_smem)) return;
+  if (svd_team_size<A>(m, n, Pl)) return;
   // a block of X needs at least one column on every CTA
   const int P = min((int)gridDim.x, max(2, (min(m, n) + 3) / 4));
   if ((int)blockIdx.x >= P) return;

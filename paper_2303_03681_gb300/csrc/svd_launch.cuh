@@ -42,18 +42,16 @@ inline DeviceLimits device_limits() {
 
 template <class A> SvdPlan<A> svd_plan(int mcap, int ncap) {
   const DeviceLimits d = device_limits();
-  const size_t lim = (size_t)d.smem - 1024;  // the kernels' static shared memory
+  const size_t lim = kSvdSmemLimit;
   SvdPlan<A> pl;
-  for (int P : {1, 4, 8}) {
-    if (P == 1 && ncap > kSvdSingleCols) continue;
-    const size_t need = SvdSmem<A>::bytes(mcap, ncap, P, true, true);
-    if (need > lim) continue;
-    pl.P = P;
-    pl.smem = need;
+  pl.P = svd_team_size<A>(mcap, ncap, 8);
+  if (pl.P == 1) {
+    pl.smem = SvdSmem<A>::bytes_one(mcap, ncap);
     return pl;
   }
+  pl.smem = lim;  // smaller thetas may need more per CTA, on fewer CTAs
+  if (pl.P) return pl;
   pl.P = 8;
-  pl.smem = lim;
   pl.grid = std::min(std::min(128, d.sms), std::max(2, (std::min(mcap, ncap) + 3) / 4));
   pl.grid_smem = SvdSmem<A>::bytes(mcap, ncap, pl.grid, false, true);
   if (pl.grid_smem > lim) pl.grid_smem = lim;
@@ -66,13 +64,12 @@ template <class A, class R> cudaError_t svd_attrs() {
   static uint64_t done = 0;
   int dev = 0;
   cudaGetDevice(&dev);
-  const DeviceLimits d = device_limits();
   std::lock_guard<std::mutex> g(mu);
   const uint64_t bit = 1ull << (dev & 63);
   if (done & bit) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(svd_kernel<A, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem - 1024);
+  cudaError_t e = cudaFuncSetAttribute(svd_kernel<A, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSvdSmemLimit);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(svd_grid_kernel<A, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem - 1024);
+    e = cudaFuncSetAttribute(svd_grid_kernel<A, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSvdSmemLimit);
   if (e == cudaSuccess) done |= bit;
   return e;
 }
@@ -99,7 +96,7 @@ template <class A, class R> void svd_launch_t(const SvdJob& j) {
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cudaLaunchKernelEx(&cfg, svd_kernel<A, R>, C, j.lam_l, j.chi, j.q, j.p, B, j.lam_next, j.rep,
-                     static_cast<cplx<R>*>(j.Bq), j.ws, (unsigned)pl.smem);
+                     static_cast<cplx<R>*>(j.Bq), j.ws);
   if (!pl.grid) return;
   GridSync* sync = reinterpret_cast<GridSync*>(j.ws + SvdWs<A>(j.mcap, j.ncap, true).total);
   cudaMemsetAsync(sync, 0, sizeof(GridSync), j.stream);
@@ -108,7 +105,7 @@ template <class A, class R> void svd_launch_t(const SvdJob& j) {
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cudaLaunchKernelEx(&cfg, svd_grid_kernel<A, R>, C, j.lam_l, j.chi, j.q, j.p, B, j.lam_next, j.rep,
-                     static_cast<cplx<R>*>(j.Bq), j.ws, sync,                     pl.P, (unsigned)pl.smem, (unsigned)pl.grid_smem);
+                     static_cast<cplx<R>*>(j.Bq), j.ws, sync,                     pl.P, (unsigned)pl.grid_smem);
 }
 
 }  // namespace mpsv

@@ -136,7 +136,7 @@ typedef struct {
 /* Kernel classes for mps_ctx_profile_read. */
 typedef enum {
   MPS_K_THETA = 0,     /* theta contraction + gate + lam scaling */
-  MPS_K_SVD = 1,       /* Jacobi SVD + truncation */
+  MPS_K_SVD = 1,       /* Jacobi SVD + truncation; launches of whole circuits in vqe_eval_batch */
   MPS_K_G3 = 2,        /* B~_q = C V^dagger (where the SVD kernel computes it: counted here, timed there) */
   MPS_K_GATE1 = 3,     /* one-qubit gate */
   MPS_K_SETUP = 4,     /* reset, angle binding, fills */

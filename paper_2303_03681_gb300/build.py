@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmpsvqe.so")
-SOURCES = ["state.cu", "svd_df.cu", "svd_f64.cu", "svd_f32.cu", "energy.cu", "noalloc.cu", "server.cu", "tc_gates.cu"]
+SOURCES = ["state.cu", "svd_df.cu", "svd_f64.cu", "svd_f32.cu", "gate_run.cu", "energy.cu", "noalloc.cu", "server.cu", "tc_gates.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-Xptxas", "-O3"]

@@ -589,6 +589,46 @@ static mps_status run_batch(const vqe_request* reqs, size_t n, double* energies_
       groups[gi].push_back(i);
     }
   }
+  // Past the 8 hardware queues that a process gets by default, streams share a
+  // queue, and a stream whose next launch waits for its last one holds up the
+  // others behind it: 16 UCCSD evaluations of 16 qubits, gate by gate, took
+  // 181 ms against 97 ms for 8 (with 32 queues 110 ms).  From there on a
+  // circuit goes out as a run of gates, a few launches each, which this thread
+  // issues tier by tier over all requests, so that no request's later launches
+  // stand before another's first: 113 ms, and 136 against 282 ms for 32.  Up
+  // to 8 streams the separate launches are the faster form (79 against 85 ms
+  // for one): more CTAs contract a theta, and the SVD keeps more registers.
+  constexpr size_t kQueues = 8;
+  std::vector<char> whole(n, 0);
+  if (groups.size() > kQueues) {
+    std::vector<std::vector<size_t>> rest(groups.size());
+    for (size_t gi = 0; gi < groups.size(); ++gi)
+      for (size_t i : groups[gi]) {
+        const vqe_request& r = reqs[i];
+        whole[i] = state_runs(r.state, r.circuit->q.data(), r.circuit->arity.data(), r.circuit->n_gates);
+        if (!whole[i]) {
+          rest[gi].push_back(i);
+          continue;
+        }
+        DeviceGuard guard(r.state->ctx->device);
+        rc[i] = state_reset(r.state, r.init_bits);
+        if (rc[i] == MPS_OK) rc[i] = state_bind_circuit(r.state, r.circuit, r.theta, on_device ? 1 : 0);
+      }
+    for (int tier = 0; tier < kRunTiers; ++tier)
+      for (size_t gi = 0; gi < groups.size(); ++gi)
+        for (size_t i : groups[gi]) {
+          if (!whole[i] || rc[i] != MPS_OK) continue;
+          const vqe_request& r = reqs[i];
+          DeviceGuard guard(r.state->ctx->device);
+          rc[i] = state_run_tier(r.state, r.state->d_bound, r.circuit->q.data(), r.circuit->arity.data(),
+                                 r.circuit->n_gates, tier);
+          if (rc[i] != MPS_OK) r.state->broken = true;
+        }
+    std::vector<std::vector<size_t>> left;
+    for (auto& g : rest)
+      if (!g.empty()) left.push_back(std::move(g));
+    groups = std::move(left);
+  }
   const size_t hw = std::max(1u, std::thread::hardware_concurrency());
   const size_t n_threads = std::min<size_t>({groups.size(), std::max<size_t>(1, hw / 2), 16});
   std::vector<std::string> errs(n_threads);
@@ -604,11 +644,11 @@ static mps_status run_batch(const vqe_request* reqs, size_t n, double* energies_
     }
     int max_gates = 0;
     for (size_t i : mine)
-      if (rc[i] == MPS_OK) max_gates = std::max(max_gates, reqs[i].circuit->n_gates);
+      if (rc[i] == MPS_OK && !whole[i]) max_gates = std::max(max_gates, reqs[i].circuit->n_gates);
     for (int g = 0; g < max_gates; ++g) {
       for (size_t i : mine) {
         const vqe_request& r = reqs[i];
-        if (rc[i] != MPS_OK || g >= r.circuit->n_gates) continue;
+        if (rc[i] != MPS_OK || whole[i] || g >= r.circuit->n_gates) continue;
         DeviceGuard guard(r.state->ctx->device);
         rc[i] = state_apply_device_gates(r.state, r.state->d_bound + g, &r.circuit->q[g], &r.circuit->arity[g], 1);
         if (rc[i] != MPS_OK) r.state->broken = true;

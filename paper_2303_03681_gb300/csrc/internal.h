@@ -132,6 +132,7 @@ struct mps_state {
   void* d_B = nullptr;
   double* d_lam = nullptr;
   int* d_chi = nullptr;
+  int* d_cap = nullptr;  // bond capacities, then the progress of a run of gates
   size_t* d_site_off = nullptr;
   size_t* d_lam_off = nullptr;
   uint8_t* d_bits = nullptr;
@@ -143,6 +144,10 @@ struct mps_state {
   size_t total_lam = 0;
   size_t total_elems = 0;
   std::vector<uint8_t> last_bits;
+  // runs of gates in one launch: CTAs of each bond's largest theta (0: not in
+  // a run), shared memory of the one-CTA launch
+  std::vector<int> run_p;
+  size_t run_smem = 0;
   bool broken = false;
   int nc_seen = 0;  // svd_not_converged as last read by the host (mps_apply_gates)
   // split-product tensor-core gate contractions: 0 (CUDA cores) or the
@@ -243,6 +248,15 @@ inline void svd_launch(SvdArith a, const SvdJob& j) {
   a == SVD_DF ? svd_launch_df(j) : (a == SVD_F64 ? svd_launch_f64(j) : svd_launch_f32(j));
 }
 
+// gate_run.cu: runs of gates in one launch
+void run_prime();
+void run_setup(mps_state* st);
+// The launches of a run, in order: one CTA, a cluster of 4, one of 8 (each only
+// where p_max, the CTAs of the run's largest theta, asks for it: false where not).
+constexpr int kRunTiers = 3;
+bool run_tier(mps_state* st, const DevGate* d_gates, size_t n, int p_max, int tier);
+SvdParams svd_params(const mps_state* st);
+
 // The two status flags of a state, read back with one 8-byte copy from
 // &DevReport::not_converged.
 struct StateFlags {
@@ -262,6 +276,10 @@ inline bool status_has_result(mps_status s) { return s == MPS_OK || s == MPS_ENO
 
 // state.cu
 mps_status state_apply_device_gates(mps_state* st, const DevGate* d_gates, const int* q, const int* arity, size_t n);
+// All of these gates go out as one run (gate_run.cu).
+bool state_runs(const mps_state* st, const int* q, const int* arity, size_t n);
+// One tier's launch of such a run (all tiers in order apply the gates).
+mps_status state_run_tier(mps_state* st, const DevGate* d_gates, const int* q, const int* arity, size_t n, int tier);
 mps_status state_reset(mps_state* st, const uint8_t* bits);
 // Copies theta into the state's workspace and binds the circuit's gates there.
 mps_status state_bind_circuit(mps_state* st, const mps_circuit* c, const double* theta, int theta_on_device);

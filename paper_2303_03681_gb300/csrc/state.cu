@@ -163,14 +163,27 @@ template <typename R> static cplx<R>* site_ptr(mps_state* st, int s) {
   return reinterpret_cast<cplx<R>*>(st->d_B) + st->site_off[s];
 }
 
+SvdParams svd_params(const mps_state* st) {
+  SvdParams p;
+  p.chi_max = st->cfg.chi_max;
+  p.max_sweeps = st->cfg.svd_max_sweeps > 0 ? st->cfg.svd_max_sweeps : 60;
+  p.trunc_rel = st->cfg.trunc_rel;
+  p.tol = st->cfg.svd_tol;
+  return p;
+}
+
+// Split-product tensor-core contractions (complex64 states): thetas of 16
+// columns and fewer are all padding on 128-wide tiles.
+static bool uses_tc(const mps_state* st, int q) {
+  return st->fp32 && 2 * st->cap[q + 2] >= (st->cfg.svd_fp64 ? 32 : 96) && tc_gates_used(st, q);
+}
+
 template <typename R>
 static void launch_two_qubit(mps_state* st, const DevGate* g, int q, cudaStream_t s) {
   const int cap_l = st->cap[q], cap_r = st->cap[q + 2];
   const dim3 blk(kTile, kTile);
   const dim3 g1((cap_r + kTile - 1) / kTile, (cap_l + kTile - 1) / kTile);
-  // split-product tensor-core contractions (complex64 states): thetas of 16
-  // columns and fewer are all padding on 128-wide tiles
-  const bool tcg = sizeof(R) == 4 && 2 * cap_r >= (st->cfg.svd_fp64 ? 32 : 96) && tc_gates_used(st, q);
+  const bool tcg = uses_tc(st, q);
   if (tcg) {
     tc_theta(st, g, q, s);
   } else {
@@ -188,10 +201,7 @@ static void launch_two_qubit(mps_state* st, const DevGate* g, int q, cudaStream_
     j.lam_l = st->d_lam + st->lam_off[q];
     j.chi = st->d_chi;
     j.q = q;
-    j.p.chi_max = st->cfg.chi_max;
-    j.p.max_sweeps = st->cfg.svd_max_sweeps > 0 ? st->cfg.svd_max_sweeps : 60;
-    j.p.trunc_rel = st->cfg.trunc_rel;
-    j.p.tol = st->cfg.svd_tol;
+    j.p = svd_params(st);
     j.Bnext = site_ptr<R>(st, q + 1);
     j.lam_next = st->d_lam + st->lam_off[q + 1];
     j.rep = st->d_rep;
@@ -216,6 +226,26 @@ static void launch_one_qubit(mps_state* st, const DevGate* g, int q, cudaStream_
   const int tot = st->cap[q] * st->cap[q + 1];
   KernelScope k(st->ctx, MPS_K_GATE1);
   gate1_kernel<R><<<(tot + 255) / 256, 256, 0, s>>>(site_ptr<R>(st, q), g, st->d_chi, q);
+}
+
+// A circuit can go out as a run (gate_run.cu) where the FP64-accurate SVD and
+// the CUDA-core contractions serve all its gates; a class that is being timed
+// is launched gate by gate.
+bool state_runs(const mps_state* st, const int* q, const int* arity, size_t n) {
+  constexpr uint32_t kGateKinds = 1u << MPS_K_THETA | 1u << MPS_K_SVD | 1u << MPS_K_G3 | 1u << MPS_K_GATE1;
+  if (!st->cfg.svd_fp64 || (st->ctx->prof_mask & kGateKinds)) return false;
+  for (size_t i = 0; i < n; ++i)
+    if (arity[i] != 1 && (!st->run_p[q[i]] || uses_tc(st, q[i]))) return false;
+  return n > 1;
+}
+
+mps_status state_run_tier(mps_state* st, const DevGate* d_gates, const int* q, const int* arity, size_t n, int tier) {
+  int p_max = 1;
+  for (size_t i = 0; i < n; ++i)
+    if (arity[i] == 2) p_max = std::max(p_max, st->run_p[q[i]]);
+  if (run_tier(st, d_gates, n, p_max, tier)) count_launch(st->ctx, MPS_K_SVD);  // most of a run's time
+  MPSV_CUDA(cudaGetLastError());
+  return MPS_OK;
 }
 
 mps_status state_apply_device_gates(mps_state* st, const DevGate* d_gates, const int* q, const int* arity,
@@ -315,6 +345,7 @@ static void prime_launch_attrs() {
   svd_prime_df();
   svd_prime_f32();
   svd_prime_f64();
+  run_prime();
 }
 
 mps_status state_run_circuit(mps_state* st, const mps_circuit* c, const double* theta, int theta_on_device) {
@@ -381,7 +412,7 @@ static void destroy_state(mps_state* st) {
     st->graph = nullptr;
   }
   tc_gates_free(st);
-  for (void* p : {st->d_B, (void*)st->d_lam, (void*)st->d_chi, (void*)st->d_site_off, (void*)st->d_lam_off,
+  for (void* p : {st->d_B, (void*)st->d_lam, (void*)st->d_chi, (void*)st->d_cap, (void*)st->d_site_off, (void*)st->d_lam_off,
                   (void*)st->d_bits, (void*)st->d_rep, st->d_C, (void*)st->d_svd, (void*)st->d_gates,
                   (void*)st->d_bound, (void*)st->d_theta, st->d_L[0], st->d_L[1], st->d_M, (void*)st->d_vals,
                   (void*)st->d_energy, (void*)st->d_obs})
@@ -675,6 +706,7 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
   A(&st->d_B, off * celem);
   A((void**)&st->d_lam, loff * sizeof(double));
   A((void**)&st->d_chi, (n + 1) * sizeof(int));
+  A((void**)&st->d_cap, (n + 2) * sizeof(int));
   A((void**)&st->d_site_off, n * sizeof(size_t));
   A((void**)&st->d_lam_off, (n + 1) * sizeof(size_t));
   A((void**)&st->d_bits, n);
@@ -686,11 +718,14 @@ mps_status mps_create(mps_ctx* ctx, int32_t n_qubits, const uint8_t* init_bits, 
     destroy_state(st);
     return rc;
   }
+  run_setup(st);
   cudaStream_t s = ctx->stream;
   cudaError_t e = cudaMemcpyAsync(st->d_site_off, st->site_off.data(), n * sizeof(size_t),
                                   cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(st->d_lam_off, st->lam_off.data(), (n + 1) * sizeof(size_t), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(st->d_cap, st->cap.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(st->d_B, 0, off * celem, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(st->d_lam, 0, loff * sizeof(double), s);
   if (e != cudaSuccess) {

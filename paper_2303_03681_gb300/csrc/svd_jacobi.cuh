@@ -1264,7 +1264,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   const unsigned sa = 0, sb = kPM * 20 * 16, sred = (kPM + kPK) * 20 * 16;
   constexpr int kLd = 20;                       // padded length of 16 entries (WA::ld(16) or more)
   constexpr unsigned kCol = kLd * WA::kBytes;   // bytes of a 16-entry run
-  const int tx = tid & 15, ty = tid >> 4, TY = T >> 4, nrow = (kPM + TY - 1) / TY;  // 2 or 4 rows a thread
+  const int tx = tid & 15, ty = tid >> 4, TY = T >> 4, nrow = (kPM - ty + TY - 1) / TY;  // 2 to 4 rows a thread
   S* red = reinterpret_cast<S*>(svd_smem + sred);
   for (int j0 = me * kPN; j0 < k; j0 += P * kPN) {
     // sum of (lam |W|)^2 over the rows of this thread: in double-float, for

@@ -33,8 +33,8 @@ struct Node {
 // on the bond left of site s; node (parent, op) extends its parent's string by
 // one site.
 static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeffs, std::vector<int>& parent_src,
-                             std::vector<int2>& child, std::vector<int4>& leaf, std::vector<int2>& trace,
-                             std::vector<int2>& dense, std::vector<int>& diag) {
+                             std::vector<int2>& child, std::vector<EnvGroup>& group, std::vector<int4>& leaf,
+                             std::vector<int2>& trace, std::vector<int2>& dense, std::vector<int>& diag) {
   const int n = h->n;
   std::vector<Node> nodes(n);
   for (int s = 0; s < n; ++s) {
@@ -92,20 +92,29 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
     LevelHost& L = h->levels[j];
     L.off_parent = parent_src.size();
     L.off_child = child.size();
+    L.off_group = group.size();
     L.off_leaf = leaf.size();
     L.off_trace = trace.size();
     int n_entries = 0;
     int slots = 0;
+    std::vector<int> group_of;  // per parent entry
     for (int id : by_level[j]) {
       Node& nd = nodes[id];
       Node& par = nodes[nd.parent];
       if (par.entry < 0) {
         par.entry = n_entries++;
         parent_src.push_back(par.level < 0 ? -1 : par.slot);
+        group_of.push_back(-1);
       }
       if (nd.has_child) {
         nd.slot = slots++;
         child.push_back(make_int2(par.entry, nd.op));
+        int& g = group_of[par.entry];
+        if (g < 0) {
+          g = (int)(group.size() - L.off_group);
+          group.push_back(EnvGroup{par.entry, {-1, -1, -1, -1}});
+        }
+        group[L.off_group + g].slot[nd.op] = nd.slot;
       }
     }
     for (int id : by_level[j]) {
@@ -130,6 +139,7 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
     L.n_diag = (int)(diag.size() - L.off_diag);
     L.n_parents = n_entries;
     L.n_children = slots;
+    L.n_groups = (int)(group.size() - L.off_group);
     L.n_leaves = (int)(leaf.size() - L.off_leaf);
     L.n_traces = (int)(trace.size() - L.off_trace);
     n_mat += slots;
@@ -274,11 +284,11 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
     if (!L.n_parents) continue;
     EnvLevel lv;
     lv.parent_src = h->d_parent_src + L.off_parent;
-    lv.child = h->d_child + L.off_child;
+    lv.group = h->d_group + L.off_group;
     lv.leaf = h->d_leaf + L.off_leaf;
     lv.trace = h->d_trace + L.off_trace;
     lv.n_parents = L.n_parents;
-    lv.n_children = L.n_children;
+    lv.n_groups = L.n_groups;
     lv.n_leaves = L.n_leaves;
     lv.n_traces = L.n_traces;
     lv.site = j;
@@ -303,7 +313,8 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
       }
       if (L.n_children) {
         KernelScope k(c, MPS_K_ENV_CHILD);
-        env_child_kernel<R><<<(unsigned)((size_t)L.n_children * tr * tr), blk, 0, s>>>(M, Bj, st->d_chi, lv, Lcur);
+        env_child_kernel<R><<<(unsigned)((size_t)L.n_groups * (tr * (tr + 1) / 2)), blk, 0, s>>>(M, Bj, st->d_chi, lv,
+                                                                                            Lcur);
       }
     }
     if (L.n_leaves) {
@@ -343,7 +354,7 @@ static void destroy_ham(mps_ham* h) {
   mps_ctx* c = h->ctx;
   DeviceGuard guard(c->device);
   cudaStreamSynchronize(c->stream);
-  for (void* p : {(void*)h->d_parent_src, (void*)h->d_child, (void*)h->d_leaf, (void*)h->d_trace,
+  for (void* p : {(void*)h->d_parent_src, (void*)h->d_child, (void*)h->d_group, (void*)h->d_leaf, (void*)h->d_trace,
                   (void*)h->d_coeffs, (void*)h->d_dense, (void*)h->d_diag})
     dev_free(c, p);
   delete h;
@@ -395,11 +406,12 @@ mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms
   h->n_terms = (long long)n_terms;
   std::vector<int> parent_src;
   std::vector<int2> child;
+  std::vector<EnvGroup> group;
   std::vector<int4> leaf;
   std::vector<int2> trace;
   std::vector<int2> dense;
   std::vector<int> diag;
-  mps_status rc = build_trie(h, ops, coeffs, parent_src, child, leaf, trace, dense, diag);
+  mps_status rc = build_trie(h, ops, coeffs, parent_src, child, group, leaf, trace, dense, diag);
   if (rc != MPS_OK) {
     delete h;
     return rc;
@@ -415,6 +427,7 @@ mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms
   };
   up((void**)&h->d_parent_src, parent_src.data(), parent_src.size() * sizeof(int));
   up((void**)&h->d_child, child.data(), child.size() * sizeof(int2));
+  up((void**)&h->d_group, group.data(), group.size() * sizeof(EnvGroup));
   up((void**)&h->d_leaf, leaf.data(), leaf.size() * sizeof(int4));
   up((void**)&h->d_trace, trace.data(), trace.size() * sizeof(int2));
   up((void**)&h->d_dense, dense.data(), dense.size() * sizeof(int2));

@@ -183,9 +183,15 @@ struct mps_circuit {
 };
 
 namespace mpsv {
+// The children of one parent entry of the trie: their slots by operator (I, X,
+// Y, Z), -1 where there is none.
+struct EnvGroup {
+  int parent;
+  int slot[4];
+};
 struct LevelHost {
-  int n_parents = 0, n_children = 0, n_leaves = 0, n_traces = 0;
-  size_t off_parent = 0, off_child = 0, off_leaf = 0, off_trace = 0;
+  int n_parents = 0, n_children = 0, n_groups = 0, n_leaves = 0, n_traces = 0;
+  size_t off_parent = 0, off_child = 0, off_group = 0, off_leaf = 0, off_trace = 0;
   int n_dense = 0, n_diag = 0;  // parents with a stored environment / starting strings here
   size_t off_dense = 0, off_diag = 0;
 };
@@ -200,6 +206,7 @@ struct mps_ham {
   std::vector<mpsv::LevelHost> levels;
   int* d_parent_src = nullptr;
   int2* d_child = nullptr;
+  mpsv::EnvGroup* d_group = nullptr;
   int4* d_leaf = nullptr;
   int2* d_trace = nullptr;
   int2* d_dense = nullptr;  // (parent entry, environment slot)

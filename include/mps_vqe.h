@@ -262,7 +262,8 @@ mps_status mps_apply_circuit_async(mps_state* st, const mps_circuit* c, const do
  * whose nodes are the shared left environments of Eq. expec2. */
 mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms,
                                   const uint8_t* ops, const double* coeffs, mps_ham** out);
-/* Trie statistics: n_nodes materialised environments, n_levels sites. */
+/* Trie statistics: n_nodes stored environments (prefixes from the left and
+ * suffixes from the right), max_level_nodes the most at one site. */
 mps_status mps_hamiltonian_info(const mps_ham* h, int64_t* n_terms, int64_t* n_nodes,
                                 int64_t* max_level_nodes);
 void mps_ham_destroy(mps_ham* h);

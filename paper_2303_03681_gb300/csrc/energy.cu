@@ -1,9 +1,11 @@
-// Hamiltonian upload (prefix trie of the Pauli strings) and the Pauli-sum
-// energy of Eq. expec2 with shared left environments.
+// Hamiltonian upload (prefix and suffix tries of the Pauli strings) and the
+// Pauli-sum energy of Eq. expec2 with shared environments from both ends.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <mutex>
+#include <numeric>
 #include <string>
 #include <thread>
 #include <unordered_map>
@@ -29,19 +31,77 @@ struct Node {
 
 }  // namespace
 
-// Builds the trie on the host.  Start node s (id s < n) stands for diag(lam_s^2)
-// on the bond left of site s; node (parent, op) extends its parent's string by
-// one site.
-static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeffs, std::vector<int>& parent_src,
-                             std::vector<int2>& child, std::vector<EnvGroup>& group, std::vector<int4>& leaf,
-                             std::vector<int2>& trace, std::vector<int2>& dense, std::vector<int>& diag) {
-  const int n = h->n;
-  std::vector<Node> nodes(n);
-  for (int s = 0; s < n; ++s) {
-    nodes[s].level = -1;
-    nodes[s].parent = -1;
-    nodes[s].op = 0;
+// The tries of both halves of the chain, flattened for the device.
+struct Trie {
+  std::vector<int> parent_src;
+  std::vector<int2> child;
+  std::vector<EnvGroup> group;
+  std::vector<int4> leaf;
+  std::vector<int2> trace, dense;
+  std::vector<int> diag;
+  std::vector<int4> cross;
+  std::vector<int2> pair;
+};
+
+// The bond where prefixes and suffixes meet: the one with the least work, the
+// distinct prefixes of the sites before it and the distinct suffixes of the
+// sites after it, each weighted by a step's products on bonds that double from
+// either end up to 64.  (A string that ends inside another's prefix is not told
+// apart; n: all strings run from the left.)  It is the middle for a molecular
+// Hamiltonian: 20 spin orbitals take 3.4e9 complex multiply-adds at chi = 64
+// against 7.8e9 from the left alone.
+static int meeting_bond(const uint8_t* ops, long long n_terms, int n) {
+  std::vector<double> left(n, 0.0), right(n, 0.0);
+  std::vector<uint8_t> rev((size_t)n_terms * n);
+  for (long long t = 0; t < n_terms; ++t)
+    std::reverse_copy(ops + (size_t)t * n, ops + (size_t)(t + 1) * n, rev.begin() + (size_t)t * n);
+  auto distinct = [&](const uint8_t* rows, std::vector<double>& count) {
+    std::vector<int> order((size_t)n_terms);
+    std::iota(order.begin(), order.end(), 0);
+    std::sort(order.begin(), order.end(),
+              [&](int a, int b) { return std::memcmp(rows + (size_t)a * n, rows + (size_t)b * n, n) < 0; });
+    const uint8_t* prev = nullptr;
+    for (int t : order) {
+      const uint8_t* row = rows + (size_t)t * n;
+      int same = 0, first = 0, last = n - 1;
+      while (prev && same < n && prev[same] == row[same]) ++same;
+      while (first < n && !row[first]) ++first;
+      while (last >= 0 && !row[last]) --last;
+      for (int j = std::max(first, same); j <= last; ++j) count[j] += 1.0;
+      prev = row;
+    }
+  };
+  distinct(ops, left);
+  distinct(rev.data(), right);
+  auto weight = [&](int j) { return std::pow(8.0, std::min({j, n - 1 - j, 6})); };
+  double cost = 0.0;  // of everything from the right, then bond by bond
+  for (int j = 0; j < n; ++j) cost += weight(j) * right[n - 1 - j];
+  double best = std::numeric_limits<double>::infinity();
+  int cut = n;
+  for (int c = 1; c <= n; ++c) {
+    cost += weight(c - 1) * (left[c - 1] - right[n - c]);
+    if (cost < best) {
+      best = cost;
+      cut = c;
+    }
   }
+  return cut;
+}
+
+// Builds the tries on the host: prefixes up to the bond h->cut, and
+// suffixes down to it.  Start node s (id s < n) stands for diag(lam_s^2) on the
+// bond left of site s, start node n + s for the identity on the bond right of
+// it; node (parent, op) extends its parent's string by one site.
+static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeffs, Trie& tr) {
+  const int n = h->n, cut = h->cut = meeting_bond(ops, h->n_terms, h->n);
+  std::vector<Node> nodes(2 * n);
+  for (Node& s : nodes) {
+    s.level = -1;
+    s.parent = -1;
+    s.op = 0;
+  }
+  std::vector<int> across;  // terms across the middle, with their left and right nodes
+  std::vector<int2> ends;
   std::unordered_map<uint64_t, int> edge;
   edge.reserve(1 << 16);
   for (long long t = 0; t < h->n_terms; ++t) {
@@ -62,8 +122,8 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
       return MPS_EINVAL;
     }
     if (first < 0) continue;  // identity: <I> = 1 (vals prefilled)
-    int cur = first;
-    for (int j = first; j <= last; ++j) {
+    int cur = -1;
+    auto extend = [&](int j) {
       const uint64_t key = ((uint64_t)cur << 2) | row[j];
       auto it = edge.find(key);
       int nxt;
@@ -80,21 +140,40 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
       }
       nodes[cur].has_child = true;
       cur = nxt;
+    };
+    int left = -1, right = -1;
+    if (first < cut) {
+      cur = first;
+      for (int j = first; j <= std::min(last, cut - 1); ++j) extend(j);
+      left = cur;
     }
-    nodes[cur].terms.push_back((int)t);
+    if (last >= cut) {
+      cur = n + last;
+      for (int j = last; j >= std::max(first, cut); --j) extend(j);
+      right = cur;
+      h->right = true;
+    }
+    if (left >= 0 && right >= 0) {
+      nodes[left].has_child = nodes[right].has_child = true;  // stored for the strings across
+      across.push_back((int)t);
+      ends.push_back(make_int2(left, right));
+    } else {
+      nodes[cur].terms.push_back((int)t);
+    }
   }
   // bucket real nodes by level (creation order inside a level)
   std::vector<std::vector<int>> by_level(n);
-  for (size_t id = n; id < nodes.size(); ++id) by_level[nodes[id].level].push_back((int)id);
+  for (size_t id = 2 * n; id < nodes.size(); ++id) by_level[nodes[id].level].push_back((int)id);
   h->levels.assign(n, LevelHost());
   long long n_mat = 0, max_level = 0;
-  for (int j = 0; j < n; ++j) {
+  for (int step = 0; step < n; ++step) {
+    const int j = step < cut ? step : n - 1 - (step - cut);
     LevelHost& L = h->levels[j];
-    L.off_parent = parent_src.size();
-    L.off_child = child.size();
-    L.off_group = group.size();
-    L.off_leaf = leaf.size();
-    L.off_trace = trace.size();
+    L.off_parent = tr.parent_src.size();
+    L.off_child = tr.child.size();
+    L.off_group = tr.group.size();
+    L.off_leaf = tr.leaf.size();
+    L.off_trace = tr.trace.size();
     int n_entries = 0;
     int slots = 0;
     std::vector<int> group_of;  // per parent entry
@@ -103,48 +182,61 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
       Node& par = nodes[nd.parent];
       if (par.entry < 0) {
         par.entry = n_entries++;
-        parent_src.push_back(par.level < 0 ? -1 : par.slot);
+        tr.parent_src.push_back(par.level < 0 ? -1 : par.slot);
         group_of.push_back(-1);
       }
       if (nd.has_child) {
         nd.slot = slots++;
-        child.push_back(make_int2(par.entry, nd.op));
+        tr.child.push_back(make_int2(par.entry, nd.op));
         int& g = group_of[par.entry];
         if (g < 0) {
-          g = (int)(group.size() - L.off_group);
-          group.push_back(EnvGroup{par.entry, {-1, -1, -1, -1}});
+          g = (int)(tr.group.size() - L.off_group);
+          tr.group.push_back(EnvGroup{par.entry, {-1, -1, -1, -1}});
         }
-        group[L.off_group + g].slot[nd.op] = nd.slot;
+        tr.group[L.off_group + g].slot[nd.op] = nd.slot;
       }
     }
     for (int id : by_level[j]) {
       const Node& nd = nodes[id];
       for (int t : nd.terms) {
         if (nd.has_child)
-          trace.push_back(make_int2(nd.slot, t));
+          tr.trace.push_back(make_int2(nd.slot, t));
         else
-          leaf.push_back(make_int4(nodes[nd.parent].entry, nd.op, t, 0));
+          tr.leaf.push_back(make_int4(nodes[nd.parent].entry, nd.op, t, 0));
       }
     }
-    L.off_dense = dense.size();
-    L.off_diag = diag.size();
+    L.off_dense = tr.dense.size();
+    L.off_diag = tr.diag.size();
     for (int e = 0; e < n_entries; ++e) {
-      const int src = parent_src[L.off_parent + e];
+      const int src = tr.parent_src[L.off_parent + e];
       if (src < 0)
-        diag.push_back(e);
+        tr.diag.push_back(e);
       else
-        dense.push_back(make_int2(e, src));
+        tr.dense.push_back(make_int2(e, src));
     }
-    L.n_dense = (int)(dense.size() - L.off_dense);
-    L.n_diag = (int)(diag.size() - L.off_diag);
+    L.n_dense = (int)(tr.dense.size() - L.off_dense);
+    L.n_diag = (int)(tr.diag.size() - L.off_diag);
     L.n_parents = n_entries;
     L.n_children = slots;
-    L.n_groups = (int)(group.size() - L.off_group);
-    L.n_leaves = (int)(leaf.size() - L.off_leaf);
-    L.n_traces = (int)(trace.size() - L.off_trace);
+    L.n_groups = (int)(tr.group.size() - L.off_group);
+    L.n_leaves = (int)(tr.leaf.size() - L.off_leaf);
+    L.n_traces = (int)(tr.trace.size() - L.off_trace);
     n_mat += slots;
     max_level = std::max<long long>(max_level, slots);
   }
+  // strings across the middle by prefix, in groups of up to kCross
+  std::vector<int> order(across.size());
+  std::iota(order.begin(), order.end(), 0);
+  auto slots = [&](int i) { return std::make_pair(nodes[ends[i].x].slot, nodes[ends[i].y].slot); };
+  std::sort(order.begin(), order.end(), [&](int a, int b) { return slots(a) < slots(b); });
+  for (int i : order) {
+    const auto [l, r] = slots(i);
+    if (tr.cross.empty() || tr.cross.back().x != l || tr.cross.back().z == kCross)
+      tr.cross.push_back(make_int4(l, (int)tr.pair.size(), 0, 0));
+    tr.cross.back().z += 1;
+    tr.pair.push_back(make_int2(r, across[i]));
+  }
+  h->n_cross = (int)tr.cross.size();
   h->n_nodes = n_mat;
   h->max_level_nodes = max_level;
   return MPS_OK;
@@ -154,23 +246,35 @@ static mps_status build_trie(mps_ham* h, const uint8_t* ops, const double* coeff
 // (grow-only); slot strides follow the same dimensions.
 template <typename R>
 static mps_status ensure_env_buffers(const std::vector<int>& chi, mps_state* st, const mps_ham* h) {
-  size_t Lneed = 16, Mneed = 16;
+  size_t Lneed = 16, Mneed = 16, Tneed = 0;
   for (int j = 0; j < h->n; ++j) {
     const LevelHost& L = h->levels[j];
-    const size_t cl = chi[j], cr = chi[j + 1];
-    Lneed = std::max(Lneed, (size_t)L.n_children * cr * cr * sizeof(cplx<R>));
+    const size_t cl = chi[j], cr = chi[j + 1], out = j < h->cut ? cr : cl;
+    Lneed = std::max(Lneed, (size_t)L.n_children * out * out * sizeof(cplx<R>));
     Mneed = std::max(Mneed, (size_t)L.n_parents * 2 * cl * cr * sizeof(cplx<R>));
+    if (j >= h->cut && h->right) Tneed += 2 * cl * cr * sizeof(cplx<R>);
   }
   mps_ctx* c = st->ctx;
-  if (Lneed > st->L_bytes) {
-    dev_free(c, st->d_L[0]);
-    dev_free(c, st->d_L[1]);
-    st->d_L[0] = st->d_L[1] = nullptr;
+  if (Lneed > st->L_bytes || (h->right && !st->d_L[2])) {
+    Lneed = std::max(Lneed, st->L_bytes);
     st->L_bytes = 0;
-    mps_status rc = dev_alloc(c, &st->d_L[0], Lneed);
-    if (rc == MPS_OK) rc = dev_alloc(c, &st->d_L[1], Lneed);
-    if (rc != MPS_OK) return rc;
+    for (void*& p : st->d_L) {
+      dev_free(c, p);
+      p = nullptr;
+    }
+    for (int i = 0; i < (h->right ? 3 : 2); ++i) {
+      mps_status rc = dev_alloc(c, &st->d_L[i], Lneed);
+      if (rc != MPS_OK) return rc;
+    }
     st->L_bytes = Lneed;
+  }
+  if (Tneed > st->BT_bytes) {
+    dev_free(c, st->d_BT);
+    st->d_BT = nullptr;
+    st->BT_bytes = 0;
+    mps_status rc = dev_alloc(c, &st->d_BT, Tneed);
+    if (rc != MPS_OK) return rc;
+    st->BT_bytes = Tneed;
   }
   if (Mneed > st->M_bytes) {
     dev_free(c, st->d_M);
@@ -201,13 +305,13 @@ constexpr int kTcMinChi = 64;
 
 // Tensor-core path of one level (complex64 only).  Returns false if a launch failed.
 template <typename R>
-static bool launch_env_tc(mps_state*, mps_ham*, const LevelHost&, int, const std::vector<int>&, const cplx<R>*,
+static bool launch_env_tc(mps_state*, mps_ham*, const LevelHost&, int, int, const double*, const cplx<R>*,
                           const cplx<R>*, cplx<R>*, cplx<R>*) {
   return false;  // complex128 states never take this path
 }
 
 template <>
-bool launch_env_tc<float>(mps_state* st, mps_ham* h, const LevelHost& L, int j, const std::vector<int>& chi,
+bool launch_env_tc<float>(mps_state* st, mps_ham* h, const LevelHost& L, int chi_l, int chi_r, const double* lam,
                           const float2* Lprev, const float2* Bj, float2* M, float2* Lcur) {
   // the shared-memory opt-in is a per-device function attribute
   static std::mutex mu;
@@ -226,13 +330,12 @@ bool launch_env_tc<float>(mps_state* st, mps_ham* h, const LevelHost& L, int j, 
     }
   }
   cudaStream_t s = c->stream;
-  const int chi_l = chi[j], chi_r = chi[j + 1];
   int* err = &st->d_rep->tc_error;
   if (L.n_diag) {
     KernelScope k(c, MPS_K_ENV_M);
     const size_t tot = (size_t)L.n_diag * chi_l * 2 * chi_r;
     env_m_diag_kernel<float><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-        h->d_diag + L.off_diag, L.n_diag, Bj, st->d_lam + st->lam_off[j], chi_l, chi_r, M);
+        h->d_diag + L.off_diag, L.n_diag, Bj, lam, chi_l, chi_r, M);
   }
   if (L.n_dense) {
     KernelScope k(c, MPS_K_ENV_M);
@@ -275,13 +378,22 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
     fill_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(st->d_vals, nt, 1.0);
   }
   const cplx<R>* B = reinterpret_cast<const cplx<R>*>(st->d_B);
-  cplx<R>* Lprev = reinterpret_cast<cplx<R>*>(st->d_L[0]);
-  cplx<R>* Lcur = reinterpret_cast<cplx<R>*>(st->d_L[1]);
+  cplx<R>* BT = reinterpret_cast<cplx<R>*>(st->d_BT);
   cplx<R>* M = reinterpret_cast<cplx<R>*>(st->d_M);
   const dim3 blk(kTile, kTile);
-  for (int j = 0; j < h->n; ++j) {
+  if (h->right) {
+    size_t most = 0;
+    for (int j = h->cut; j < h->n; ++j) most = std::max(most, (size_t)2 * chi[j] * chi[j + 1]);
+    KernelScope k(c, MPS_K_SETUP);
+    transpose_sites_kernel<R><<<dim3((unsigned)std::min<size_t>((most + 255) / 256, 64), h->n - h->cut), 256, 0, s>>>(
+        B, st->d_site_off, st->d_chi, h->cut, BT);
+  }
+  // one step from the environments in Lprev to those in Lcur, over site j from
+  // a bond of dimension chi_l to one of chi_r
+  auto level = [&](int j, int chi_l, int chi_r, const cplx<R>* Bj, const double* lam, const double* weight,
+                   cplx<R>*& Lprev, cplx<R>*& Lcur) {
     const LevelHost& L = h->levels[j];
-    if (!L.n_parents) continue;
+    if (!L.n_parents) return true;
     EnvLevel lv;
     lv.parent_src = h->d_parent_src + L.off_parent;
     lv.group = h->d_group + L.off_group;
@@ -291,41 +403,56 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
     lv.n_groups = L.n_groups;
     lv.n_leaves = L.n_leaves;
     lv.n_traces = L.n_traces;
-    lv.site = j;
-    lv.cap_l = chi[j];
-    lv.cap_r = chi[j + 1];
-    const cplx<R>* Bj = B + st->site_off[j];
-    const int tl = (lv.cap_l + kTile - 1) / kTile, tr = (lv.cap_r + kTile - 1) / kTile;
-    if (st->tc && std::max(chi[j], chi[j + 1]) >= kTcMinChi) {
+    lv.chi_l = chi_l;
+    lv.chi_r = chi_r;
+    lv.weight = weight;
+    const int tl = (chi_l + kTile - 1) / kTile, tr = (chi_r + kTile - 1) / kTile;
+    if (st->tc && std::max(chi_l, chi_r) >= kTcMinChi) {
       // complex64 on the tensor cores: diagonal parents by scaling, stored
       // environments and children as batched tcgen05 complex GEMMs (below
       // kTcMinChi a 128-row tile is mostly padding and the CUDA-core
       // kernels are faster)
-      if (!launch_env_tc<R>(st, h, L, j, chi, Lprev, Bj, M, Lcur)) {
+      if (!launch_env_tc<R>(st, h, L, chi_l, chi_r, lam, Lprev, Bj, M, Lcur)) {
         set_error("energy: tensor-core launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-        return MPS_ECUDA;
+        return false;
       }
     } else {
       {
         KernelScope k(c, MPS_K_ENV_M);
-        env_m_kernel<R><<<(unsigned)((size_t)L.n_parents * tl * tr), blk, 0, s>>>(
-            Lprev, Bj, st->d_lam + st->lam_off[j], st->d_chi, lv, M);
+        env_m_kernel<R><<<(unsigned)((size_t)L.n_parents * tl * tr), blk, 0, s>>>(Lprev, Bj, lam, lv, M);
       }
       if (L.n_children) {
         KernelScope k(c, MPS_K_ENV_CHILD);
-        env_child_kernel<R><<<(unsigned)((size_t)L.n_groups * (tr * (tr + 1) / 2)), blk, 0, s>>>(M, Bj, st->d_chi, lv,
-                                                                                            Lcur);
+        env_child_kernel<R><<<(unsigned)((size_t)L.n_groups * (tr * (tr + 1) / 2)), blk, 0, s>>>(M, Bj, lv, Lcur);
       }
     }
     if (L.n_leaves) {
       KernelScope k(c, MPS_K_ENV_LEAF);
-      env_leaf_kernel<R><<<(L.n_leaves + 7) / 8, 256, 0, s>>>(M, Bj, st->d_chi, lv, st->d_vals);
+      env_leaf_kernel<R><<<L.n_leaves, 128, 0, s>>>(M, Bj, lv, st->d_vals);
     }
     if (L.n_traces) {
       KernelScope k(c, MPS_K_ENV_TRACE);
-      env_trace_kernel<R><<<(L.n_traces + 7) / 8, 256, 0, s>>>(Lcur, st->d_chi, lv, st->d_vals);
+      env_trace_kernel<R><<<(L.n_traces + 7) / 8, 256, 0, s>>>(Lcur, lv, st->d_vals);
     }
     if (L.n_children) std::swap(Lprev, Lcur);
+    return true;
+  };
+  cplx<R>* left = reinterpret_cast<cplx<R>*>(st->d_L[0]);
+  cplx<R>* other = reinterpret_cast<cplx<R>*>(st->d_L[1]);
+  cplx<R>* right = reinterpret_cast<cplx<R>*>(st->d_L[2]);
+  for (int j = 0; j < h->cut; ++j)
+    if (!level(j, chi[j], chi[j + 1], B + st->site_off[j], st->d_lam + st->lam_off[j], nullptr, left, other))
+      return MPS_ECUDA;
+  if (h->right) {
+    std::vector<size_t> off(h->n + 1, 0);
+    for (int j = h->cut; j < h->n; ++j) off[j + 1] = off[j] + (size_t)2 * chi[j] * chi[j + 1];
+    for (int j = h->n - 1; j >= h->cut; --j)
+      if (!level(j, chi[j + 1], chi[j], BT + off[j], nullptr, st->d_lam + st->lam_off[j], right, other))
+        return MPS_ECUDA;
+  }
+  if (h->n_cross) {
+    KernelScope k(c, MPS_K_ENV_LEAF);
+    env_cross_kernel<R><<<h->n_cross, 128, 0, s>>>(left, right, chi[h->cut], h->d_cross, h->d_pair, st->d_vals);
   }
   {
     KernelScope k(c, MPS_K_REDUCE);
@@ -355,7 +482,7 @@ static void destroy_ham(mps_ham* h) {
   DeviceGuard guard(c->device);
   cudaStreamSynchronize(c->stream);
   for (void* p : {(void*)h->d_parent_src, (void*)h->d_child, (void*)h->d_group, (void*)h->d_leaf, (void*)h->d_trace,
-                  (void*)h->d_coeffs, (void*)h->d_dense, (void*)h->d_diag})
+                  (void*)h->d_coeffs, (void*)h->d_dense, (void*)h->d_diag, (void*)h->d_cross, (void*)h->d_pair})
     dev_free(c, p);
   delete h;
 }
@@ -404,14 +531,8 @@ mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms
   h->ctx = ctx;
   h->n = n_qubits;
   h->n_terms = (long long)n_terms;
-  std::vector<int> parent_src;
-  std::vector<int2> child;
-  std::vector<EnvGroup> group;
-  std::vector<int4> leaf;
-  std::vector<int2> trace;
-  std::vector<int2> dense;
-  std::vector<int> diag;
-  mps_status rc = build_trie(h, ops, coeffs, parent_src, child, group, leaf, trace, dense, diag);
+  Trie tr;
+  mps_status rc = build_trie(h, ops, coeffs, tr);
   if (rc != MPS_OK) {
     delete h;
     return rc;
@@ -425,13 +546,15 @@ mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms
       if (e != cudaSuccess) rc = cuda_fail(e, "mps_hamiltonian_create upload");
     }
   };
-  up((void**)&h->d_parent_src, parent_src.data(), parent_src.size() * sizeof(int));
-  up((void**)&h->d_child, child.data(), child.size() * sizeof(int2));
-  up((void**)&h->d_group, group.data(), group.size() * sizeof(EnvGroup));
-  up((void**)&h->d_leaf, leaf.data(), leaf.size() * sizeof(int4));
-  up((void**)&h->d_trace, trace.data(), trace.size() * sizeof(int2));
-  up((void**)&h->d_dense, dense.data(), dense.size() * sizeof(int2));
-  up((void**)&h->d_diag, diag.data(), diag.size() * sizeof(int));
+  up((void**)&h->d_parent_src, tr.parent_src.data(), tr.parent_src.size() * sizeof(int));
+  up((void**)&h->d_child, tr.child.data(), tr.child.size() * sizeof(int2));
+  up((void**)&h->d_group, tr.group.data(), tr.group.size() * sizeof(EnvGroup));
+  up((void**)&h->d_leaf, tr.leaf.data(), tr.leaf.size() * sizeof(int4));
+  up((void**)&h->d_trace, tr.trace.data(), tr.trace.size() * sizeof(int2));
+  up((void**)&h->d_dense, tr.dense.data(), tr.dense.size() * sizeof(int2));
+  up((void**)&h->d_diag, tr.diag.data(), tr.diag.size() * sizeof(int));
+  up((void**)&h->d_cross, tr.cross.data(), tr.cross.size() * sizeof(int4));
+  up((void**)&h->d_pair, tr.pair.data(), tr.pair.size() * sizeof(int2));
   up((void**)&h->d_coeffs, coeffs, n_terms * sizeof(double));
   if (rc == MPS_OK) {
     cudaError_t e = cudaStreamSynchronize(ctx->stream);

@@ -5,15 +5,30 @@
 //   T_P(L)[b, d] = sum_{a, c, i} conj(B[a, i, b]) L[a, c] P[i, pi(i)] B[c, pi(i), d],
 // where pi(i) is the column of the single nonzero entry of row i of the
 // Pauli matrix.  Strings are arranged in a prefix trie; the environment L of
-// a trie node is computed once and shared by every string through it.  Site
-// j (level j) runs:
+// a trie node is computed once and shared by every string through it.
+//
+// The prefixes go up to the middle of the chain only.  From the other end the
+// suffixes run down to it, with
+//   T*_P(R)[a, c] = sum conj(B[a, i, b]) P[i, pi(i)] B[c, pi(i), d] R[b, d]
+// from the identity (the site tensors are right-canonical), and a string across
+// the middle is <P> = sum_{bd} L[b, d] R[b, d].  The number of distinct
+// prefixes of a molecular Hamiltonian grows with the cube of the sites they
+// cover: meeting halfway takes 8.4 -> 3.6 ms for the 14,251 strings of 20 spin
+// orbitals at chi = 64, and for the 571,876 of 50 it stores 176 thousand environments
+// instead of 1.14 million.  T* is T with the site tensor transposed: the
+// suffixes run on the same kernels over transposed copies, and what is written below for
+// the left half holds for the right half with the bonds exchanged.
+//
+// Site j (level j) runs:
 //   env_m_kernel      M^b_p = L_p B_j[:, b, :] for each parent entry p
 //                     (L_p = diag(lam_j^2) for strings starting at j),
 //   env_child_kernel  L_c = sum_i ph_i B_j[:, i, :]^H M^{pi(i)}_p for the
 //                     nodes c under p that have children,
 //   env_leaf_kernel   <P> = Re sum_i ph_i <B_j[:, i, :], M^{pi(i)}_p> for a
 //                     string ending at j whose node has no children,
-//   env_trace_kernel  <P> = Re Tr L_c for a string ending at a node with children;
+//   env_trace_kernel  <P> = Re Tr L_c for a string ending at a node with children
+// (in the right half both weight the last bond with lam^2);
+// env_cross_kernel sums the strings across the middle;
 // energy_reduce_kernel sums c_k <P_k> in FP64 in a fixed order.
 #pragma once
 
@@ -49,31 +64,31 @@ struct EnvLevel {
   const int4* leaf;       // per string ending at a leaf node: (parent entry, op, term, 0)
   const int2* trace;      // per string ending at a materialised node: (slot, term)
   int n_parents, n_groups, n_leaves, n_traces;
-  int site;
-  int cap_l, cap_r;  // bond dimensions left / right of the site at launch (grid extents and slot strides)
+  int chi_l, chi_r;        // bond dimensions the step comes from and goes to
+  const double* weight;    // lam of the bond that leaves and traces end on (null: ones)
 };
 
 // M_p[a][b][d] = sum_c L_p[a][c] B[c][b][d]   (b = 0, 1): row-major chi_l x 2 chi_r,
-// i.e. M_p = L_p B with B viewed as chi_l x 2 chi_r; slot stride of M: 2 cap_l cap_r
+// i.e. M_p = L_p B with B viewed as chi_l x 2 chi_r; slot stride of M: 2 chi_l chi_r
 template <typename R>
 __global__ void __launch_bounds__(kTile* kTile)
     env_m_kernel(const cplx<R>* __restrict__ Lprev, const cplx<R>* __restrict__ B, const double* __restrict__ lam,
-                 const int* __restrict__ chi, EnvLevel lv, cplx<R>* __restrict__ M) {
+                 EnvLevel lv, cplx<R>* __restrict__ M) {
   using C = cplx<R>;
-  const int chi_l = chi[lv.site], chi_r = chi[lv.site + 1];
-  const int tiles_c = (lv.cap_r + kTile - 1) / kTile, tiles_r = (lv.cap_l + kTile - 1) / kTile;
+  const int chi_l = lv.chi_l, chi_r = lv.chi_r;
+  const int tiles_c = (lv.chi_r + kTile - 1) / kTile, tiles_r = (lv.chi_l + kTile - 1) / kTile;
   const int per = tiles_c * tiles_r;
   const int p = blockIdx.x / per, tile = blockIdx.x % per;
   const int a0 = (tile / tiles_c) * kTile, d0 = (tile % tiles_c) * kTile;
   if (p >= lv.n_parents || a0 >= chi_l || d0 >= chi_r) return;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int src = lv.parent_src[p];
-  C* out = M + (size_t)p * 2 * lv.cap_l * lv.cap_r;
+  C* out = M + (size_t)p * 2 * lv.chi_l * lv.chi_r;
   const int a = a0 + ty, d = d0 + tx;
   const C zero = cmk<R>(0, 0);
   if (src < 0) {
     if (a < chi_l && d < chi_r) {
-      const R w = R(lam[a] * lam[a]);
+      const R w = lam ? R(lam[a] * lam[a]) : R(1);
       const C b0 = B[(size_t)(a * 2 + 0) * chi_r + d], b1 = B[(size_t)(a * 2 + 1) * chi_r + d];
       out[(size_t)a * 2 * chi_r + d] = cscale(b0, w);
       out[(size_t)a * 2 * chi_r + chi_r + d] = cscale(b1, w);
@@ -82,7 +97,7 @@ __global__ void __launch_bounds__(kTile* kTile)
   }
   using MT = Mac<R>;
   using E = typename MT::Elem;
-  const C* L = Lprev + (size_t)src * lv.cap_l * lv.cap_l;
+  const C* L = Lprev + (size_t)src * lv.chi_l * lv.chi_l;
   __shared__ E sL[kTile][kTile + 1];
   __shared__ E sB[2][kTile][kTile + 1];
   typename MT::Acc acc0, acc1;
@@ -117,11 +132,11 @@ __global__ void __launch_bounds__(kTile* kTile)
 // 14,251 strings of 10 orbitals at chi = 64, against one child and every tile.
 template <typename R>
 __global__ void __launch_bounds__(kTile* kTile)
-    env_child_kernel(const cplx<R>* __restrict__ M, const cplx<R>* __restrict__ B, const int* __restrict__ chi,
-                     EnvLevel lv, cplx<R>* __restrict__ Lcur) {
+    env_child_kernel(const cplx<R>* __restrict__ M, const cplx<R>* __restrict__ B, EnvLevel lv,
+                     cplx<R>* __restrict__ Lcur) {
   using C = cplx<R>;
-  const int chi_l = chi[lv.site], chi_r = chi[lv.site + 1];
-  const int tiles = (lv.cap_r + kTile - 1) / kTile;
+  const int chi_l = lv.chi_l, chi_r = lv.chi_r;
+  const int tiles = (lv.chi_r + kTile - 1) / kTile;
   const int per = tiles * (tiles + 1) / 2;
   const int gidx = blockIdx.x / per;
   int bi = 0, di = blockIdx.x % per;  // the tile's row and, counted from the diagonal, column
@@ -130,7 +145,7 @@ __global__ void __launch_bounds__(kTile* kTile)
   if (gidx >= lv.n_groups || d0 >= chi_r) return;
   const EnvGroup gr = lv.group[gidx];
   const bool iz = gr.slot[0] >= 0 || gr.slot[3] >= 0, xy = gr.slot[1] >= 0 || gr.slot[2] >= 0;
-  const C* M0 = M + (size_t)gr.parent * 2 * lv.cap_l * lv.cap_r;  // row stride 2 chi_r
+  const C* M0 = M + (size_t)gr.parent * 2 * lv.chi_l * lv.chi_r;  // row stride 2 chi_r
   const C* M1 = M0 + chi_r;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int b = b0 + ty, d = d0 + tx;
@@ -177,7 +192,7 @@ __global__ void __launch_bounds__(kTile* kTile)
   if (d >= chi_r || b > d) return;
   const C p = MT::value_conj(s00), q = MT::value_conj(s11);
   const C u = MT::value_conj(s01), v = MT::value_conj(s10);
-  const size_t size = (size_t)lv.cap_r * lv.cap_r;
+  const size_t size = (size_t)lv.chi_r * lv.chi_r;
   auto put = [&](int slot, C z) {
     if (slot < 0) return;
     C* out = Lcur + slot * size;
@@ -190,52 +205,146 @@ __global__ void __launch_bounds__(kTile* kTile)
   put(gr.slot[2], cmk<R>(u.y - v.y, v.x - u.x));  // -i u + i v
 }
 
-// One warp per leaf: Re sum_i ph_i sum_{a,b} conj(B[a][i][b]) M^{pi(i)}[a][b], FP64 accumulation.
+// A real as a double-float value.
+template <typename R> __device__ __forceinline__ ff as_ff(R x) {
+  if constexpr (sizeof(R) == 8)
+    return ff_split(x);
+  else
+    return ff_make(x, 0.f);
+}
+__device__ __forceinline__ ff warp_sum_ff(ff s) {
+  for (int x = 16; x > 0; x >>= 1) s = ff_add(s, ff_shfl_xor(s, x));
+  return s;
+}
+
+// One block of four warps per leaf: Re sum_i ph_i sum_{a,b} conj(B[a][i][b]) M^{pi(i)}[a][b],
+// in double-float sums.  One warp per leaf with FP64 sums was a chain of 128
+// iterations at chi = 64: 0.8 of 8.4 ms for the strings of 10 orbitals.
 template <typename R>
-__global__ void env_leaf_kernel(const cplx<R>* __restrict__ M, const cplx<R>* __restrict__ B,
-                                const int* __restrict__ chi, EnvLevel lv, double* __restrict__ vals) {
+__global__ void __launch_bounds__(128)
+    env_leaf_kernel(const cplx<R>* __restrict__ M, const cplx<R>* __restrict__ B, EnvLevel lv,
+                    double* __restrict__ vals) {
   using C = cplx<R>;
-  const int lane = threadIdx.x & 31;
-  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (w >= lv.n_leaves) return;
-  const int chi_l = chi[lv.site], chi_r = chi[lv.site + 1];
-  const int4 lf = lv.leaf[w];
+  const int tid = threadIdx.x;
+  const int chi_l = lv.chi_l, chi_r = lv.chi_r;
+  const int4 lf = lv.leaf[blockIdx.x];
   const PauliRow pr = pauli_row(lf.y);
-  const C* Mp = M + (size_t)lf.x * 2 * lv.cap_l * lv.cap_r;
+  const C ph0 = ccast<C>(pr.ph0), ph1 = ccast<C>(pr.ph1);
+  const C* Mp = M + (size_t)lf.x * 2 * lv.chi_l * lv.chi_r;
   const C* Mi0 = Mp + (size_t)pr.p0 * chi_r;  // row stride 2 chi_r
   const C* Mi1 = Mp + (size_t)pr.p1 * chi_r;
-  double2 s0 = make_double2(0, 0), s1 = make_double2(0, 0);
+  GramAcc acc;
   const int tot = chi_l * chi_r;
-  for (int t = lane; t < tot; t += 32) {
-    const int a = t / chi_r, b = t % chi_r;
-    const C x0 = B[(size_t)(a * 2 + 0) * chi_r + b], x1 = B[(size_t)(a * 2 + 1) * chi_r + b];
-    const C y0 = Mi0[(size_t)a * 2 * chi_r + b], y1 = Mi1[(size_t)a * 2 * chi_r + b];
-    const double2 p0 = ccast<double2>(cmulc(x0, y0)), p1 = ccast<double2>(cmulc(x1, y1));
-    s0.x += p0.x; s0.y += p0.y;
-    s1.x += p1.x; s1.y += p1.y;
+#pragma unroll 2
+  for (int t = tid; t < tot; t += 128) {
+    const int a = t / chi_r, b = t - a * chi_r;
+    const size_t at = (size_t)a * 2 * chi_r + b;
+    const C x0 = B[at], x1 = B[at + chi_r];
+    const C y0 = cmul(ph0, Mi0[at]), y1 = cmul(ph1, Mi1[at]);  // phases of 1, -1, i, -i: exact
+    ff f0 = as_ff(x0.x), f1 = as_ff(x0.y), f2 = as_ff(x1.x), f3 = as_ff(x1.y);
+    if (lv.weight) {
+      ff w = as_ff(lv.weight[b]);
+      w = ff_mul(w, w);
+      f0 = ff_mul(w, f0);
+      f1 = ff_mul(w, f1);
+      f2 = ff_mul(w, f2);
+      f3 = ff_mul(w, f3);
+    }
+    acc.add(f0, as_ff(y0.x));
+    acc.add(f1, as_ff(y0.y));
+    acc.add(f2, as_ff(y1.x));
+    acc.add(f3, as_ff(y1.y));
   }
-  s0.x = warp_sum(s0.x); s0.y = warp_sum(s0.y);
-  s1.x = warp_sum(s1.x); s1.y = warp_sum(s1.y);
-  if (lane == 0) {
-    const double re = (pr.ph0.x * s0.x - pr.ph0.y * s0.y) + (pr.ph1.x * s1.x - pr.ph1.y * s1.y);
-    vals[lf.z] = re;
-  }
+  __shared__ ff part[4];
+  const ff s = warp_sum_ff(acc.value());
+  if ((tid & 31) == 0) part[tid >> 5] = s;
+  __syncthreads();
+  if (tid == 0) vals[lf.z] = ff_join(ff_add(ff_add(part[0], part[1]), ff_add(part[2], part[3])));
 }
 
 // One warp per string ending at a materialised node: Re Tr L.
 template <typename R>
-__global__ void env_trace_kernel(const cplx<R>* __restrict__ Lcur, const int* __restrict__ chi, EnvLevel lv,
-                                 double* __restrict__ vals) {
+__global__ void env_trace_kernel(const cplx<R>* __restrict__ Lcur, EnvLevel lv, double* __restrict__ vals) {
   const int lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (w >= lv.n_traces) return;
-  const int chi_r = chi[lv.site + 1];
+  const int chi_r = lv.chi_r;
   const int2 tr = lv.trace[w];
-  const cplx<R>* L = Lcur + (size_t)tr.x * lv.cap_r * lv.cap_r;
+  const cplx<R>* L = Lcur + (size_t)tr.x * lv.chi_r * lv.chi_r;
   double s = 0.0;
-  for (int b = lane; b < chi_r; b += 32) s += (double)L[(size_t)b * chi_r + b].x;
+  for (int b = lane; b < chi_r; b += 32) {
+    const double wt = lv.weight ? lv.weight[b] * lv.weight[b] : 1.0;
+    s += wt * (double)L[(size_t)b * chi_r + b].x;
+  }
   s = warp_sum(s);
   if (lane == 0) vals[tr.y] = s;
+}
+
+// Transposed site tensors of the right half, [d][i][a] from [a][i][d], one after
+// another (blockIdx.y: the site).
+template <typename R>
+__global__ void transpose_sites_kernel(const cplx<R>* __restrict__ B, const size_t* __restrict__ site_off,
+                                       const int* __restrict__ chi, int cut, cplx<R>* __restrict__ BT) {
+  const int site = cut + blockIdx.y, cl = chi[site], cr = chi[site + 1];
+  size_t off = 0;
+  for (int s = cut; s < site; ++s) off += (size_t)2 * chi[s] * chi[s + 1];
+  const cplx<R>* src = B + site_off[site];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 2 * cl * cr; t += gridDim.x * blockDim.x) {
+    const int d = t / (2 * cl), e = t - d * 2 * cl, i = e >= cl, a = e - i * cl;
+    BT[off + t] = src[(size_t)(a * 2 + i) * cr + d];
+  }
+}
+
+// <P> = sum_{bd} L[b][d] R[b][d] of the strings across the middle: both are
+// Hermitian, so it is the sum over d >= b of Re(L R), twice off the diagonal.
+// One block of four warps takes up to kCross strings of one prefix, so L is
+// read once for them and the loads of the R (L2 latency bounds it) are in flight together;
+// a group's missing strings repeat its last one.  The sums are double-float:
+// in FP64 they would be bound by the FP64 unit.  Row p of the triangle is joined
+// to row chi - 1 - p, which gives chi + 1 entries.
+constexpr int kCross = 8;
+template <typename R>
+__global__ void __launch_bounds__(128)
+    env_cross_kernel(const cplx<R>* __restrict__ L, const cplx<R>* __restrict__ Rm, int chi,
+                     const int4* __restrict__ item, const int2* __restrict__ pair, double* __restrict__ vals) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int4 it = item[blockIdx.x];
+  const size_t size = (size_t)chi * chi;
+  const cplx<R>* Lp = L + it.x * size;
+  const cplx<R>* Rp[kCross];
+  GramAcc acc[kCross];
+#pragma unroll
+  for (int k = 0; k < kCross; ++k) Rp[k] = Rm + pair[it.y + min(k, it.z - 1)].x * size;
+  const int total = chi * (chi + 1) / 2;
+  int p = 0, o = tid;
+  for (int t = tid; t < total; t += 128, o += 128) {
+    while (o > chi) {
+      o -= chi + 1;
+      ++p;
+    }
+    const int b = o < chi - p ? p : chi - 1 - p, d = o < chi - p ? p + o : o - 1;
+    const size_t at = (size_t)b * chi + d;
+    const cplx<R> z = Lp[at];
+    cplx<R> v[kCross];
+#pragma unroll
+    for (int k = 0; k < kCross; ++k) v[k] = Rp[k][at];
+    const R f = b == d ? R(1) : R(2);
+    const ff zr = as_ff(f * z.x), zi = as_ff(-f * z.y);
+#pragma unroll
+    for (int k = 0; k < kCross; ++k) {
+      acc[k].add(zr, as_ff(v[k].x));
+      acc[k].add(zi, as_ff(v[k].y));
+    }
+  }
+  __shared__ ff part[4][kCross];
+#pragma unroll
+  for (int k = 0; k < kCross; ++k) {
+    const ff s = warp_sum_ff(acc[k].value());
+    if (lane == k) part[tid >> 5][k] = s;
+  }
+  __syncthreads();
+  if (tid < it.z)
+    vals[pair[it.y + tid].y] = ff_join(ff_add(ff_add(part[0][tid], part[1][tid]), ff_add(part[2][tid], part[3][tid])));
 }
 
 // E = constant + sum_k c_k vals[k] (terms with an empty support keep vals = 1).
@@ -355,7 +464,7 @@ __global__ void env_m_diag_kernel(const int* __restrict__ list, int n, const cpl
   const int z = (int)(t / per);
   const size_t e = t % per;
   const int a = (int)(e / (2 * chi_r));
-  const R w = R(lam[a] * lam[a]);
+  const R w = lam ? R(lam[a] * lam[a]) : R(1);
   M[(size_t)list[z] * per + e] = cscale(B[e], w);
 }
 

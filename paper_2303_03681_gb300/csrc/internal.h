@@ -160,9 +160,10 @@ struct mps_state {
   double* d_theta = nullptr;
   size_t theta_cap = 0;
   // energy workspace (per state, so states sharing a Hamiltonian can run concurrently)
-  void* d_L[2] = {nullptr, nullptr};
+  void* d_L[3] = {nullptr, nullptr, nullptr};
   void* d_M = nullptr;
-  size_t L_bytes = 0, M_bytes = 0;
+  void* d_BT = nullptr;  // transposed site tensors of the right half
+  size_t L_bytes = 0, M_bytes = 0, BT_bytes = 0;
   double* d_vals = nullptr;
   size_t vals_cap = 0;
   double* d_energy = nullptr;
@@ -206,11 +207,16 @@ struct mps_ham {
   std::vector<mpsv::LevelHost> levels;
   int* d_parent_src = nullptr;
   int2* d_child = nullptr;
+  int cut = 0;        // the bond where prefixes and suffixes meet
+  int n_cross = 0;    // groups of strings across it
+  bool right = false;  // some string reaches past it
   mpsv::EnvGroup* d_group = nullptr;
   int4* d_leaf = nullptr;
   int2* d_trace = nullptr;
   int2* d_dense = nullptr;  // (parent entry, environment slot)
   int* d_diag = nullptr;    // parent entry
+  int4* d_cross = nullptr;  // (left slot, first pair, pairs, 0)
+  int2* d_pair = nullptr;   // (right slot, term)
   double* d_coeffs = nullptr;
 };
 

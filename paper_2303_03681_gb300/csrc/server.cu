@@ -103,12 +103,15 @@ size_t estimate_bytes(const Fragment& f) {
   size_t sites = 0, mn = 1;
   for (int s = 0; s < n; ++s) sites += (size_t)cap(s) * 2 * cap(s + 1);
   for (int q = 0; q + 1 < n; ++q) mn = std::max(mn, (size_t)4 * cap(q) * cap(q + 2));
-  size_t env = 0;
+  size_t env_l = 0, env_m = 0, env_t = 0;
   for (int j = 0; j < n; ++j) {
     const LevelHost& L = f.ham->levels[j];
-    const size_t cl = cap(j), cr = cap(j + 1);
-    env = std::max(env, 2 * (size_t)L.n_children * cr * cr * elem + (size_t)L.n_parents * 2 * cl * cr * elem);
+    const size_t cl = cap(j), cr = cap(j + 1), out = j < f.ham->cut ? cr : cl;
+    env_l = std::max(env_l, (size_t)L.n_children * out * out * elem);
+    env_m = std::max(env_m, (size_t)L.n_parents * 2 * cl * cr * elem);
+    if (j >= f.ham->cut && f.ham->right) env_t += 2 * cl * cr * elem;
   }
+  const size_t env = (f.ham->right ? 3 : 2) * env_l + env_m + env_t;
   // the operand planes of the split-product tensor-core contractions: A and B
   // pieces of (2 and 4) x maxcap rows by 4 maxcap FP32 values, hi and lo
   size_t tc = 0;

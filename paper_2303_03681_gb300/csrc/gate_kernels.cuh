@@ -93,13 +93,21 @@ __global__ void reset_kernel(cplx<R>* __restrict__ B, const size_t* __restrict__
 // ---------------------------------------------------------------------------
 // theta = B_q B_{q+1}; gate (G1 + G2; the SVD applies the lam scaling as it loads)
 // ---------------------------------------------------------------------------
+// The gate's entries for theta_tile, by the block's first 16 threads (one load
+// each that hides behind the first tile's; read where they are used they added
+// a load's latency to every gate).  The tile loop's barrier stands between.
+template <typename R>
+__device__ __forceinline__ void load_gate(const DevGate* gate, int tid, typename Mac<R>::Elem* u) {
+  if (tid < 16) u[tid] = Mac<R>::load(ccast<cplx<R>>(__ldcg(gate->u + tid)));
+}
+
 // One 16 x 16 tile (a_l, a_r) with both physical indices, by 256 threads (tx,
-// ty).  sL, sR: the group's tiles, 2 x 16 x 17 entries each.  Every thread of
+// ty).  u: the gate in shared memory.  sL, sR: the group's tiles, 2 x 16 x 17 entries each.  Every thread of
 // the block calls it (act false: no tile, only the barriers).  The site tensors
 // are read past L1: a run of gates changes them between calls.
 template <typename R>
 __device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const cplx<R>* __restrict__ Br,
-                                           const double2* __restrict__ u, int chi_l, int chi_m, int chi_r, int al0,
+                                           const typename Mac<R>::Elem* u, int chi_l, int chi_m, int chi_r, int al0,
                                            int ar0, int tx, int ty, bool act, typename Mac<R>::Elem (*sL)[kTile][kTile + 1],
                                            typename Mac<R>::Elem (*sR)[kTile][kTile + 1], cplx<R>* __restrict__ Cm) {
   using C = cplx<R>;
@@ -153,7 +161,7 @@ __device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const
       for (int ip = 0; ip < 2; ++ip)
 #pragma unroll
         for (int jp = 0; jp < 2; ++jp)
-          MT::fma(out, MT::load(ccast<C>(u[(2 * i + j) * 4 + 2 * ip + jp])), th[ip][jp]);
+          MT::fma(out, u[(2 * i + j) * 4 + 2 * ip + jp], th[ip][jp]);
       Cm[(size_t)(2 * al + i) * n + j * chi_r + ar] = MT::value(out);
     }
   }
@@ -165,10 +173,16 @@ __global__ void __launch_bounds__(kTile* kTile)
                  const DevGate* __restrict__ gate, const int* __restrict__ chi, int q, cplx<R>* __restrict__ Cm) {
   __shared__ typename Mac<R>::Elem sL[2][kTile][kTile + 1];
   __shared__ typename Mac<R>::Elem sR[2][kTile][kTile + 1];
-  const int chi_l = chi[q], chi_r = chi[q + 2];
+  // launched while the gate before may still run (gate by gate on a stream):
+  // its results are read after this, and past L1
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int chi_l = __ldcg(chi + q), chi_r = __ldcg(chi + q + 2);
   const int al0 = blockIdx.y * kTile, ar0 = blockIdx.x * kTile;
   if (al0 >= chi_l || ar0 >= chi_r) return;
-  theta_tile<R>(Bl, Br, gate->u, chi_l, chi[q + 1], chi_r, al0, ar0, threadIdx.x, threadIdx.y, true, sL, sR, Cm);
+  __shared__ typename Mac<R>::Elem s_u[16];
+  load_gate<R>(gate, threadIdx.y * kTile + threadIdx.x, s_u);
+  theta_tile<R>(Bl, Br, s_u, chi_l, __ldcg(chi + q + 1), chi_r, al0, ar0, threadIdx.x, threadIdx.y, true, sL, sR, Cm);
 }
 
 // ---------------------------------------------------------------------------

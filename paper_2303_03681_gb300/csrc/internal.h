@@ -244,6 +244,7 @@ struct SvdJob {
   void* Bq;  // B~_q = C V^H / ||s[:k]|| (nullable: not wanted)
   char* ws;
   cudaStream_t stream;
+  bool early = false;  // may be launched before the kernel ahead of it on the stream ends
 };
 #define MPSV_SVD_DECL(x)                            \
   size_t svd_workspace_##x(int mcap, int ncap);     \

@@ -1197,6 +1197,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     __syncthreads();
   };
 
+  cudaTriggerProgrammaticLaunchCompletion();  // the next gate's launch overlaps the rest
   if (direct) {
     // ---- one CTA: W = C V^H from shared memory, one column of W per group of
     // lanes (a lane takes every g-th row); W replaces A.  Against the tiles
@@ -1402,7 +1403,8 @@ __global__ void __launch_bounds__(kSvdThreads<A>, 1)
                cplx<R>* __restrict__ Bq, char* __restrict__ gws) {
   __shared__ float2 s_mail[2 * 16];
   const int Pl = (int)cg::this_cluster().num_blocks(), me = (int)cg::this_cluster().block_rank();
-  const int m = 2 * chi[q], n = 2 * chi[q + 2];
+  cudaGridDependencySynchronize();  // may be launched while the theta contraction runs
+  const int m = 2 * __ldcg(chi + q), n = 2 * __ldcg(chi + q + 2);
   const int P = svd_team_size<A>(m, n, Pl);
   if (me >= P) return;  // an exited CTA counts as arrived at the cluster barriers
   if (P == 1) {

@@ -84,7 +84,7 @@ template <class A, class R> void svd_launch_t(const SvdJob& j) {
   const cplx<R>* C = static_cast<const cplx<R>*>(j.C);
   cplx<R>* B = static_cast<cplx<R>*>(j.Bnext);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(kSvdThreads<A>);
   cfg.stream = j.stream;
   cfg.attrs = attr;
@@ -95,17 +95,23 @@ template <class A, class R> void svd_launch_t(const SvdJob& j) {
   attr[0].val.clusterDim.x = pl.P;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  if (j.early) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   cudaLaunchKernelEx(&cfg, svd_kernel<A, R>, C, j.lam_l, j.chi, j.q, j.p, B, j.lam_next, j.rep,
                      static_cast<cplx<R>*>(j.Bq), j.ws);
   if (!pl.grid) return;
   GridSync* sync = reinterpret_cast<GridSync*>(j.ws + SvdWs<A>(j.mcap, j.ncap, true).total);
   cudaMemsetAsync(sync, 0, sizeof(GridSync), j.stream);
   cfg.gridDim = dim3(pl.grid);
+  cfg.numAttrs = 1;
   cfg.dynamicSmemBytes = pl.grid_smem;
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cudaLaunchKernelEx(&cfg, svd_grid_kernel<A, R>, C, j.lam_l, j.chi, j.q, j.p, B, j.lam_next, j.rep,
-                     static_cast<cplx<R>*>(j.Bq), j.ws, sync,                     pl.P, (unsigned)pl.grid_smem);
+                     static_cast<cplx<R>*>(j.Bq), j.ws, sync, pl.P, (unsigned)pl.grid_smem);
 }
 
 }  // namespace mpsv

@@ -117,28 +117,37 @@ __device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const
   const int al = al0 + ty, ar = ar0 + tx;
   act = act && al0 < chi_l && ar0 < chi_r;
   const bool mine = act && al < chi_l && ar < chi_r;
+  // the next tiles are loaded while these are summed: a small theta is a chain
+  // of its chi_m / 16 load latencies (28-qubit UCCSD 53.8 -> 53.0 ms)
+  C l0 = cmk<R>(0, 0), l1 = l0, r0 = l0, r1 = l0;
+  auto fetch = [&](int m0) {
+    const int mm = m0 + tx, mr = m0 + ty;
+    const bool ok = al < chi_l && mm < chi_m, okr = mr < chi_m && ar < chi_r;
+    l0 = ok ? __ldcg(Bl + (size_t)(al * 2 + 0) * chi_m + mm) : cmk<R>(0, 0);
+    l1 = ok ? __ldcg(Bl + (size_t)(al * 2 + 1) * chi_m + mm) : cmk<R>(0, 0);
+    r0 = okr ? __ldcg(Br + (size_t)(mr * 2 + 0) * chi_r + ar) : cmk<R>(0, 0);
+    r1 = okr ? __ldcg(Br + (size_t)(mr * 2 + 1) * chi_r + ar) : cmk<R>(0, 0);
+  };
+  if (act) fetch(0);
   for (int m0 = 0; m0 < chi_m; m0 += kTile) {
     if (act) {
-      const int mm = m0 + tx;
-      const bool ok = al < chi_l && mm < chi_m;
-      sL[0][ty][tx] = ok ? MT::load(__ldcg(Bl + (size_t)(al * 2 + 0) * chi_m + mm)) : MT::zero();
-      sL[1][ty][tx] = ok ? MT::load(__ldcg(Bl + (size_t)(al * 2 + 1) * chi_m + mm)) : MT::zero();
-      const int mr = m0 + ty;
-      const bool okr = mr < chi_m && ar < chi_r;
-      sR[0][ty][tx] = okr ? MT::load(__ldcg(Br + (size_t)(mr * 2 + 0) * chi_r + ar)) : MT::zero();
-      sR[1][ty][tx] = okr ? MT::load(__ldcg(Br + (size_t)(mr * 2 + 1) * chi_r + ar)) : MT::zero();
+      sL[0][ty][tx] = MT::load(l0);
+      sL[1][ty][tx] = MT::load(l1);
+      sR[0][ty][tx] = MT::load(r0);
+      sR[1][ty][tx] = MT::load(r1);
     }
     __syncthreads();
+    if (act && m0 + kTile < chi_m) fetch(m0 + kTile);
     if (mine) {
       const int kend = min(kTile, chi_m - m0);
 #pragma unroll 4
       for (int kk = 0; kk < kend; ++kk) {
-        const E l0 = sL[0][ty][kk], l1 = sL[1][ty][kk];
-        const E r0 = sR[0][kk][tx], r1 = sR[1][kk][tx];
-        MT::fma(acc[0][0], l0, r0);
-        MT::fma(acc[0][1], l0, r1);
-        MT::fma(acc[1][0], l1, r0);
-        MT::fma(acc[1][1], l1, r1);
+        const E x0 = sL[0][ty][kk], x1 = sL[1][ty][kk];
+        const E y0 = sR[0][kk][tx], y1 = sR[1][kk][tx];
+        MT::fma(acc[0][0], x0, y0);
+        MT::fma(acc[0][1], x0, y1);
+        MT::fma(acc[1][0], x1, y0);
+        MT::fma(acc[1][1], x1, y1);
       }
     }
     __syncthreads();

@@ -217,10 +217,23 @@ template <int M> void set_attrs() {
   });
 }
 
-// The GEMM over a grid of (column tiles, row tiles).
+// The GEMM over a grid of (column tiles, row tiles), right after the split
+// kernel: its CTAs set up their barriers and tensor memory while that runs and
+// wait for it in the kernel (chi = 512 theta in TF32X3 30.2 -> 29.9 us; eight
+// 12-qubit evaluations 12.6 -> 12.2 ms).
 template <int M, class Epi>
 void launch_gemm(const TcWork& w, dim3 grid, const Epi& epi, int* err, cudaStream_t s) {
-  cgemm_tma_kernel<M, Epi><<<grid, kThreads, kSmemBytes, s>>>(w.maps[0], w.maps[1], w.maps[2], w.maps[3], epi, err);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, cgemm_tma_kernel<M, Epi>, w.maps[0], w.maps[1], w.maps[2], w.maps[3], epi, err);
 }
 
 // Blocks of 256 threads for `items` work items (grid-stride beyond 152 x 16 blocks).

@@ -270,6 +270,7 @@ __global__ void __launch_bounds__(256) split_ab_kernel(SrcA sa, SrcB sb, int ld,
                                                         typename ModeTraits<M>::T* __restrict__ blo) {
   using T = typename ModeTraits<M>::T;
   __shared__ float2 tile[kSplitTile][kSplitTile + 1];
+  cudaTriggerProgrammaticLaunchCompletion();
   if ((int)blockIdx.x < a_blocks) {
     int rows, Ka;
     sa.dims(rows, Ka);
@@ -396,6 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_s;
+  cudaGridDependencySynchronize();  // launched while the split kernel runs: its planes from here on
   const int n0r = blockIdx.x * kBNr;  // first real B row (embedded column) of the tile
 
   if (warp == 0) {

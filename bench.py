@@ -414,8 +414,8 @@ def run_gpu(args):
                                               "auto": "complex64 storage, TF32x3 contractions at capacity >= 256, "}
                                              [w["precision"]]
                                              + {"fp32": "FP32 Jacobi SVD",
-                                                "fp64": ("FP64-accurate Jacobi SVD (FP32 sweeps, FP64 "
-                                                         "re-orthonormalisation, double-float sweeps)"),
+                                                "fp64": ("FP64-accurate SVD (pivoted Gram-Schmidt and Jacobi in "
+                                                         "double-float, below 32 columns in FP64)"),
                                                 "fp64-all": "FP64 Jacobi SVD"}[args.svd]
                                              + ", FP64 energy sum"),
                        contractions=contraction_label(args, w, reps),
@@ -698,7 +698,7 @@ def svd_study(mps, device, sizes=(128, 256, 512, 1024), reps=3):
                      "max_sv_error_vs_lapack": err})
     ctx.close()
     return {"what": "2chi x 2chi complex128 theta, graded spectrum (1 .. 1e-10), keep chi_max = chi at eps 1e-8",
-            "ours": "FP64-accurate one-sided Jacobi (FP32 sweeps, FP64 sweeps) on a thread-block cluster",
+            "ours": "FP64-accurate pivoted Gram-Schmidt and one-sided Jacobi (double-float) on a thread-block cluster",
             "cusolver": "torch.linalg.svd on the GPU (cuSOLVER, run-only comparator)",
             "lapack": f"numpy.linalg.svd on the host (zgesdd, {blas_threads()} threads)", "rows": rows}
 

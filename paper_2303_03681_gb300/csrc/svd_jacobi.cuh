@@ -28,11 +28,11 @@
 // memory of a ping-pong hand-over, and the same code for cluster and grid.
 //
 // What it measured (one theta, against FP32-then-double-float sweeps of [A; V]
-// on 8 CTAs, which it replaced): 124 x 124 over ten decades 19.2 -> 4.7 ms (36
-// -> 10 sweeps), 62 x 94 of rank 31 8.2 -> 0.94 ms, 512 x 512 1.21 s -> 48 ms
-// (8 CTAs -> a grid of 128), 16 x 16 in FP64 1.06 -> 0.56 ms.  It is bound by
-// the FP32 pipe in the rotations (about a third of its rate at 124 x 124, the
-// rest is latency of the dependent pair steps and barriers).
+// on 8 CTAs, which it replaced): 124 x 124 over ten decades 19.5 -> 4.4 ms (36
+// -> 10 sweeps), 62 x 94 of rank 31 8.2 -> 0.89 ms, 512 x 512 1.20 s -> 47 ms
+// (8 CTAs -> a grid of 128), 16 x 16 in FP64 1.10 -> 0.57 ms.  It is bound by
+// the dependent pair steps and the barrier that ends each (at 124 x 124 the FP32
+// pipe is busy for 37 % of the time, barriers are most of the stalls).
 //
 // A pair of columns is one step of a group of 8 to 32 lanes: as few lanes as
 // give every warp a pair, because the angle and the reductions cost each

@@ -61,13 +61,19 @@ constexpr int kScaleExp = 40;
 constexpr float kZeroNorm2 = 1e-34f * 1.2089258e24f;  // (1e-17 2^40)^2
 
 // ---- teams: the CTAs that work on one theta --------------------------------
-// publish / fetch exchange one (value, index) candidate per CTA in each
-// Gram-Schmidt step; column() gives a readable copy of another CTA's column.
+// publish / candidate exchange one (value, index) pair per CTA in each
+// Gram-Schmidt step; remote() reads another CTA's column.  barrier() returns,
+// for the whole CTA alike, whether every CTA arrived: where it is false (only a
+// grid can give up) what the others published must not be read, and the CTA
+// leaves at once.
 
 struct OneTeam {
   static constexpr bool kGlobalA = false;
   static constexpr int me = 0, P = 1;
-  __device__ void barrier() { __syncthreads(); }
+  __device__ bool barrier() {
+    __syncthreads();
+    return true;
+  }
 };
 
 struct ClusterTeam {
@@ -75,9 +81,10 @@ struct ClusterTeam {
   int me, P;
   float2* mail;  // shared memory: [2][16] candidates
   int barriers = 0;
-  __device__ void barrier() {
+  __device__ bool barrier() {
     cg::this_cluster().sync();
     ++barriers;
+    return true;
   }
   __device__ void publish(int par, float v, int idx) {  // threads 0 .. P-1 of one warp
     const int t = threadIdx.x;
@@ -90,8 +97,9 @@ struct ClusterTeam {
 };
 
 // Barrier of a co-resident (cooperative) grid.  A wait that does not end
-// within about two seconds sets the abort flag, which every CTA checks: the
-// kernel then leaves with MPS_ETIMEOUT.
+// within about two seconds sets the abort flag, which ends every other wait: a
+// CTA whose wait was given up leaves the kernel, which reports MPS_ETIMEOUT.
+// (A CTA that still finds all others arrived goes on to its next barrier.)
 struct GridSync {
   unsigned count, gen, abort, pad;
 };
@@ -101,9 +109,10 @@ struct GridTeam {
   int me, P;
   GridSync* sync;
   float2* mail;  // global memory: [2][P]
-  __device__ void barrier() {
+  __device__ bool barrier() {
     __threadfence();
     __syncthreads();
+    bool gave_up = false;
     if (threadIdx.x == 0) {
       volatile unsigned* gen = &sync->gen;
       const unsigned g = *gen;
@@ -116,6 +125,7 @@ struct GridTeam {
         while (*gen == g) {
           if (clock64() - t0 > 4000000000ll || *(volatile unsigned*)&sync->abort) {
             atomicExch(&sync->abort, 1u);
+            gave_up = true;
             break;
           }
           __nanosleep(20);
@@ -123,9 +133,8 @@ struct GridTeam {
       }
       __threadfence();
     }
-    __syncthreads();
+    return !__syncthreads_or(gave_up);
   }
-  __device__ bool aborted() const { return *(volatile unsigned*)&sync->abort != 0; }
   __device__ void publish(int par, float v, int idx) {
     if (threadIdx.x == 0) __stcg(mail + par * P + me, make_float2(v, __int_as_float(idx)));
   }
@@ -390,7 +399,7 @@ __device__ __forceinline__ bool jacobi_pair(typename Mem<kG>::H cx, typename Mem
 // (SvdWs).  C and lam_l are read past L1: a run of gates changes them between
 // calls.  The dynamic shared memory holds an SvdSmem of the team's size.  kGX: X's blocks stay in the
 // global workspace.  Writes B~_{q+1} (k x n), lam_{q+1}, *chi_out and the
-// report; returns k.  Bq (nullable): B~_q = C V^H / ||s[:k]|| as well.
+// report; returns k, or 0 when a barrier was given up.  Bq (nullable): B~_q = C V^H / ||s[:k]|| as well.
 template <class A, class R, class Team, bool kGX>
 __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* __restrict__ lam_l, int m, int n,
                         const SvdParams& p, cplx<R>* __restrict__ Bnext, double* __restrict__ lam_next, int* chi_out,
@@ -485,7 +494,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   __syncthreads();
   if constexpr (!std::is_same<Team, OneTeam>::value) {
     if (tid < 32) tm.publish(0, (float)s_i[1], s_i[0]);
-    tm.barrier();
+    if (!tm.barrier()) return 0;
     int e = -100000;
     float c = -100000.f;
     for (int r = 0; r < P; ++r) {
@@ -558,7 +567,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         f = warp_sum(f);
         tm.publish(1, f, 0);
       }
-      tm.barrier();
+      if (!tm.barrier()) return 0;
       for (int k = 0; k < P; ++k) fro2 += tm.candidate(1, k).x;
     } else {
       float f = 0.f;
@@ -586,7 +595,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           warp_argmax(nc, nloc, best, li);
           tm.publish(j & 1, best, li);
         }
-        tm.barrier();
+        if (!tm.barrier()) return 0;
         best = -1.f;
         li = 0;
         for (int k0 = 0; k0 < P; k0 += 32) {
@@ -613,7 +622,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         __syncthreads();
         for (int i = tid; i < nloc; i += T)
           if (nc[i] >= 0.f) nc[i] *= up * up;
-        tm.barrier();
+        if (!tm.barrier()) return 0;
         continue;
       }
       const int pc = owner + li * P;  // pivot column of A
@@ -775,7 +784,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       fl[id] = __ldcg(gfl + id);
     }
   };
-  tm.barrier();  // X complete (and, with several CTAs, A's shared memory free)
+  if (!tm.barrier()) return 0;  // X complete (and, with several CTAs, A's shared memory free)
   if (P > 1)
     for (int slot = 0; slot < nslots; ++slot) fetch(slot, block_at(slot, 0));
   for (int id = tid; id < r; id += T) fl[id] = 2;  // bit 0: rotated in this sweep, bit 1: in the previous one
@@ -823,7 +832,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         }
       }
     }
-    tm.barrier();
+    if (!tm.barrier()) return 0;
     if (P > 1)
       for (int id = tid; id < r; id += T) sg[id] = __ldcg(gnrm + id);
     if (sweep > 0) {
@@ -847,8 +856,6 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       if (heads && off < 1e-6f) heads = false;
     }
     __syncthreads();
-    if constexpr (std::is_same<Team, GridTeam>::value)
-      if (tm.aborted()) break;
     if (converged || sweep >= p.max_sweeps) break;
     // ---- tail: T = the smallest columns, all outside the kept set, whose
     // total weight is at most a quarter of the next larger column's and, when
@@ -997,7 +1004,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       // hand the blocks on: position pos -> pos + 1 (pos >= 1), 2P - 1 -> 1
       for (int slot = 0; slot < 2; ++slot)
         if (!(slot == 0 && me == 0)) flush(slot, slot ? b1 : b0);
-      tm.barrier();
+      if (!tm.barrier()) return 0;
       for (int slot = 0; slot < 2; ++slot)
         if (!(slot == 0 && me == 0)) {
           const int nb = block_at(slot, rnd + 1);
@@ -1257,7 +1264,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     }
     return k;
   }
-  tm.barrier();  // every row of B~_{q+1} is written, X's shared memory is free
+  if (!tm.barrier()) return 0;  // every row of B~_{q+1} is written, X's shared memory is free
 
   // ---- W = C V^H
   using WA = A;  // complex64 states too: one rounding to FP32 instead of n
@@ -1353,7 +1360,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     }
   }
   if (refine) {
-    tm.barrier();
+    if (!tm.barrier()) return 0;
     finish_lam([&](int a) {
       const double d = __ldcg(gnrm + a);
       if constexpr (std::is_same<A, ArF64>::value) {
@@ -1431,11 +1438,12 @@ __global__ void __launch_bounds__(kSvdThreads<A>, 1)
   const int P = min((int)gridDim.x, max(2, (min(m, n) + 3) / 4));
   if ((int)blockIdx.x >= P) return;
   GridTeam tm{(int)blockIdx.x, P, sync, reinterpret_cast<float2*>(gws + SvdWs<A>(m, n, true).mail)};
+  int k;
   if (SvdSmem<A>::bytes(m, n, P, false, true) <= smem_bytes)
-    svd_body<A, R, GridTeam, false>(tm, Cm, lam_l, m, n, p, Bnext, lam_next, chi + q + 1, rep, Bq, gws);
+    k = svd_body<A, R, GridTeam, false>(tm, Cm, lam_l, m, n, p, Bnext, lam_next, chi + q + 1, rep, Bq, gws);
   else
-    svd_body<A, R, GridTeam, true>(tm, Cm, lam_l, m, n, p, Bnext, lam_next, chi + q + 1, rep, Bq, gws);
-  if (tm.aborted() && blockIdx.x == 0 && threadIdx.x == 0) rep->tc_error = 1;
+    k = svd_body<A, R, GridTeam, true>(tm, Cm, lam_l, m, n, p, Bnext, lam_next, chi + q + 1, rep, Bq, gws);
+  if (k == 0 && threadIdx.x == 0) rep->tc_error = 1;  // any CTA that gave up: its part is missing
 }
 
 }  // namespace mpsv

@@ -43,7 +43,8 @@ typedef enum {
   MPS_EINVAL = 1,     /* bad argument (null handle, non-adjacent gate, size) */
   MPS_ENOMEM = 2,     /* device allocation failed or the allocation cap was hit */
   MPS_ECUDA = 3,      /* a CUDA runtime call failed */
-  MPS_ETIMEOUT = 4,   /* a bounded device-side wait ran out */
+  MPS_ETIMEOUT = 4,   /* a bounded device-side wait ran out: the result is not usable, and a state
+                         it happened on reports it until it is reset */
   MPS_ENOTCONV = 5,   /* a truncation SVD reached its Jacobi sweep cap (Algorithm 1's
                          stopping test was not met).  The result is still delivered: the
                          state is updated and the energy written with that SVD as it stood,

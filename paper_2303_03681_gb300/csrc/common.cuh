@@ -108,7 +108,8 @@ struct DevReport {
   int max_chi;
   int degenerate_cuts;
   int not_converged;  // SVDs that reached the sweep cap
-  int tc_error;       // a tensor-core kernel ran out of its bounded wait (read with not_converged in one copy)
+  int tc_error;       // a bounded wait of a tensor-core contraction or a grid SVD ran out: cleared by a reset
+                      // only, since every later result rests on it (read with not_converged in one copy)
   int max_sweeps;
   int pad;
   long long two_qubit_gates;

@@ -372,7 +372,6 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
   if (rc != MPS_OK) return rc;
   const long long nt = h->n_terms;
   mps_ctx* c = st->ctx;
-  if (st->tc) MPSV_CUDA(cudaMemsetAsync(&st->d_rep->tc_error, 0, sizeof(int), s));
   if (nt) {
     KernelScope k(c, MPS_K_SETUP);
     fill_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(st->d_vals, nt, 1.0);
@@ -456,7 +455,7 @@ static mps_status energy_levels(mps_state* st, mps_ham* h, double* d_out) {
   }
   {
     KernelScope k(c, MPS_K_REDUCE);
-    energy_reduce_kernel<<<1, 1024, 0, s>>>(st->d_vals, h->d_coeffs, nt, 0.0, st->tc ? &st->d_rep->tc_error : nullptr,
+    energy_reduce_kernel<<<1, 1024, 0, s>>>(st->d_vals, h->d_coeffs, nt, 0.0, &st->d_rep->tc_error,
                                             d_out ? d_out : st->d_energy);
   }
   MPSV_CUDA(cudaGetLastError());
@@ -499,9 +498,22 @@ cudaError_t queue_flags(mps_state* st, StateFlags* f) {
   return cudaMemcpyAsync(f, &st->d_rep->not_converged, sizeof(StateFlags), cudaMemcpyDeviceToHost, st->ctx->stream);
 }
 
+mps_status svd_status(const DevReport& r, const char* who, int not_converged) {
+  if (r.tc_error) {
+    set_error("%s: a bounded wait on the device ran out; the result is not usable", who);
+    return MPS_ETIMEOUT;
+  }
+  if (not_converged > 0) {
+    set_error("%s: %d truncation SVDs reached the Jacobi sweep cap; their results were used as they stand", who,
+              not_converged);
+    return MPS_ENOTCONV;
+  }
+  return MPS_OK;
+}
+
 mps_status flags_status(const StateFlags& f, bool gates) {
   if (f.tc_error) {
-    set_error("energy: a tensor-core contraction ran out of its bounded wait");
+    set_error("a bounded wait on the device ran out (a tensor-core contraction or a co-resident SVD); reset the state");
     return MPS_ETIMEOUT;
   }
   if (gates && f.not_converged) {

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(128)
 
 // E = constant + sum_k c_k vals[k] (terms with an empty support keep vals = 1).
 // One block of 1024 threads; fixed summation order.
-// A set *err (a tensor-core contraction gave up waiting) turns the energy into NaN.
+// A set *err (a bounded wait of this state's kernels ran out) turns the energy into NaN.
 static __global__ void energy_reduce_kernel(const double* __restrict__ vals, const double* __restrict__ coeffs,
                                             long long n_terms, double constant, const int* __restrict__ err,
                                             double* __restrict__ out) {

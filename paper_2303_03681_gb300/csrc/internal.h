@@ -281,10 +281,12 @@ static_assert(offsetof(DevReport, tc_error) == offsetof(DevReport, not_converged
               "StateFlags mirrors two adjacent DevReport fields");
 // Queues the read of a state's flags into *f (valid once the stream has synchronised).
 cudaError_t queue_flags(mps_state* st, StateFlags* f);
-// The status an evaluation reports for its flags: MPS_ETIMEOUT for a
-// tensor-core timeout, else MPS_ENOTCONV when gates count and an SVD reached
+// The status an evaluation reports for its flags: MPS_ETIMEOUT where a bounded
+// wait on the device ran out, else MPS_ENOTCONV when gates count and an SVD reached
 // its sweep cap (the results are written as they stand), else MPS_OK.
 mps_status flags_status(const StateFlags& f, bool gates);
+// The status of SVDs whose whole report the host has read.
+mps_status svd_status(const DevReport& r, const char* who, int not_converged);
 // A status that still delivers its result (the energy, the updated state).
 inline bool status_has_result(mps_status s) { return s == MPS_OK || s == MPS_ENOTCONV; }
 

@@ -417,6 +417,26 @@ mps_status state_run_circuit(mps_state* st, const mps_circuit* c, const double* 
   return MPS_OK;
 }
 
+static void copy_report(const DevReport& r, mps_report* out) {
+  out->discarded_weight = r.discarded_weight;
+  out->min_kept_sv = r.min_kept_sv;
+  out->max_chi = r.max_chi;
+  out->degenerate_cuts = r.degenerate_cuts;
+  out->svd_not_converged = r.not_converged;
+  out->max_sweeps_used = r.max_sweeps;
+  out->two_qubit_gates = r.two_qubit_gates;
+  out->svd_flops = r.svd_flops;
+  out->svd_sweeps_fp32 = r.sweeps_fp32;
+  out->svd_sweeps_fp64 = r.sweeps_fp64;
+  for (int i = 0; i < 4; ++i) out->svd_phase_cycles[i] = r.phase_cycles[i];
+}
+
+static mps_status read_report(mps_state* st, DevReport* r) {
+  MPSV_CUDA(cudaMemcpyAsync(r, st->d_rep, sizeof(*r), cudaMemcpyDeviceToHost, st->ctx->stream));
+  MPSV_CUDA(cudaStreamSynchronize(st->ctx->stream));
+  return MPS_OK;
+}
+
 static void destroy_state(mps_state* st) {
   if (!st) return;
   mps_ctx* c = st->ctx;
@@ -775,20 +795,9 @@ mps_status mps_get_report(mps_state* st, mps_report* out) {
   }
   DeviceGuard guard(st->ctx->device);
   DevReport r;
-  MPSV_CUDA(cudaMemcpyAsync(&r, st->d_rep, sizeof(r), cudaMemcpyDeviceToHost, st->ctx->stream));
-  MPSV_CUDA(cudaStreamSynchronize(st->ctx->stream));
-  out->discarded_weight = r.discarded_weight;
-  out->min_kept_sv = r.min_kept_sv;
-  out->max_chi = r.max_chi;
-  out->degenerate_cuts = r.degenerate_cuts;
-  out->svd_not_converged = r.not_converged;
-  out->max_sweeps_used = r.max_sweeps;
-  out->two_qubit_gates = r.two_qubit_gates;
-  out->svd_flops = r.svd_flops;
-  out->svd_sweeps_fp32 = r.sweeps_fp32;
-  out->svd_sweeps_fp64 = r.sweeps_fp64;
-  for (int i = 0; i < 4; ++i) out->svd_phase_cycles[i] = r.phase_cycles[i];
-  return MPS_OK;
+  mps_status rc = read_report(st, &r);
+  if (rc == MPS_OK) copy_report(r, out);
+  return rc;
 }
 
 mps_status mps_apply_gates(mps_state* st, const mps_gate* gates, size_t n, mps_report* report) {
@@ -839,19 +848,16 @@ mps_status mps_apply_gates(mps_state* st, const mps_gate* gates, size_t n, mps_r
     st->broken = true;
     return cuda_fail(e, "mps_apply_gates");
   }
-  mps_report r;
-  mps_status rc = mps_get_report(st, &r);
+  DevReport r;
+  mps_status rc = read_report(st, &r);
   if (rc != MPS_OK) return rc;
-  if (report) *report = r;
+  if (report) copy_report(r, report);
   // SVDs that reached the sweep cap since the host last looked (reset clears the count)
-  const int fresh = r.svd_not_converged - st->nc_seen;
-  st->nc_seen = r.svd_not_converged;
-  if (fresh > 0) {
-    set_error("mps_apply_gates: %d truncation SVDs reached the Jacobi sweep cap; their results were used as they stand",
-              fresh);
-    return MPS_ENOTCONV;
-  }
-  return MPS_OK;
+  const int fresh = r.not_converged - st->nc_seen;
+  st->nc_seen = r.not_converged;
+  rc = svd_status(r, "mps_apply_gates", fresh);
+  if (rc == MPS_ETIMEOUT) st->broken = true;
+  return rc;
 }
 
 mps_status mps_bond_dims(mps_state* st, int32_t* chi_out) {
@@ -1014,24 +1020,8 @@ mps_status mps_truncated_svd(mps_ctx* ctx, int32_t precision, int32_t m, int32_t
   MPSV_CUDA(cudaMemcpyAsync(&k, ctx->svdw->d_chi + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   MPSV_CUDA(cudaStreamSynchronize(ctx->stream));
   *k_out = k;
-  if (report) {
-    report->discarded_weight = r.discarded_weight;
-    report->min_kept_sv = r.min_kept_sv;
-    report->max_chi = r.max_chi;
-    report->degenerate_cuts = r.degenerate_cuts;
-    report->svd_not_converged = r.not_converged;
-    report->max_sweeps_used = r.max_sweeps;
-    report->two_qubit_gates = r.two_qubit_gates;
-    report->svd_flops = r.svd_flops;
-    report->svd_sweeps_fp32 = r.sweeps_fp32;
-    report->svd_sweeps_fp64 = r.sweeps_fp64;
-    for (int i = 0; i < 4; ++i) report->svd_phase_cycles[i] = r.phase_cycles[i];
-  }
-  if (r.not_converged) {
-    set_error("mps_truncated_svd: the Jacobi SVD reached its sweep cap; the result is used as it stands");
-    return MPS_ENOTCONV;
-  }
-  return MPS_OK;
+  if (report) copy_report(r, report);
+  return svd_status(r, "mps_truncated_svd", r.not_converged);
 }
 
 mps_status mps_apply_circuit_async(mps_state* st, const mps_circuit* c, const double* theta, int theta_on_device) {

@@ -1274,12 +1274,11 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   constexpr unsigned kCol = kLd * WA::kBytes;   // bytes of a 16-entry run
   const int tx = tid & 15, ty = tid >> 4, TY = T >> 4, nrow = (kPM - ty + TY - 1) / TY;  // 2 to 4 rows a thread
   S* red = reinterpret_cast<S*>(svd_smem + sred);
+  S* rowsq = reinterpret_cast<S*>(svd_smem + sa);  // of a tile's 64 rows, where C's tile was
   for (int j0 = me * kPN; j0 < k; j0 += P * kPN) {
-    // sum of (lam |W|)^2 over the rows of this thread: in double-float, for
-    // FP64 sweeps in FP64
-    constexpr bool kD = std::is_same<A, ArF64>::value;
-    GramAcc s2;
-    double d2 = 0.0;
+    // sums of (lam |W|)^2 down a column: rows part, part + 16, ... by one thread
+    // of the first 256, whatever the block size (a run's is another one)
+    S col2 = A::zero();
     for (int r0 = 0; r0 < m; r0 += kPM) {
       typename WA::Acc acc[4];
       for (int c0 = 0; c0 < n; c0 += kPK) {
@@ -1315,6 +1314,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int row = r0 + ty + i * TY;
+        S sq = A::zero();
         if (i < nrow && row < m && j0 + tx < k) {
           typename WA::S wr, wi;
           WA::dot_sum(acc[i], 1, wr, wi);
@@ -1326,32 +1326,30 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
             __stcg(Bq + (size_t)row * k + j0 + tx, refine ? cmk<R>(R(zr), R(zi)) : cmk<R>(R(zr * f), R(zi * f)));
           }
           if (refine) {
-            const double lam = __ldcg(lam_l + (row >> 1));
-            if constexpr (kD) {
-              const double ur = lam * WA::to_double(wr), ui = lam * WA::to_double(wi);
-              d2 = fma(ur, ur, fma(ui, ui, d2));
-            } else {
-              const ff w = ff_split(lam);
-              const ff ur = ff_mul(w, wr), ui = ff_mul(w, wi);
-              s2.add(ur, ur);
-              s2.add(ui, ui);
-            }
+            const S w = A::from_double(__ldcg(lam_l + (row >> 1)));
+            typename A::NAcc q2;
+            A::nrm(q2, A::cval(A::mul(w, wr), A::mul(w, wi)));
+            sq = A::nrm_value(q2);
           }
         }
+        if (refine && i < nrow && ty + i * TY < kPM) rowsq[(ty + i * TY) * 16 + tx] = sq;
+      }
+      if (refine) {
+        __syncthreads();
+        if (tid < 256)
+          for (int row = ty; row < kPM; row += 16) col2 = A::add(col2, rowsq[row * 16 + tx]);
+        __syncthreads();
       }
     }
     if (refine) {
-      S v0;
-      if constexpr (kD)
-        v0 = d2;
-      else
-        v0 = s2.value();
-      const S v1 = A::shfl_add(v0, 16);
-      if (lane < 16) red[(tid >> 5) * 16 + tx] = v1;
+      if (tid < 256) {
+        const S v1 = A::shfl_add(col2, 16);
+        if (lane < 16) red[(tid >> 5) * 16 + tx] = v1;
+      }
       __syncthreads();
       if (tid < 16 && j0 + tid < k) {
         S v = red[tid];
-        for (int w = 1; w < (T >> 5); ++w) v = A::add(v, red[w * 16 + tid]);
+        for (int w = 1; w < 8; ++w) v = A::add(v, red[w * 16 + tid]);
         double d = 0.0;
         memcpy(&d, &v, sizeof(S));
         __stcg(gnrm + j0 + tid, d);
@@ -1393,11 +1391,11 @@ template <class A> constexpr int kSvdThreads = std::is_same<A, ArF64>::value ? 2
 // Columns up to which one CTA takes the theta although more were launched.
 constexpr int kSvdSingleCols = 48;
 
-// CTAs that a theta of m x n gets out of the Pl launched; 0: it does not fit
-// (the grid kernel takes it).
+// CTAs that a theta of m x n gets, by its sizes alone; 0: more than the Pl
+// launched (a run's next tier or the grid kernel takes it).
 template <class A>
 __host__ __device__ inline int svd_team_size(int m, int n, int Pl) {
-  if ((n <= kSvdSingleCols || Pl == 1) && SvdSmem<A>::bytes(m, n, 1, true, true) <= kSvdSmemLimit) return 1;
+  if (n <= kSvdSingleCols && SvdSmem<A>::bytes(m, n, 1, true, true) <= kSvdSmemLimit) return 1;
   for (int P = 4; P <= Pl; P *= 2)
     if (SvdSmem<A>::bytes(m, n, P, true, true) <= kSvdSmemLimit) return P;
   return 0;

@@ -112,8 +112,9 @@ struct GridTeam {
   __device__ bool barrier() {
     __threadfence();
     __syncthreads();
-    bool gave_up = false;
+    __shared__ int s_gave_up;
     if (threadIdx.x == 0) {
+      int gave_up = 0;
       volatile unsigned* gen = &sync->gen;
       const unsigned g = *gen;
       if (atomicAdd(&sync->count, 1u) == (unsigned)P - 1) {
@@ -125,15 +126,17 @@ struct GridTeam {
         while (*gen == g) {
           if (clock64() - t0 > 4000000000ll || *(volatile unsigned*)&sync->abort) {
             atomicExch(&sync->abort, 1u);
-            gave_up = true;
+            gave_up = 1;
             break;
           }
           __nanosleep(20);
         }
       }
+      s_gave_up = gave_up;
       __threadfence();
     }
-    return !__syncthreads_or(gave_up);
+    __syncthreads();
+    return !s_gave_up;
   }
   __device__ void publish(int par, float v, int idx) {
     if (threadIdx.x == 0) __stcg(mail + par * P + me, make_float2(v, __int_as_float(idx)));

@@ -1,6 +1,7 @@
 // Hamiltonian upload (prefix and suffix tries of the Pauli strings) and the
 // Pauli-sum energy of Eq. expec2 with shared environments from both ends.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <limits>
@@ -692,6 +693,23 @@ namespace mpsv {
 
 // Shared body of vqe_eval_batch (host theta and energies, synchronising) and
 // vqe_eval_batch_async (device theta and energies).
+// Which of a batch's streams (given by their devices) are fed gate by gate.  Past
+// the 8 hardware queues that a process gets by default streams share a queue, and
+// one whose next launch waits for its last holds up the others behind it; up to
+// there the separate launches are the faster form (8 streams: 83.7 against 87.8
+// ms): more CTAs contract a theta, and the SVD keeps more registers.  16-qubit
+// UCCSD evaluations, gate by gate / as runs of gates (gate_run.cu), in ms:
+//   streams             9           12          16           24           32
+//   8 queues    153.8 / 88.3  165.6 / 89.2  150.2 / 91.2  187.5 / 95.9  227 / 103.3
+//   32 queues    88.0 / 88.5   90.7 / 89.4   94.7 / 91.5  106.2 / 96.3  121.3 / 103.7
+// Both forms give the same bits.
+std::vector<char> gate_by_gate_streams(const std::vector<int>& device) {
+  constexpr long kQueues = 8;
+  std::vector<char> by_gate;
+  for (int d : device) by_gate.push_back(std::count(device.begin(), device.end(), d) <= kQueues);
+  return by_gate;
+}
+
 static mps_status run_batch(const vqe_request* reqs, size_t n, double* energies_out, mps_status* status_out,
                             bool on_device) {
   if (n && (!reqs || !energies_out)) {
@@ -737,91 +755,35 @@ static mps_status run_batch(const vqe_request* reqs, size_t n, double* energies_
       groups[gi].push_back(i);
     }
   }
-  // Past the 8 hardware queues that a process gets by default, streams share a
-  // queue, and a stream whose next launch waits for its last one holds up the
-  // others behind it: 16 UCCSD evaluations of 16 qubits, gate by gate, took
-  // 181 ms against 97 ms for 8 (with 32 queues 110 ms).  From there on a
-  // circuit goes out as a run of gates, a few launches each, which this thread
-  // issues tier by tier over all requests, so that no request's later launches
-  // stand before another's first: 113 ms, and 136 against 282 ms for 32.  Up
-  // to 8 streams the separate launches are the faster form (79 against 85 ms
-  // for one): more CTAs contract a theta, and the SVD keeps more registers.
-  constexpr size_t kQueues = 8;
-  std::vector<char> whole(n, 0);
-  if (groups.size() > kQueues) {
-    std::vector<std::vector<size_t>> rest(groups.size());
-    for (size_t gi = 0; gi < groups.size(); ++gi)
-      for (size_t i : groups[gi]) {
-        const vqe_request& r = reqs[i];
-        whole[i] = state_runs(r.state, r.circuit->q.data(), r.circuit->arity.data(), r.circuit->n_gates);
-        if (!whole[i]) {
-          rest[gi].push_back(i);
-          continue;
-        }
-        DeviceGuard guard(r.state->ctx->device);
-        rc[i] = state_reset(r.state, r.init_bits);
-        if (rc[i] == MPS_OK) rc[i] = state_bind_circuit(r.state, r.circuit, r.theta, on_device ? 1 : 0);
-      }
-    for (int tier = 0; tier < kRunTiers; ++tier)
-      for (size_t gi = 0; gi < groups.size(); ++gi)
-        for (size_t i : groups[gi]) {
-          if (!whole[i] || rc[i] != MPS_OK) continue;
-          const vqe_request& r = reqs[i];
-          DeviceGuard guard(r.state->ctx->device);
-          rc[i] = state_run_tier(r.state, r.state->d_bound, r.circuit->q.data(), r.circuit->arity.data(),
-                                 r.circuit->n_gates, tier);
-          if (rc[i] != MPS_OK) r.state->broken = true;
-        }
-    std::vector<std::vector<size_t>> left;
-    for (auto& g : rest)
-      if (!g.empty()) left.push_back(std::move(g));
-    groups = std::move(left);
+  // Streams that are not fed gate by gate get whole circuits as runs of gates, a
+  // few launches each.
+  std::vector<int> device;
+  for (const auto& g : groups) device.push_back(reqs[g[0]].state->ctx->device);
+  const std::vector<char> by_gate = gate_by_gate_streams(device);
+  std::vector<size_t> runs;
+  {
+    std::vector<std::vector<size_t>> rest;
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+      bool whole = !by_gate[gi];
+      for (size_t i : groups[gi])
+        whole = whole && state_runs(reqs[i].state, reqs[i].circuit->q.data(), reqs[i].circuit->arity.data(),
+                                    reqs[i].circuit->n_gates);
+      if (whole)
+        runs.insert(runs.end(), groups[gi].begin(), groups[gi].end());
+      else
+        rest.push_back(std::move(groups[gi]));
+    }
+    groups = std::move(rest);
   }
-  const size_t hw = std::max(1u, std::thread::hardware_concurrency());
-  const size_t n_threads = std::min<size_t>({groups.size(), std::max<size_t>(1, hw / 2), 16});
-  std::vector<std::string> errs(n_threads);
-  auto work = [&](size_t t) {
-    std::vector<size_t> mine;
-    for (size_t gi = t; gi < groups.size(); gi += n_threads)
-      for (size_t i : groups[gi]) mine.push_back(i);
-    for (size_t i : mine) {
-      const vqe_request& r = reqs[i];
-      DeviceGuard guard(r.state->ctx->device);
-      rc[i] = state_reset(r.state, r.init_bits);
-      if (rc[i] == MPS_OK) rc[i] = state_bind_circuit(r.state, r.circuit, r.theta, on_device ? 1 : 0);
-    }
-    int max_gates = 0;
-    for (size_t i : mine)
-      if (rc[i] == MPS_OK && !whole[i]) max_gates = std::max(max_gates, reqs[i].circuit->n_gates);
-    for (int g = 0; g < max_gates; ++g) {
-      for (size_t i : mine) {
-        const vqe_request& r = reqs[i];
-        if (rc[i] != MPS_OK || whole[i] || g >= r.circuit->n_gates) continue;
-        DeviceGuard guard(r.state->ctx->device);
-        rc[i] = state_apply_device_gates(r.state, r.state->d_bound + g, &r.circuit->q[g], &r.circuit->arity[g], 1);
-        if (rc[i] != MPS_OK) r.state->broken = true;
-      }
-    }
-    for (size_t i : mine)
-      if (rc[i] != MPS_OK && errs[t].empty()) errs[t] = last_error();
+  auto begin = [&](size_t i) {
+    const vqe_request& r = reqs[i];
+    DeviceGuard guard(r.state->ctx->device);
+    rc[i] = state_reset(r.state, r.init_bits);
+    if (rc[i] == MPS_OK) rc[i] = state_bind_circuit(r.state, r.circuit, r.theta, on_device ? 1 : 0);
   };
-  if (n_threads <= 1) {
-    if (!groups.empty()) work(0);
-  } else {
-    std::vector<std::thread> pool;
-    for (size_t t = 1; t < n_threads; ++t) pool.emplace_back(work, t);
-    work(0);
-    for (auto& th : pool) th.join();
-    for (auto& e : errs)
-      if (!e.empty()) {
-        set_error("%s", e.c_str());
-        break;
-      }
-  }
-  // energies (each reads its bond dimensions once), then the results
+  // reads the bond dimensions once, which waits for the request's gates
   std::vector<StateFlags> flags(n);
-  for (size_t i = 0; i < n; ++i) {
-    if (rc[i] != MPS_OK) continue;
+  auto energy = [&](size_t i) {
     const vqe_request& r = reqs[i];
     DeviceGuard guard(r.state->ctx->device);
     rc[i] = ham_energy_async(r.state, const_cast<mps_ham*>(r.ham), on_device ? energies_out + i : nullptr);
@@ -831,7 +793,83 @@ static mps_status run_batch(const vqe_request* reqs, size_t n, double* energies_
       if (e == cudaSuccess) e = queue_flags(r.state, &flags[i]);
       if (e != cudaSuccess) rc[i] = cuda_fail(e, "vqe_eval_batch");
     }
+  };
+  const size_t hw = std::max(1u, std::thread::hardware_concurrency());
+  const size_t n_threads = std::min<size_t>({groups.size(), std::max<size_t>(1, hw / 2), 16});
+  std::vector<std::string> errs(n_threads + 1);
+  auto work = [&](size_t t) {
+    std::vector<size_t> mine;
+    for (size_t gi = t; gi < groups.size(); gi += n_threads)
+      for (size_t i : groups[gi]) mine.push_back(i);
+    for (size_t i : mine) begin(i);
+    int max_gates = 0;
+    for (size_t i : mine)
+      if (rc[i] == MPS_OK) max_gates = std::max(max_gates, reqs[i].circuit->n_gates);
+    for (int g = 0; g < max_gates; ++g) {
+      for (size_t i : mine) {
+        const vqe_request& r = reqs[i];
+        if (rc[i] != MPS_OK || g >= r.circuit->n_gates) continue;
+        DeviceGuard guard(r.state->ctx->device);
+        rc[i] = state_apply_device_gates(r.state, r.state->d_bound + g, &r.circuit->q[g], &r.circuit->arity[g], 1);
+        if (rc[i] != MPS_OK) r.state->broken = true;
+      }
+    }
+    for (size_t i : mine)
+      if (rc[i] != MPS_OK && errs[t].empty()) errs[t] = last_error();
+  };
+  // Runs: a stream's next launch, and after the last its energy, goes out when
+  // the one before is done.  One that waits in a hardware queue holds up the
+  // streams that share it, and the circuits leave a tier at different times.
+  auto feed = [&] {
+    std::vector<int> tier(n, 0);
+    for (size_t i : runs) begin(i);
+    std::vector<size_t> open = runs;
+    while (!open.empty()) {
+      bool launched = false;
+      size_t kept = 0;
+      for (size_t i : open) {
+        const vqe_request& r = reqs[i];
+        DeviceGuard guard(r.state->ctx->device);
+        if (rc[i] == MPS_OK) {
+          const cudaError_t e = tier[i] ? cudaStreamQuery(r.state->ctx->stream) : cudaSuccess;
+          if (e == cudaSuccess && tier[i] == kRunTiers) {
+            energy(i);
+            tier[i] += 1;
+            launched = true;
+          } else if (e == cudaSuccess) {
+            rc[i] = state_run_tier(r.state, r.state->d_bound, r.circuit->q.data(), r.circuit->arity.data(),
+                                   r.circuit->n_gates, tier[i]++);
+            if (rc[i] != MPS_OK) r.state->broken = true;
+            launched = true;
+          } else if (e != cudaErrorNotReady) {
+            rc[i] = cuda_fail(e, "vqe_eval_batch");
+            r.state->broken = true;
+          }
+        }
+        if (rc[i] != MPS_OK && errs[n_threads].empty()) errs[n_threads] = last_error();
+        if (rc[i] == MPS_OK && tier[i] <= kRunTiers) open[kept++] = i;
+      }
+      open.resize(kept);
+      if (!launched) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    }
+  };
+  if (groups.empty()) {
+    feed();
+  } else {
+    std::vector<std::thread> pool;
+    if (!runs.empty()) pool.emplace_back(feed);
+    for (size_t t = 1; t < n_threads; ++t) pool.emplace_back(work, t);
+    work(0);
+    for (auto& th : pool) th.join();
   }
+  for (auto& e : errs)
+    if (!e.empty()) {
+      set_error("%s", e.c_str());
+      break;
+    }
+  for (const auto& g : groups)
+    for (size_t i : g)
+      if (rc[i] == MPS_OK) energy(i);
   mps_status first_bad = MPS_OK;
   for (size_t i = 0; i < n; ++i) {
     if (rc[i] == MPS_OK && !on_device) {

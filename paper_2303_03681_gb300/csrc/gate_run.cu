@@ -7,15 +7,17 @@
 // Launched one by one, many evaluations at once are bound by the hardware
 // queues that their streams share and by the rate at which the host threads
 // can launch.  Here the bond dimensions and the report stay on the SM and a
-// whole circuit is at most three launches: 16 evaluations of a 16-qubit UCCSD
-// circuit take 113 ms instead of 181 (8 queues), 32 take 136 instead of 282.
-// What bounds a run is the chain of dependent steps inside its SVDs.
+// whole circuit is at most three launches: 32 evaluations of a 16-qubit UCCSD
+// circuit take 103 ms instead of 227 with the default 8 hardware queues, 104
+// instead of 121 with 32 (gate_by_gate_streams in energy.cu has the rule and the
+// other figures).  What bounds a run is the chain of dependent steps inside
+// its SVDs.
 //
 // Tiers.  A theta gets 1, 4 or 8 CTAs by its sizes alone (svd_team_size), so
-// its arithmetic does not depend on the launch.  The runs are issued as a
-// chain: a launch of one CTA goes on until a gate needs more, then one of 4
+// its arithmetic does not depend on the launch.  The runs are issued one
+// after another: a launch of one CTA goes on until a gate needs more, then one of 4
 // CTAs, then one of 8 where the capacities ask for it; each starts where the
-// one before it stopped (RunProgress) and returns at once when nothing is
+// one before it stopped (progress) and returns at once when nothing is
 // left.  A launch of one CTA holds one SM, so that many evaluations of
 // small fragments run side by side.
 #include <algorithm>

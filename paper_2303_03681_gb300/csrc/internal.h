@@ -270,6 +270,8 @@ void run_setup(mps_state* st);
 constexpr int kRunTiers = 3;
 bool run_tier(mps_state* st, const DevGate* d_gates, size_t n, int p_max, int tier);
 SvdParams svd_params(const mps_state* st);
+// How a batch's streams are fed (energy.cu).
+std::vector<char> gate_by_gate_streams(const std::vector<int>& device);
 
 // The two status flags of a state, read back with one 8-byte copy from
 // &DevReport::not_converged.

@@ -1,7 +1,7 @@
 """A request's result does not depend on how many others are in its batch (GPU).
 
-Up to eight streams ``vqe_eval_batch`` launches gate by gate, beyond that whole
-circuits as runs of gates.  The number of CTAs that a theta gets, the order of
+Up to eight streams ``vqe_eval_batch`` feeds gate by gate, beyond that it gives
+them whole circuits as runs of gates.  The number of CTAs that a theta gets, the order of
 its column pairs and the order of every sum follow from its sizes alone, so
 both forms give the same bits.  The cases take a circuit through the sizes on
 both sides of each change: one CTA up to 48 columns, clusters of 4 and of 8,

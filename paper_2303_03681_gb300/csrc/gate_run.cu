@@ -31,9 +31,9 @@ namespace mpsv {
 
 namespace {
 
-// 12 warps: 168 registers a thread, which the FP64 body (188 alone) just exceeds
-// and the double-float one does not.  One evaluation takes 84.8 ms, with 8 warps
-// 86.3 and with 16 (128 registers) 88.9.
+// 12 warps: 168 registers a thread, at which the one-CTA bodies spill 32 to 40
+// bytes a thread and the cluster's double-float one 350 (1,100 read).  One
+// evaluation takes 84.8 ms, with 8 warps 86.3 and with 16 (128 registers) 88.9.
 constexpr int kRunThreads = 384;
 
 struct RunArgs {
@@ -73,15 +73,14 @@ __device__ __forceinline__ void run_theta(const RunArgs& a, const DevGate* g, in
   const int chi_l = __ldcg(a.chi + q), chi_m = __ldcg(a.chi + q + 1), chi_r = __ldcg(a.chi + q + 2);
   __shared__ E s_u[16];
   load_gate<R>(g, threadIdx.x, s_u);
-  const int half = threadIdx.x >> 8, t = threadIdx.x & 255, halves = blockDim.x >> 8;
-  E* base = reinterpret_cast<E*>(svd_smem) + min(half, halves - 1) * 4 * kTile * (kTile + 1);
+  // 256 of the threads take the tiles; the others join the barriers only
+  const int t = threadIdx.x & 255;
+  E* base = reinterpret_cast<E*>(svd_smem);
   const int tr = (chi_r + kTile - 1) / kTile, tiles = tr * ((chi_l + kTile - 1) / kTile);
-  for (int t0 = me * halves; t0 < tiles; t0 += P * halves) {
-    const int tile = t0 + half;
+  for (int tile = me; tile < tiles; tile += P)
     theta_tile<R>(B + a.site_off[q], B + a.site_off[q + 1], s_u, chi_l, chi_m, chi_r, (tile / tr) * kTile,
-                  (tile % tr) * kTile, t & 15, t >> 4, half < halves && tile < tiles, reinterpret_cast<Tile>(base),
+                  (tile % tr) * kTile, t & 15, t >> 4, threadIdx.x < 256, reinterpret_cast<Tile>(base),
                   reinterpret_cast<Tile>(base + 2 * kTile * (kTile + 1)), static_cast<cplx<R>*>(a.C));
-  }
 }
 
 // Not inlined: each instance gets its own registers.
@@ -234,8 +233,7 @@ void run_prime() {
 }
 
 void run_setup(mps_state* st) {
-  // theta's tiles of two 256-thread halves
-  size_t smem = (size_t)2 * 4 * kTile * (kTile + 1) * sizeof(Cff);
+  size_t smem = (size_t)4 * kTile * (kTile + 1) * sizeof(Cff);  // theta's tiles
   st->run_p.assign(st->n, 0);
   for (int q = 0; q + 1 < st->n; ++q) {
     const int m = 2 * st->cap[q], n = 2 * st->cap[q + 2];

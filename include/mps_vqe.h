@@ -81,7 +81,9 @@ typedef enum {
 typedef struct {
   int32_t chi_max;        /* bond-dimension cap (>= 1) */
   int32_t precision;      /* mps_precision */
-  double trunc_rel;       /* keep s_i > trunc_rel * s_1 (0: keep all nonzero) */
+  double trunc_rel;       /* keep s_i > trunc_rel * s_1 (0: keep all nonzero).  Below the SVD's own
+                             accuracy (about 1e-13 in double-float, 1e-15 in FP64, times s_1) the
+                             s_i, and so what is kept, are rounding noise */
   int32_t svd_fp64;       /* 0: Jacobi SVD in FP32;
                              1: FP64-accurate SVD: pivoted Gram-Schmidt, then Jacobi sweeps on the
                                 triangular factor, in double-float on the FP32 units to a stopping

@@ -583,7 +583,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     // right-canonical on the rows that lam_q weighs with rounding noise): a
     // residual below the noise floor is scaled up to u ||A||_F, a perturbation
     // of A within its own rounding, and the factorisation goes on.
-    const bool keep_noise = p.trunc_rel < 8.0 * A::unit();
+    const bool keep_noise = p.trunc_rel == 0.0;
     const float floor2 = (float)(A::unit() * A::unit()) * fro2;
     for (int j = 0; j < rmax;) {
       float* nc = nrm + (j & 1) * n;

@@ -1,0 +1,43 @@
+"""Truncation thresholds at the rounding level (GPU).
+
+Diagonal thetas whose entries are powers of two: every step of the
+factorisation is exact on them, so the kept count has to be the rule's, s_i >
+trunc_rel s_1, even where the threshold lies below the arithmetic's noise
+floor (8 u: 1.1e-13 in double-float, 8.9e-16 in FP64).
+"""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _svd(A, trunc, mode):
+    import torch
+
+    from paper_2303_03681_gb300 import mps
+
+    n = A.shape[0]
+    ctx = mps.Context(0)
+    d = torch.from_numpy(np.ascontiguousarray(A, dtype=np.complex128)).cuda()
+    s = torch.full((n,), float("nan"), dtype=torch.float64, device="cuda")
+    vh = torch.zeros((n, n), dtype=torch.complex128, device="cuda")
+    k, rep, rc = mps.truncated_svd(ctx, "fp64", n, n, d.data_ptr(), n, trunc, mode, s.data_ptr(), vh.data_ptr())
+    assert rc == mps.MPS_OK
+    return k, s.cpu().numpy()[:k], vh.cpu().numpy()[:k], rep
+
+
+# mode, columns, small entries, threshold between them and the others
+@pytest.mark.parametrize("mode,n,small,trunc", [
+    (1, 32, 2.0 ** -53, 1e-14),   # double-float, one CTA
+    (1, 64, 2.0 ** -53, 1e-14),   # a cluster
+    (1, 340, 2.0 ** -52, 1e-14),  # a grid
+    (1, 16, 2.0 ** -54, 2e-16),   # FP64
+    (2, 64, 2.0 ** -54, 2e-16),
+])
+def test_directions_below_a_tiny_threshold_are_dropped(mode, n, small, trunc):
+    big = 2.0 ** -(np.arange(n // 2) % 4)
+    k, s, V, _ = _svd(np.diag(np.r_[big, np.full(n - n // 2, small)]), trunc, mode)
+    assert k == n // 2
+    assert np.array_equal(np.abs(V).sum(axis=0) > 0, np.arange(n) < n // 2)
+    assert np.max(np.abs(s - np.sort(big)[::-1])) <= 4 * np.sqrt(n) * 2.0 ** (-46 if mode == 1 and n >= 32 else -53)

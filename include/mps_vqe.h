@@ -239,7 +239,8 @@ mps_status mps_contract_theta(mps_ctx* ctx, int32_t precision, int32_t chi_l, in
  * 2 chi_r in the gate update) and in 2..4096.  The kept count k =
  * min(chi_max, #{s_i > trunc_rel s_1}) >= 1 goes to *k_out (host); s_out
  * (device, room for min(m, n) doubles) receives s_1 >= ... >= s_k, not
- * renormalised; Vh_out (device, room for min(chi_max, m, n) x n entries of the
+ * renormalised (complex128: one kept below 1e-18 of the kept norm, which needs trunc_rel
+ * = 0, as 1e-18 of it); Vh_out (device, room for min(chi_max, m, n) x n entries of the
  * input precision, row-major) the rows of V^H, i.e. the right singular
  * vectors conjugated.  svd_fp64 as in mps_config.  `report` (nullable)
  * receives the sweep counts and the discarded weight.  The context keeps a

@@ -1108,7 +1108,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
       if (!refine) s_d[1] = inv;
       if (me == 0) {
         rep->discarded_weight += share;
-        if (ratio < rep->min_kept_sv) rep->min_kept_sv = ratio;
+        if (!refine && ratio < rep->min_kept_sv) rep->min_kept_sv = ratio;
         if (k > rep->max_chi) rep->max_chi = k;
         // s_k and s_{k+1} equal to 1e-10 (their squares to 2e-10)
         if (k < r && k == p.chi_max && A::to_float(vnext) > 0.f &&
@@ -1166,31 +1166,41 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
   S* kn = reinterpret_cast<S*>(nrm);  // squared kept values, in units of 4^ec
   // ||s||, and lam = s / ||s|| in descending order (a running minimum: the
   // refined values of a degenerate pair can differ in their last bits either
-  // way), by warp 0.  Roots: double-float seeds, one FP64 Newton step each.
+  // way), by warp 0.  Below 1e-18 of ||C|| (double-float: the FP32 range of the
+  // roots' seeds) a value becomes a token, which keeps the direction alive for the
+  // next gate on its bond.  FP64 sweeps are finished in FP64; the double-float
+  // roots take one FP64 Newton step each.
+  constexpr bool kF64 = std::is_same<A, ArF64>::value;
   auto finish_lam = [&](auto value) {
     if (tid < 32) {
-      ff kept = ff_make(0.f, 0.f);
-      for (int a = lane; a < k; a += 32) kept = ff_add(kept, value(a));
+      S kept = A::zero();
+      for (int a = lane; a < k; a += 32) kept = A::add(kept, value(a));
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) kept = ff_add(kept, ff_shfl_xor(kept, o));
-      const ff one = ff_make(1.f, 0.f);
-      const bool any = kept.h > 1e-36f;
-      const double kd = any ? ff_join(kept) : 1.0;
-      double inv = ff_join(ff_rsqrt(any ? kept : one));
-      inv = inv * fma(-0.5 * kd * inv, inv, 1.5);
-      if (lane == 0) s_d[1] = inv;  // 1 / ||s|| in units of 2^-ec
+      for (int o = 16; o > 0; o >>= 1) kept = A::shfl_add(kept, o);
+      double inv;  // 1 / ||s|| in units of 2^-ec
+      if constexpr (kF64) {
+        inv = kept > 0.0 ? 1.0 / sqrt(kept) : 1.0;
+      } else {
+        const bool any = kept.h > 1e-36f;
+        const double kd = any ? ff_join(kept) : 1.0;
+        inv = ff_join(ff_rsqrt(any ? kept : ff_make(1.f, 0.f)));
+        inv = inv * fma(-0.5 * kd * inv, inv, 1.5);
+      }
+      if (lane == 0) s_d[1] = inv;
       if (me == 0) {
         double run = 1e300;
         for (int a0 = 0; a0 < k; a0 += 32) {
           double l = run;
           if (a0 + lane < k) {
-            const ff v = value(a0 + lane);
-            // below the FP32 range of the roots (1e-18 of ||C||): a token value,
-            // which keeps the direction alive for the next gate on its bond
-            const bool pos = v.h > 1e-36f;
-            const double vd = pos ? ff_join(v) : 0.0, y = ff_join(ff_rsqrt(pos ? v : one));
-            const double s0 = vd * y;
-            l = pos ? fma(0.5 * y, fma(-s0, s0, vd), s0) * inv : 1e-18;
+            const S v = value(a0 + lane);
+            if constexpr (kF64) {
+              l = v > 1e-36 ? sqrt(v) * inv : 1e-18;
+            } else {
+              const bool pos = v.h > 1e-36f;
+              const double vd = pos ? ff_join(v) : 0.0, y = ff_join(ff_rsqrt(pos ? v : ff_make(1.f, 0.f)));
+              const double s0 = vd * y;
+              l = pos ? fma(0.5 * y, fma(-s0, s0, vd), s0) * inv : 1e-18;
+            }
           }
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
@@ -1201,7 +1211,10 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
           run = __shfl_sync(0xffffffffu, l, 31);
           if (a0 + lane < k) lam_next[a0 + lane] = l;
         }
-        if (lane == 0) rep->inv_norm = inv * cscl;
+        if (lane == 0) {
+          if (run < rep->min_kept_sv) rep->min_kept_sv = run;
+          rep->inv_norm = inv * cscl;
+        }
       }
     }
     __syncthreads();
@@ -1246,12 +1259,7 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     }
     __syncthreads();
     if (refine)
-      finish_lam([&](int a) {
-        if constexpr (std::is_same<A, ArDF>::value)
-          return kn[a];
-        else
-          return ff_split(kn[a]);
-      });
+      finish_lam([&](int a) { return kn[a]; });
     if (Bq) {
       const S inv = A::from_double(refine ? s_d[1] : s_d[1] * w_unit);
       for (int t = tid; t < m * k; t += T) {
@@ -1364,13 +1372,9 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     if (!tm.barrier()) return 0;
     finish_lam([&](int a) {
       const double d = __ldcg(gnrm + a);
-      if constexpr (std::is_same<A, ArF64>::value) {
-        return ff_split(d);
-      } else {
-        ff v;
-        memcpy(&v, &d, sizeof(ff));
-        return v;
-      }
+      S v;
+      memcpy(&v, &d, sizeof(S));
+      return v;
     });
   }
   // ---- scale this CTA's columns of B~_q (only it wrote and reads them)

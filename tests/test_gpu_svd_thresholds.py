@@ -41,3 +41,22 @@ def test_directions_below_a_tiny_threshold_are_dropped(mode, n, small, trunc):
     assert k == n // 2
     assert np.array_equal(np.abs(V).sum(axis=0) > 0, np.arange(n) < n // 2)
     assert np.max(np.abs(s - np.sort(big)[::-1])) <= 4 * np.sqrt(n) * 2.0 ** (-46 if mode == 1 and n >= 32 else -53)
+
+
+def test_fp64_svd_normalises_in_fp64():
+    """svd_fp64 = 2: the kept singular values of every bond have norm one to FP64 rounding.
+
+    Each value's own roundings (root, quotient: 4 u) and those of the norm's sum
+    of k <= 64 squares over 32 lanes (7 u, halved by the root) give 2 (4 + 4) u,
+    and the check's sum another 7 u; 2^-53 = u.
+    """
+    from paper_2303_03681_gb300 import mps
+    from paper_2303_03681_gb300.inputs import MASTER_SEED, brickwork_circuit, make_rng
+
+    n = 12
+    ctx = mps.Context(0)
+    for seed in range(4):
+        st = mps.State(ctx, n, None, chi_max=64, precision="fp64", svd_fp64=2)
+        st.apply_gates(brickwork_circuit(n, 10, make_rng(MASTER_SEED + 1600 + seed)))
+        for lam in st.export()[1]:
+            assert abs(float(np.sum(lam * lam)) - 1.0) <= 24 * 2.0 ** -53

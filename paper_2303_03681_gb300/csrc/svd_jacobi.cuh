@@ -580,11 +580,11 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
     const float stop2 = fmaxf(kZeroNorm2, cut_rel * cut_rel * fro2);
     // Without a truncation threshold every nonzero direction is kept (the rows
     // of B~_{q+1} then span those of the unscaled C, which keeps B~_q
-    // right-canonical on the rows that lam_q weighs with rounding noise): a
-    // residual below the noise floor is scaled up to u ||A||_F, a perturbation
-    // of A within its own rounding, and the factorisation goes on.
+    // right-canonical on the rows that lam_q weighs with rounding noise): residuals
+    // that count as zero columns are scaled up to just above them, at most 4e-17
+    // of the largest entry, a perturbation of A below its rounding, and the
+    // factorisation goes on.
     const bool keep_noise = p.trunc_rel == 0.0;
-    const float floor2 = (float)(A::unit() * A::unit()) * fro2;
     for (int j = 0; j < rmax;) {
       float* nc = nrm + (j & 1) * n;
       float* nn = nrm + ((j & 1) ^ 1) * n;
@@ -614,8 +614,8 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         }
       }
       if (!(best > stop2)) {
-        if (!keep_noise || !(best > 0.f) || !(floor2 > stop2)) break;
-        const float up = pow2f(max(1, min(60, (exp_of(floor2) - exp_of(best)) / 2)));
+        if (!keep_noise || !(best > 0.f)) break;
+        const float up = pow2f(max(1, min(60, (exp_of(stop2) - exp_of(best)) / 2 + 1)));
         for (int t = tid; t < m * nloc; t += T) {
           const int i = t / m, rr = t - i * m;
           if (nc[i] < 0.f) continue;

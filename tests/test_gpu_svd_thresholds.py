@@ -43,6 +43,25 @@ def test_directions_below_a_tiny_threshold_are_dropped(mode, n, small, trunc):
     assert np.max(np.abs(s - np.sort(big)[::-1])) <= 4 * np.sqrt(n) * 2.0 ** (-46 if mode == 1 and n >= 32 else -53)
 
 
+@pytest.mark.parametrize("mode,n", [(1, 16), (2, 16), (2, 64), (1, 64), (1, 340)])
+def test_rounding_level_singular_values_without_a_threshold(mode, n):
+    """Directions that count as zero columns are kept, their values moved by at most 4e-17 of the largest entry.
+
+    (They are scaled up to just above 1e-17 of it, a quarter of FP64's unit
+    roundoff.)  All other values are their own, exact to the roots' rounding.
+    """
+    tiny = [2.0 ** -58, 2.0 ** -64, 2.0 ** -70]
+    d = np.r_[2.0 ** -(np.arange(n - 6) % 4), 2.0 ** -50, 2.0 ** -52, 2.0 ** -54, tiny]
+    k, s, V, rep = _svd(np.diag(d), 0.0, mode)
+    assert k == n
+    err = np.abs(s - np.sort(d)[::-1])
+    tol = 8 * 2.0 ** -46 if mode == 1 and n >= 32 else 16 * 2.0 ** -53
+    assert np.max(err[:-4] / s[:-4]) <= tol
+    assert np.max(err[-4:]) <= 4e-17
+    assert np.max(np.abs(V @ V.conj().T - np.eye(n))) <= tol
+    assert rep["min_kept_sv"] * np.linalg.norm(d) <= 4e-17
+
+
 def test_fp64_svd_normalises_in_fp64():
     """svd_fp64 = 2: the kept singular values of every bond have norm one to FP64 rounding.
 

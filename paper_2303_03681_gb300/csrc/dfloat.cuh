@@ -204,10 +204,6 @@ struct CAcc {
   __device__ __forceinline__ double2 value() const {  // sum of x y
     return make_double2(ff_join(sum(a, -1.f)), ff_join(sum(b, 1.f)));
   }
-  __device__ __forceinline__ Cff value_ff() const {
-    const ff r = sum(a, -1.f), i = sum(b, 1.f);
-    return Cff{mk2(r.h, i.h), mk2(r.l, i.l)};
-  }
   __device__ __forceinline__ double2 value_conj() const {  // sum of conj(x) y
     return make_double2(ff_join(sum(a, 1.f)), ff_join(sum(b, -1.f)));
   }

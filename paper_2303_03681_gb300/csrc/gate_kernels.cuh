@@ -41,7 +41,6 @@ template <> struct Mac<float> {
   static __device__ __forceinline__ void fmac(Acc& a, Elem x, Elem y) { cfmac(a.v, x, y); }  // += conj(x) y
   static __device__ __forceinline__ float2 value(const Acc& a) { return a.v; }       // of fma sums
   static __device__ __forceinline__ float2 value_conj(const Acc& a) { return a.v; }  // of fmac sums
-  static __device__ __forceinline__ Elem as_elem(const Acc& a) { return a.v; }
 };
 template <> struct Mac<double> {
   using Elem = Cff;
@@ -52,7 +51,6 @@ template <> struct Mac<double> {
   static __device__ __forceinline__ void fmac(Acc& a, Elem x, Elem y) { a.add(x, y); }
   static __device__ __forceinline__ double2 value(const Acc& a) { return a.value(); }
   static __device__ __forceinline__ double2 value_conj(const Acc& a) { return a.value_conj(); }
-  static __device__ __forceinline__ Elem as_elem(const Acc& a) { return a.value_ff(); }
 };
 
 // ---------------------------------------------------------------------------
@@ -96,18 +94,26 @@ __global__ void reset_kernel(cplx<R>* __restrict__ B, const size_t* __restrict__
 // The gate's entries for theta_tile, by the block's first 16 threads (one load
 // each that hides behind the first tile's; read where they are used they added
 // a load's latency to every gate).  The tile loop's barrier stands between.
+template <typename R> struct GateTile {
+  cplx<R> u[16];
+  bool real;  // every imaginary part is zero
+};
 template <typename R>
-__device__ __forceinline__ void load_gate(const DevGate* gate, int tid, typename Mac<R>::Elem* u) {
-  if (tid < 16) u[tid] = Mac<R>::load(ccast<cplx<R>>(__ldcg(gate->u + tid)));
+__device__ __forceinline__ void load_gate(const DevGate* gate, int tid, GateTile<R>& g) {
+  if (tid >= 32) return;
+  const double2 z = tid < 16 ? __ldcg(gate->u + tid) : make_double2(0.0, 0.0);
+  if (tid < 16) g.u[tid] = ccast<cplx<R>>(z);
+  const bool im = __any_sync(0xffffffffu, (__double_as_longlong(z.y) << 1) != 0);
+  if (tid == 0) g.real = !im;
 }
 
 // One 16 x 16 tile (a_l, a_r) with both physical indices, by 256 threads (tx,
-// ty).  u: the gate in shared memory.  sL, sR: the group's tiles, 2 x 16 x 17 entries each.  Every thread of
+// ty).  g: the gate in shared memory.  sL, sR: the group's tiles, 2 x 16 x 17 entries each.  Every thread of
 // the block calls it (act false: no tile, only the barriers).  The site tensors
 // are read past L1: a run of gates changes them between calls.
 template <typename R>
 __device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const cplx<R>* __restrict__ Br,
-                                           const typename Mac<R>::Elem* u, int chi_l, int chi_m, int chi_r, int al0,
+                                           const GateTile<R>& g, int chi_l, int chi_m, int chi_r, int al0,
                                            int ar0, int tx, int ty, bool act, typename Mac<R>::Elem (*sL)[kTile][kTile + 1],
                                            typename Mac<R>::Elem (*sR)[kTile][kTile + 1], cplx<R>* __restrict__ Cm) {
   using C = cplx<R>;
@@ -153,27 +159,38 @@ __device__ __forceinline__ void theta_tile(const cplx<R>* __restrict__ Bl, const
     __syncthreads();
   }
   if (!mine) return;
-  // the gate on (i', j'), in the tile's arithmetic (64 FP64 multiply-adds a
-  // thread took as long as a 16-column theta's sums)
+  // the gate on (i', j'), in the storage precision.  Complex128 takes FP64
+  // multiply-adds, two per clock and SM: the 64 of a thread are as long as a
+  // 16-column theta's sums, so a real gate (nine in ten of a UCCSD circuit) takes
+  // its 32 only (28-qubit UCCSD 54.2 -> 52.5 ms; in double-float, which would
+  // round theta to 2^-47 once more, 52.3)
   const int n = 2 * chi_r;
-  E th[2][2];
+  C th[2][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) th[i][j] = MT::as_elem(acc[i][j]);
+    for (int j = 0; j < 2; ++j) th[i][j] = MT::value(acc[i][j]);
+  auto apply = [&](auto term) {
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 2; ++i) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      typename MT::Acc out;
+      for (int j = 0; j < 2; ++j) {
+        C out = cmk<R>(0, 0);
 #pragma unroll
-      for (int ip = 0; ip < 2; ++ip)
+        for (int ip = 0; ip < 2; ++ip)
 #pragma unroll
-        for (int jp = 0; jp < 2; ++jp)
-          MT::fma(out, u[(2 * i + j) * 4 + 2 * ip + jp], th[ip][jp]);
-      Cm[(size_t)(2 * al + i) * n + j * chi_r + ar] = MT::value(out);
+          for (int jp = 0; jp < 2; ++jp) term(out, g.u[(2 * i + j) * 4 + 2 * ip + jp], th[ip][jp]);
+        Cm[(size_t)(2 * al + i) * n + j * chi_r + ar] = out;
+      }
     }
-  }
+  };
+  if (sizeof(R) == 8 && g.real)
+    apply([](C& out, C u, C t) {
+      out.x = fma(u.x, t.x, out.x);
+      out.y = fma(u.x, t.y, out.y);
+    });
+  else
+    apply([](C& out, C u, C t) { cfma(out, u, t); });
 }
 
 template <typename R>
@@ -189,9 +206,9 @@ __global__ void __launch_bounds__(kTile* kTile)
   const int chi_l = __ldcg(chi + q), chi_r = __ldcg(chi + q + 2);
   const int al0 = blockIdx.y * kTile, ar0 = blockIdx.x * kTile;
   if (al0 >= chi_l || ar0 >= chi_r) return;
-  __shared__ typename Mac<R>::Elem s_u[16];
-  load_gate<R>(gate, threadIdx.y * kTile + threadIdx.x, s_u);
-  theta_tile<R>(Bl, Br, s_u, chi_l, __ldcg(chi + q + 1), chi_r, al0, ar0, threadIdx.x, threadIdx.y, true, sL, sR, Cm);
+  __shared__ GateTile<R> s_g;
+  load_gate<R>(gate, threadIdx.y * kTile + threadIdx.x, s_g);
+  theta_tile<R>(Bl, Br, s_g, chi_l, __ldcg(chi + q + 1), chi_r, al0, ar0, threadIdx.x, threadIdx.y, true, sL, sR, Cm);
 }
 
 // ---------------------------------------------------------------------------

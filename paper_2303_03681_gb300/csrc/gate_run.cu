@@ -71,14 +71,14 @@ __device__ __forceinline__ void run_theta(const RunArgs& a, const DevGate* g, in
   using Tile = E(*)[kTile][kTile + 1];
   const cplx<R>* B = static_cast<const cplx<R>*>(a.B);
   const int chi_l = __ldcg(a.chi + q), chi_m = __ldcg(a.chi + q + 1), chi_r = __ldcg(a.chi + q + 2);
-  __shared__ E s_u[16];
-  load_gate<R>(g, threadIdx.x, s_u);
+  __shared__ GateTile<R> s_g;
+  load_gate<R>(g, threadIdx.x, s_g);
   // 256 of the threads take the tiles; the others join the barriers only
   const int t = threadIdx.x & 255;
   E* base = reinterpret_cast<E*>(svd_smem);
   const int tr = (chi_r + kTile - 1) / kTile, tiles = tr * ((chi_l + kTile - 1) / kTile);
   for (int tile = me; tile < tiles; tile += P)
-    theta_tile<R>(B + a.site_off[q], B + a.site_off[q + 1], s_u, chi_l, chi_m, chi_r, (tile / tr) * kTile,
+    theta_tile<R>(B + a.site_off[q], B + a.site_off[q + 1], s_g, chi_l, chi_m, chi_r, (tile / tr) * kTile,
                   (tile % tr) * kTile, t & 15, t >> 4, threadIdx.x < 256, reinterpret_cast<Tile>(base),
                   reinterpret_cast<Tile>(base + 2 * kTile * (kTile + 1)), static_cast<cplx<R>*>(a.C));
 }

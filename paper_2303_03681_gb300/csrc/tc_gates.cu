@@ -360,10 +360,10 @@ static __global__ void __launch_bounds__(kTile* kTile)
                       float2* __restrict__ Cm) {
   __shared__ float2 sL[2][kTile][kTile + 1];
   __shared__ float2 sR[2][kTile][kTile + 1];
-  __shared__ float2 s_u[16];
+  __shared__ GateTile<float> s_g;
   const int t = threadIdx.y * kTile + threadIdx.x;
-  if (t < 16) s_u[t] = ccast<float2>(a.u[t]);
-  theta_tile<float>(Bl, Br, s_u, a.chi[0], a.chi[1], a.chi[2], blockIdx.y * kTile, blockIdx.x * kTile, threadIdx.x,
+  if (t < 16) s_g.u[t] = ccast<float2>(a.u[t]);
+  theta_tile<float>(Bl, Br, s_g, a.chi[0], a.chi[1], a.chi[2], blockIdx.y * kTile, blockIdx.x * kTile, threadIdx.x,
                     threadIdx.y, true, sL, sR, Cm);
 }
 static __global__ void theta_setup_kernel(const ThetaArgs a, DevGate* __restrict__ g, int* __restrict__ chi) {

@@ -13,7 +13,7 @@
 // from the identity (the site tensors are right-canonical), and a string across
 // the middle is <P> = sum_{bd} L[b, d] R[b, d].  The number of distinct
 // prefixes of a molecular Hamiltonian grows with the cube of the sites they
-// cover: meeting halfway takes 8.4 -> 3.6 ms for the 14,251 strings of 20 spin
+// cover: meeting halfway takes 8.4 -> 3.4 ms for the 14,251 strings of 20 spin
 // orbitals at chi = 64, and for the 571,876 of 50 it stores 176 thousand environments
 // instead of 1.14 million.  T* is T with the site tensor transposed: the
 // suffixes run on the same kernels over transposed copies, and what is written below for
@@ -205,21 +205,38 @@ __global__ void __launch_bounds__(kTile* kTile)
   put(gr.slot[2], cmk<R>(u.y - v.y, v.x - u.x));  // -i u + i v
 }
 
-// A real as a double-float value.
-template <typename R> __device__ __forceinline__ ff as_ff(R x) {
-  if constexpr (sizeof(R) == 8)
-    return ff_split(x);
-  else
-    return ff_make(x, 0.f);
-}
-__device__ __forceinline__ ff warp_sum_ff(ff s) {
-  for (int x = 16; x > 0; x >>= 1) s = ff_add(s, ff_shfl_xor(s, x));
-  return s;
-}
+// Sums of real products for string values: FP64 for complex128 states (splitting
+// their entries costs more than the FP64 multiply-adds: the 14,251 strings of 10
+// orbitals at chi = 64 take 3.40 ms, in double-float 3.56), and double-float for
+// complex64 ones, whose entries' products are exact in it.
+template <typename R> struct RealSum;
+template <> struct RealSum<double> {
+  using E = double;
+  double v = 0.0;
+  static __device__ __forceinline__ E elem(double x) { return x; }
+  static __device__ __forceinline__ E mul(E a, E b) { return a * b; }
+  __device__ __forceinline__ void add(E a, E b) { v = fma(a, b, v); }
+  __device__ __forceinline__ E over_warp() const { return warp_sum(v); }
+  static __device__ __forceinline__ double join(E a, E b, E c, E d) { return (a + b) + (c + d); }
+};
+template <> struct RealSum<float> {
+  using E = ff;
+  GramAcc v;
+  static __device__ __forceinline__ E elem(float x) { return ff_make(x, 0.f); }
+  static __device__ __forceinline__ E elem(double x) { return ff_split(x); }
+  static __device__ __forceinline__ E mul(E a, E b) { return ff_mul(a, b); }
+  __device__ __forceinline__ void add(E a, E b) { v.add(a, b); }
+  __device__ __forceinline__ E over_warp() const {
+    ff s = v.value();
+    for (int x = 16; x > 0; x >>= 1) s = ff_add(s, ff_shfl_xor(s, x));
+    return s;
+  }
+  static __device__ __forceinline__ double join(E a, E b, E c, E d) { return ff_join(ff_add(ff_add(a, b), ff_add(c, d))); }
+};
 
-// One block of four warps per leaf: Re sum_i ph_i sum_{a,b} conj(B[a][i][b]) M^{pi(i)}[a][b],
-// in double-float sums.  One warp per leaf with FP64 sums was a chain of 128
-// iterations at chi = 64: 0.8 of 8.4 ms for the strings of 10 orbitals.
+// One block of four warps per leaf: Re sum_i ph_i sum_{a,b} conj(B[a][i][b]) M^{pi(i)}[a][b].
+// One warp per leaf was a chain of 128 iterations at chi = 64: 0.8 of 8.4 ms for
+// the strings of 10 orbitals.
 template <typename R>
 __global__ void __launch_bounds__(128)
     env_leaf_kernel(const cplx<R>* __restrict__ M, const cplx<R>* __restrict__ B, EnvLevel lv,
@@ -233,7 +250,8 @@ __global__ void __launch_bounds__(128)
   const C* Mp = M + (size_t)lf.x * 2 * lv.chi_l * lv.chi_r;
   const C* Mi0 = Mp + (size_t)pr.p0 * chi_r;  // row stride 2 chi_r
   const C* Mi1 = Mp + (size_t)pr.p1 * chi_r;
-  GramAcc acc;
+  using Sum = RealSum<R>;
+  Sum acc;
   const int tot = chi_l * chi_r;
 #pragma unroll 2
   for (int t = tid; t < tot; t += 128) {
@@ -241,25 +259,25 @@ __global__ void __launch_bounds__(128)
     const size_t at = (size_t)a * 2 * chi_r + b;
     const C x0 = B[at], x1 = B[at + chi_r];
     const C y0 = cmul(ph0, Mi0[at]), y1 = cmul(ph1, Mi1[at]);  // phases of 1, -1, i, -i: exact
-    ff f0 = as_ff(x0.x), f1 = as_ff(x0.y), f2 = as_ff(x1.x), f3 = as_ff(x1.y);
+    typename Sum::E f0 = Sum::elem(x0.x), f1 = Sum::elem(x0.y), f2 = Sum::elem(x1.x), f3 = Sum::elem(x1.y);
     if (lv.weight) {
-      ff w = as_ff(lv.weight[b]);
-      w = ff_mul(w, w);
-      f0 = ff_mul(w, f0);
-      f1 = ff_mul(w, f1);
-      f2 = ff_mul(w, f2);
-      f3 = ff_mul(w, f3);
+      typename Sum::E w = Sum::elem(lv.weight[b]);
+      w = Sum::mul(w, w);
+      f0 = Sum::mul(w, f0);
+      f1 = Sum::mul(w, f1);
+      f2 = Sum::mul(w, f2);
+      f3 = Sum::mul(w, f3);
     }
-    acc.add(f0, as_ff(y0.x));
-    acc.add(f1, as_ff(y0.y));
-    acc.add(f2, as_ff(y1.x));
-    acc.add(f3, as_ff(y1.y));
+    acc.add(f0, Sum::elem(y0.x));
+    acc.add(f1, Sum::elem(y0.y));
+    acc.add(f2, Sum::elem(y1.x));
+    acc.add(f3, Sum::elem(y1.y));
   }
-  __shared__ ff part[4];
-  const ff s = warp_sum_ff(acc.value());
+  __shared__ typename Sum::E part[4];
+  const typename Sum::E s = acc.over_warp();
   if ((tid & 31) == 0) part[tid >> 5] = s;
   __syncthreads();
-  if (tid == 0) vals[lf.z] = ff_join(ff_add(ff_add(part[0], part[1]), ff_add(part[2], part[3])));
+  if (tid == 0) vals[lf.z] = Sum::join(part[0], part[1], part[2], part[3]);
 }
 
 // One warp per string ending at a materialised node: Re Tr L.
@@ -299,8 +317,7 @@ __global__ void transpose_sites_kernel(const cplx<R>* __restrict__ B, const size
 // Hermitian, so it is the sum over d >= b of Re(L R), twice off the diagonal.
 // One block of four warps takes up to kCross strings of one prefix, so L is
 // read once for them and the loads of the R (L2 latency bounds it) are in flight together;
-// a group's missing strings repeat its last one.  The sums are double-float:
-// in FP64 they would be bound by the FP64 unit.  Row p of the triangle is joined
+// a group's missing strings repeat its last one.  Row p of the triangle is joined
 // to row chi - 1 - p, which gives chi + 1 entries.
 constexpr int kCross = 8;
 template <typename R>
@@ -312,7 +329,8 @@ __global__ void __launch_bounds__(128)
   const size_t size = (size_t)chi * chi;
   const cplx<R>* Lp = L + it.x * size;
   const cplx<R>* Rp[kCross];
-  GramAcc acc[kCross];
+  using Sum = RealSum<R>;
+  Sum acc[kCross];
 #pragma unroll
   for (int k = 0; k < kCross; ++k) Rp[k] = Rm + pair[it.y + min(k, it.z - 1)].x * size;
   const int total = chi * (chi + 1) / 2;
@@ -329,22 +347,22 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
     for (int k = 0; k < kCross; ++k) v[k] = Rp[k][at];
     const R f = b == d ? R(1) : R(2);
-    const ff zr = as_ff(f * z.x), zi = as_ff(-f * z.y);
+    const typename Sum::E zr = Sum::elem(f * z.x), zi = Sum::elem(-f * z.y);
 #pragma unroll
     for (int k = 0; k < kCross; ++k) {
-      acc[k].add(zr, as_ff(v[k].x));
-      acc[k].add(zi, as_ff(v[k].y));
+      acc[k].add(zr, Sum::elem(v[k].x));
+      acc[k].add(zi, Sum::elem(v[k].y));
     }
   }
-  __shared__ ff part[4][kCross];
+  __shared__ typename Sum::E part[4][kCross];
 #pragma unroll
   for (int k = 0; k < kCross; ++k) {
-    const ff s = warp_sum_ff(acc[k].value());
+    const typename Sum::E s = acc[k].over_warp();
     if (lane == k) part[tid >> 5][k] = s;
   }
   __syncthreads();
   if (tid < it.z)
-    vals[pair[it.y + tid].y] = ff_join(ff_add(ff_add(part[0][tid], part[1][tid]), ff_add(part[2][tid], part[3][tid])));
+    vals[pair[it.y + tid].y] = Sum::join(part[0][tid], part[1][tid], part[2][tid], part[3][tid]);
 }
 
 // E = constant + sum_k c_k vals[k] (terms with an empty support keep vals = 1).

@@ -128,7 +128,10 @@ typedef struct {
   int32_t svd_not_converged;/* SVDs that hit the sweep cap */
   int32_t max_sweeps_used;  /* largest number of Jacobi sweeps of one SVD */
   int64_t two_qubit_gates;  /* two-qubit gates applied */
-  double svd_flops;         /* real flops of the Jacobi sweeps run (dots + rotations) */
+  double svd_flops;         /* nominal real flops of the Jacobi sweeps run: every column pair of every
+                               sweep with its dot product and rotation (28 n for columns of n entries;
+                               svd_fp64 = 0: 28 m + 12 n), so an upper bound: pairs that a sweep leaves
+                               out or does not rotate are counted too */
   int64_t svd_sweeps_fp32;  /* Jacobi sweeps run in FP32, summed over SVDs */
   int64_t svd_sweeps_fp64;  /* Jacobi sweeps run in double-float or FP64, summed over SVDs */
   double svd_phase_cycles[4]; /* SM clock cycles of the SVDs (first CTA), summed: column load,

@@ -1118,8 +1118,9 @@ __device__ int svd_body(Team& tm, const cplx<R>* __restrict__ Cm, const double* 
         const int used = converged ? sweep : p.max_sweeps + 1;
         if (used > rep->max_sweeps) rep->max_sweeps = used;
         rep->two_qubit_gates += 1;
-        // per sweep and column pair: a dot product (8 n flops; 16 n with the
-        // two norms of Algorithm 1, counted as before) and a rotation (12 n)
+        // nominal: a dot product (8 n) and a rotation (20 n) for every column pair
+        // of every sweep, also where it was left out (counting the pairs that
+        // were met and rotated took 2 to 3 % of a theta's time)
         rep->svd_flops += (double)(sweep * (r * (r - 1) / 2)) * (double)(28 * n);
         rep->sweeps_fp64 += sweep;
         rep->phase_cycles[0] += double(t_load - t_start);

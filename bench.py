@@ -366,7 +366,7 @@ def run_gpu(args):
             dist.destroy_process_group()
         return
     value = job_throughput(args.steps * B, world, total_s)
-    launches_total = sum(v[0] for v in kprof.values())
+    launches_total = own_launches(kprof, prof)
     dom_launches, dom_timed, dom_ms = prof[dominant]  # of the warm-up steps
     roofline = None
     if dom_timed:
@@ -756,6 +756,16 @@ def oracle_check(mps, state, C, H, w, trunc_rel):
                 "discarded_weight_gpu": rep["discarded_weight"],
                 "discarded_weight_oracle": rec["oracle_discarded_weight"]}
     return None
+
+
+def own_launches(counts, profile):
+    """Kernel launches of the timed steps, from the class counts.
+
+    A class whose work another class's kernel does is counted but never timed
+    (B~_q inside the SVD kernel): those are not launches.
+    """
+    fused = {k for k, v in profile.items() if v[0] and not v[1]}
+    return sum(v[0] for k, v in counts.items() if k not in fused)
 
 
 def merge_profiles(profs):

@@ -60,7 +60,8 @@ typedef enum {
  * stores complex128; its CUDA-core contractions (theta, B~_q, environments)
  * and the FP64-accurate SVD compute in double-float arithmetic
  * (pairs of FP32 values, about 2^-46 relative per operation) on the FP32
- * units, since this part executes FP64 at 1/64 of the FP32 rate; results
+ * units, since this part executes FP64 at 1/64 of the FP32 rate; the gate's
+ * 4 x 4 product and the sums over a string's entries are FP64, and results
  * are stored as complex128.  The split-product modes keep
  * complex64 storage and run the theta contraction C = Q (B_q B_{q+1}) and
  * B~_q = C V^dagger (Eqs. tildeC, Bl) as tensor-core GEMMs (tcgen05, operands
@@ -265,8 +266,9 @@ mps_status mps_apply_circuit_async(mps_state* st, const mps_circuit* c, const do
 
 /* Upload a Hamiltonian sum_k coeffs[k] P_k: ops is n_terms x n_qubits bytes
  * (0=I 1=X 2=Y 3=Z), coeffs real.  The strings are arranged on the host in
- * a prefix trie (first non-identity site, then the operators left to right)
- * whose nodes are the shared left environments of Eq. expec2. */
+ * a trie of prefixes (first non-identity site, then the operators left to right)
+ * and one of suffixes from the right, up to the bond with the least work; their
+ * nodes are the shared environments of Eq. expec2. */
 mps_status mps_hamiltonian_create(mps_ctx* ctx, int32_t n_qubits, size_t n_terms,
                                   const uint8_t* ops, const double* coeffs, mps_ham** out);
 /* Trie statistics: n_nodes stored environments (prefixes from the left and
@@ -344,9 +346,13 @@ mps_status vqe_eval(mps_ctx* ctx, const vqe_request* reqs, size_t n, double* ene
  * threads issue the groups' gates, each going round-robin over its requests
  * (gate g of every request before gate g+1), so independent evaluations
  * overlap on the device; then the calling thread evaluates each energy.
- * Streams beyond the device's hardware work queues are serialised by the
- * driver: set CUDA_DEVICE_MAX_CONNECTIONS (up to 32) to at least the number
- * of contexts before the process creates its CUDA context.
+ * Streams beyond the device's hardware work queues (8; up to 32 with
+ * CUDA_DEVICE_MAX_CONNECTIONS, set before the process creates its CUDA
+ * context) are serialised by the driver, so with more than eight contexts on a
+ * device their circuits go out whole, in at most three launches each, from one
+ * host thread (where svd_fp64 is not 0, the contractions run on the CUDA cores
+ * and every theta fits a cluster).  A request's result does not depend, to the
+ * bit, on how many others are in its batch.
  * energies_out[i] / status_out[i] (host, status nullable) as in vqe_eval
  * (MPS_ENOTCONV included); the return value is the first status that is not
  * MPS_OK. */

@@ -11,7 +11,7 @@
 // of X J, and nothing accumulates V.  Drmac and Veselic (SIAM J. Matrix Anal.
 // Appl. 29, 2008, "New fast and accurate Jacobi SVD algorithm") give the
 // reason for the factorisation: the columns of X are graded and, scaled to
-// unit norm, well conditioned, so the sweeps converge in 4 to 8 instead of 15
+// unit norm, well conditioned, so the sweeps converge in 4 to 11 instead of 15
 // to 60, every column keeps its relative accuracy (normalising small columns
 // is safe, unlike columns of A itself), and the columns are n long instead of
 // the m + n of [A; V].  r is often about half of n: a theta B_q B_{q+1} has
@@ -31,8 +31,9 @@
 // on 8 CTAs, which it replaced): 124 x 124 over ten decades 19.5 -> 4.4 ms (36
 // -> 10 sweeps), 62 x 94 of rank 31 8.2 -> 0.89 ms, 512 x 512 1.20 s -> 47 ms
 // (8 CTAs -> a grid of 128), 16 x 16 in FP64 1.10 -> 0.57 ms.  It is bound by
-// the dependent pair steps and the barrier that ends each (at 124 x 124 the FP32
-// pipe is busy for 37 % of the time, barriers are most of the stalls).
+// the dependent pair steps, one block barrier each (at 124 x 124 the FP32 pipe is
+// busy for 37 % of the time; most stalls are at that barrier, where the 8 of 16
+// warps that have no pair wait; the cluster barrier comes 7 times a sweep).
 //
 // A pair of columns is one step of a group of 8 to 32 lanes: as few lanes as
 // give every warp a pair, because the angle and the reductions cost each

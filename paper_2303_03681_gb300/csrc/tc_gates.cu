@@ -219,7 +219,8 @@ template <int M> void set_attrs() {
 
 // The GEMM over a grid of (column tiles, row tiles), right after the split
 // kernel: its CTAs set up their barriers and tensor memory while that runs and
-// wait for it in the kernel (chi = 512 theta in TF32X3 30.2 -> 29.9 us; eight
+// wait for it in the kernel (chi = 512 theta in TF32X3, call after call with
+// the operands in L2, 30.2 -> 29.9 us; eight
 // 12-qubit evaluations 12.6 -> 12.2 ms).
 template <int M, class Epi>
 void launch_gemm(const TcWork& w, dim3 grid, const Epi& epi, int* err, cudaStream_t s) {
@@ -441,7 +442,7 @@ extern "C" mps_status mps_contract_theta(mps_ctx* ctx, int32_t precision, int32_
   }
   // The gate and the dimensions travel as kernel arguments: two copies from
   // pageable host memory before the kernel took a third of an ordinary call
-  // (45 x 61 x 37 in FP32: 12.2 -> 9.0 us, with the theta's tiles loaded ahead).
+  // (45 x 61 x 37 in FP32: 12.8 -> 10.3 us, with the theta's tiles loaded ahead).
   ThetaArgs args;
   for (int e = 0; e < 16; ++e) args.u[e] = make_double2(gate[2 * e], gate[2 * e + 1]);
   args.chi[0] = chi_l;
